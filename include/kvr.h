@@ -460,16 +460,18 @@ void kvr_entropy_destroy(kvr_entropy *det);
 
 /* Kernel of kvr_absorb_chunk's one-launch path (bf16, head_dim 128, G <= 8,
  * chunk <= 64, at most 192 rows after the chunk, 16-byte aligned q, k_new,
- * v_new and out; other calls run token by token).  Results agree within
- * rounding: 0 = 5th-generation tensor cores with the logits, probabilities
- * and outputs in tensor memory, for units of at most 144 rows after the
- * chunk (larger ones run kernel 1; the default), 1 = mma.sync with register
- * accumulators. */
+ * v_new and out; other calls run in blocks on the tensor cores where the
+ * outputs are bf16, else token by token).  Results agree within rounding:
+ * 0 = 5th-generation tensor cores with the logits, probabilities and outputs
+ * in tensor memory, for units of at most 144 rows after the chunk (larger
+ * ones run kernel 1; the default), 1 = mma.sync with register accumulators. */
 kvr_status kvr_cache_set_absorb_kernel(kvr_cache *cache, int kernel);
 
 /* How the cache's last kvr_absorb_chunk ran: 0 = the tensor-memory kernel,
- * 1 = the mma.sync kernel, 2 = token by token; -1 before the first call
- * (or for NULL).  Host state only: no synchronisation. */
+ * 1 = the mma.sync kernel, 2 = token by token, 3 = in blocks on the tensor
+ * cores (four launches; any chunk and unit length, bf16 in and out, head_dim
+ * 128, G <= 8, 16-byte aligned tensors); -1 before the first call (or for
+ * NULL).  Host state only: no synchronisation. */
 int kvr_cache_last_absorb_kernel(const kvr_cache *cache);
 
 /* ---- the same step for callers that cannot allocate -------------------- */

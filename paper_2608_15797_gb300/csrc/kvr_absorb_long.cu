@@ -1,0 +1,872 @@
+// kvr_absorb_long.cu -- absorbing a chunk of tokens into units of any length
+// (bf16 in and out, head_dim 128, G <= 8): what kvr_absorb_chunk runs beyond
+// the limits of the one-launch kernels of kvr_absorb.cu, a prompt's prefill
+// among it (Algorithm 1: one forward pass over an accepted step, or over the
+// prompt; Sec. 2.1: every token adds its head-mean probabilities to the
+// scores of the rows it attends; then one eviction).
+//
+// The work is a contraction: C tokens x G heads against m + C rows, causal.
+// Run token by token it was one launch a token, each reading every row again
+// (7B, two 1,000-token prompts: 140 ms; 16 sequences absorbing 57 tokens into
+// 640 rows: 39.8 ms).  Here it is four launches (1.34 ms and 0.99 ms):
+//   1. append: the chunk's rows go to slots m.. of each unit, score 0.
+//   2. attend (tcgen05): tiles of 128 query rows (128 / G whole tokens) over
+//      128-row key blocks with an online softmax; writes the outputs and each
+//      query row's log2 normaliser (into the cache's logit scratch).
+//   3. score (tcgen05): S^T = K Q^T, keys on the lanes, so a key's column sum
+//      over all queries is a sum inside one thread; the probabilities come
+//      exactly from the normalisers, and each key's sum is added once.
+//   4. finish: lengths, and the eviction where one is due (kvr_generic.cu).
+// Recomputing Q K^T in 3 costs one contraction of four, against column sums
+// over the lanes in 2 (124 shuffles a warp and block) and probabilities that
+// are only final after a row's last block.
+//
+// Precision: Q K^T accumulates in fp32; P is split into two bf16 terms (hi +
+// lo, 16 bits of mantissa) for PV, as in kvr_absorb.cu; outputs are bf16.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <math.h>
+#include <stdint.h>
+
+#include "kvr_internal.h"
+#include "kvr_ptx.cuh"
+
+namespace kvr {
+namespace {
+
+using namespace ptx;
+
+constexpr int kBlk = 128;            // keys a block; query rows a tile
+constexpr int kHalf = kBlk * 128;    // bytes of a 64-column half of a block
+constexpr int kTile = 2 * kHalf;     // bytes of a 128 x 128 bf16 block
+constexpr int kBox = 32;             // slab rows a TMA box
+// Two softmax warpgroups, and a third whose first two warps load and issue.
+// The softmax holds a block's 128 logits a thread: it takes registers from
+// the third (setmaxnreg: 2 x 200 + 104 = 3 x 168, the launch's allocation).
+constexpr int kThr = 384;
+constexpr int kTmemCols = 512;
+constexpr int kAttRing = 4;          // K and V blocks in flight (attend)
+constexpr int kQRing = 3;            // query tiles in flight (score)
+constexpr int kAttSmem = (2 + kAttRing) * kTile + 1024;
+constexpr int kScoreSmem = (4 + kQRing) * kTile + kQRing * 512 + 1024;
+// Lazy rescaling: the reference of a row's exponentials moves only when a
+// logit exceeds it by 2^kLazy; sums stay far inside fp32's range.
+constexpr float kLazy = 8.f;
+
+__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// 32 consecutive TMEM columns of this thread's lane (no wait).
+__device__ __forceinline__ void tmem_ld32(uint32_t ta, float (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"
+      "%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, "
+      "[%32];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+        "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]),
+        "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]),
+        "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]),
+        "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]),
+        "=f"(v[30]), "=f"(v[31])
+      : "r"(ta));
+}
+__device__ __forceinline__ void tmem_st32(uint32_t ta, const uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"
+      "%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,"
+      "%32};" ::"r"(ta),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
+      "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]),
+      "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]),
+      "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
+      "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"
+      "%12,%13,%14,%15,%16};" ::"r"(ta),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
+      "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]),
+      "r"(v[14]), "r"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() {
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem], issued by one thread.
+__device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t id,
+                                          bool acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "l"(b), "r"(id), "r"(acc ? 1 : 0)
+      : "memory");
+}
+
+// The unit of index x in [0, S * nl * H) and the first token row of its
+// (sequence, layer) in q, k_new, v_new and out.
+struct LUnit {
+  size_t ug, row0;
+  int h, m;  // m: rows before the chunk
+};
+__device__ __forceinline__ LUnit unit_at(const AbsorbParams &p, int x) {
+  const CacheView &c = p.c;
+  LUnit u;
+  u.h = x % c.H;
+  const int lr = (x / c.H) % p.nl, sq = x / (c.H * p.nl);
+  u.ug = ((size_t)sq * c.L + p.lb + lr) * c.H + u.h;
+  u.row0 = ((size_t)sq * p.nl + lr) * p.chunk;
+  u.m = c.state[4 * u.ug];
+  return u;
+}
+// Rows the unit could not hold: the host checked its mirror, so this says
+// that the device lengths are not what the host thinks; such units are left
+// alone by every kernel below.
+__device__ __forceinline__ bool unit_ok(const AbsorbParams &p, const LUnit &u) {
+  return u.m >= 0 && u.m + p.chunk <= p.c.cap && u.m + p.chunk <= p.max_rows;
+}
+
+// ---- 1. append ----------------------------------------------------------------
+
+constexpr int kAppendRows = 32;  // rows a CTA copies
+
+__global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) {
+  pdl_begin();
+  const CacheView &c = p.c;
+  const LUnit u = unit_at(p, blockIdx.x);
+  if (!unit_ok(p, u)) {
+    if (threadIdx.x == 0)
+      atomicOr(c.err, u.m >= 0 && u.m + p.chunk > c.cap ? ERR_CAPACITY : ERR_LENGTH);
+    return;
+  }
+  const int j0 = blockIdx.y * kAppendRows, nr = min(kAppendRows, p.chunk - j0);
+  const size_t dst = u.ug * (size_t)c.cap + u.m + j0;
+  const int4 *kn = reinterpret_cast<const int4 *>(p.k_new);
+  const int4 *vn = reinterpret_cast<const int4 *>(p.v_new);
+  int4 *K = reinterpret_cast<int4 *>(c.K) + dst * 16;
+  int4 *V = reinterpret_cast<int4 *>(c.V) + dst * 16;
+  for (int i = threadIdx.x; i < nr * 16; i += 256) {
+    const size_t src = ((u.row0 + j0 + (i >> 4)) * c.H + u.h) * 16 + (i & 15);
+    const int4 a = kn[src], b = vn[src];
+    K[i] = a;
+    V[i] = b;
+  }
+  if ((int)threadIdx.x < nr) {
+    const size_t s = u.ug * (size_t)c.sstride + u.m + j0 + threadIdx.x;
+    c.score[s] = 0.f;
+    c.pos[s] = c.state[4 * u.ug + 1] + j0 + (int)threadIdx.x;
+  }
+}
+
+// ---- 2. attend ----------------------------------------------------------------
+
+// One work item: two adjacent query tiles (2 x 128 / G tokens) of one unit.
+struct AttItem {
+  LUnit u;
+  int pair, Jt, chunk;
+  // Of tile t of the pair: its first token, its tokens (<= 0: no tile), the
+  // rows its last token sees, and its key blocks.
+  __device__ int tok0(int t) const { return (2 * pair + t) * Jt; }
+  __device__ int toks(int t) const { return min(Jt, chunk - tok0(t)); }
+  __device__ int lim(int t) const { return toks(t) > 0 ? u.m + tok0(t) + toks(t) : 0; }
+  __device__ int nb(int t) const { return (lim(t) + kBlk - 1) / kBlk; }
+  // Of the longer tile.
+  __device__ int lim_max() const { return max(lim(0), lim(1)); }
+  __device__ int nb_max() const { return max(nb(0), nb(1)); }
+};
+
+__device__ __forceinline__ bool att_item(const AbsorbParams &p, int i, int n_pairs, int Jt,
+                                         AttItem &it) {
+  const int x = i / n_pairs;
+  // Pairs rotate with the unit, so that every CTA of the persistent grid
+  // gets early (short) and late (long) tiles alike.
+  it.pair = (i % n_pairs + x) % n_pairs;
+  it.Jt = Jt;
+  it.chunk = p.chunk;
+  it.u = unit_at(p, x);
+  return unit_ok(p, it.u);
+}
+
+__global__ void __launch_bounds__(kThr, 1)
+    long_attend_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmK,
+                       const __grid_constant__ CUtensorMap tmV,
+                       const __grid_constant__ CUtensorMap tmQ, float *lse, int n_items,
+                       int n_pairs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
+  __shared__ __align__(8) uint64_t b_qfull[2], b_qfree[2], b_kvfull[kAttRing],
+      b_kvfree[kAttRing], b_s[2], b_p[2], b_o[2], b_drain;
+  unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+  const uint32_t aQ = smem_u32(smem), aR = aQ + 2 * kTile;
+  const CacheView &c = p.c;
+  const int G = c.G, Jt = kBlk / G;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  volatile int *abort = &s_abort;
+  // A whole warp's bounded wait; its lanes agree on the result.
+  auto wait_warp = [&](uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) != 0;
+  };
+  if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+  if (tid == 0) {
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(smem_u32(&b_qfull[t]), 1);
+      mbar_init(smem_u32(&b_qfree[t]), 1);
+      mbar_init(smem_u32(&b_s[t]), 1);
+      mbar_init(smem_u32(&b_p[t]), 4);
+      mbar_init(smem_u32(&b_o[t]), 1);
+    }
+    for (int s = 0; s < kAttRing; ++s) {
+      mbar_init(smem_u32(&b_kvfull[s]), 1);
+      mbar_init(smem_u32(&b_kvfree[s]), 1);
+    }
+    mbar_init(smem_u32(&b_drain), 1);
+    s_abort = 0;
+    fence_mbar_init();
+  }
+  // Query rows past the whole tokens of a tile are never loaded: zeros.
+  for (int i = tid; i < 2 * 2 * (kBlk - Jt * G) * 8; i += kThr) {
+    const int row = Jt * G + (i >> 3) % (kBlk - Jt * G), hf = (i >> 3) / (kBlk - Jt * G);
+    reinterpret_cast<int4 *>(smem + hf * kHalf + row * 128)[i & 7] = make_int4(0, 0, 0, 0);
+  }
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_begin();
+  const uint32_t tm = s_tmem;
+
+  if (warp >= 8) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+  if (warp == 8) {
+    // Producer: one thread issues every load, in the order they are used.
+    if (lane == 0) {
+      prefetch_tmap(&tmK);
+      prefetch_tmap(&tmV);
+      prefetch_tmap(&tmQ);
+      const uint32_t q_bytes = 256u * (uint32_t)(G * Jt);
+      int nq0 = 0, nq1 = 0, nkv = 0;  // loads issued
+      bool ok = true;
+      auto load_block = [&](const CUtensorMap *map, int row, int rows) {
+        const int s = nkv % kAttRing;
+        if (nkv >= kAttRing)
+          ok = mbar_wait(smem_u32(&b_kvfree[s]), (uint32_t)((nkv / kAttRing - 1) & 1), abort);
+        if (!ok) return;
+        const int nbox = (rows + kBox - 1) / kBox;
+        const uint32_t bar = smem_u32(&b_kvfull[s]), dst = aR + s * kTile;
+        mbar_expect_tx(bar, (uint32_t)nbox * 2 * kBox * 128);
+        for (int b = 0; b < nbox; ++b)
+          for (int hf = 0; hf < 2; ++hf)
+            tma_load_2d(dst + hf * kHalf + b * kBox * 128, map, 64 * hf, row + b * kBox, bar);
+        ++nkv;
+      };
+      for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+        AttItem it;
+        if (!att_item(p, i, n_pairs, Jt, it)) continue;
+        for (int t = 0; t < 2 && ok; ++t) {
+          if (!it.nb(t)) continue;
+          int &nq = t ? nq1 : nq0;
+          if (nq > 0) ok = mbar_wait(smem_u32(&b_qfree[t]), (uint32_t)((nq - 1) & 1), abort);
+          if (!ok) break;
+          mbar_expect_tx(smem_u32(&b_qfull[t]), q_bytes);
+          for (int hf = 0; hf < 2; ++hf)
+            tma_load_4d(aQ + t * kTile + hf * kHalf, &tmQ, 64 * hf, 0, it.u.h,
+                        (int)it.u.row0 + it.tok0(t), smem_u32(&b_qfull[t]));
+          ++nq;
+        }
+        const int row0 = (int)(it.u.ug * (size_t)c.cap);
+        for (int j = 0; j < it.nb_max() && ok; ++j) {
+          const int rows = min(kBlk, it.lim_max() - j * kBlk);
+          load_block(&tmK, row0 + j * kBlk, rows);
+          if (ok) load_block(&tmV, row0 + j * kBlk, rows);
+        }
+      }
+      if (!ok) {
+        if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+        *abort = 1;
+      }
+      // Whether or not another role gave up: every load issued lands
+      // (bounded) before the CTA's shared memory is given back.
+      volatile int never = 0;
+      if (nq0) mbar_wait(smem_u32(&b_qfull[0]), (uint32_t)((nq0 - 1) & 1), &never);
+      if (nq1) mbar_wait(smem_u32(&b_qfull[1]), (uint32_t)((nq1 - 1) & 1), &never);
+      for (int k = max(0, nkv - kAttRing); k < nkv; ++k)
+        mbar_wait(smem_u32(&b_kvfull[k % kAttRing]), (uint32_t)((k / kAttRing) & 1), &never);
+    }
+  } else if (warp == 9) {
+    // Issuer: S_t(j) = Q_t K_j^T, then O_t += P_t(j) V_j once the softmax
+    // has put P in place of S.  One thread issues, and its MMAs run in the
+    // order of issue, so S_t(j + 1) may follow PV_t(j), whose P it replaces;
+    // each tile's softmax runs under the other tile's contractions.
+    int kv = 0;
+    uint32_t ph_q = 0, ph_p = 0;  // phases to wait for, bit t
+    bool ok = true;
+    auto issue_s = [&](int t, int kst, int N) {
+      if (lane == 0) {
+        const uint32_t id = idesc_bf16(kBlk, N, false);
+        const uint64_t a0 = sdesc_sw128(aQ + t * kTile, 16, 1024);
+        const uint64_t b0 = sdesc_sw128(aR + kst * kTile, 16, 1024);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint64_t off = (uint64_t)(((k >> 2) * kHalf + (k & 3) * 32) >> 4);
+          tc_mma(tm + t * kBlk, a0 + off, b0 + off, id, k > 0);
+        }
+        tc_commit(smem_u32(&b_s[t]));
+      }
+    };
+    auto cols = [&](const AttItem &it, int t, int j) {
+      return min(kBlk, (it.lim(t) - j * kBlk + 15) & ~15);
+    };
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      AttItem it;
+      if (!att_item(p, i, n_pairs, Jt, it)) continue;
+      const int n = it.u.m + p.chunk;
+      int kst = kv % kAttRing;
+      ok = wait_warp(smem_u32(&b_kvfull[kst]), (uint32_t)((kv / kAttRing) & 1));
+      for (int t = 0; t < 2 && ok; ++t) {
+        if (!it.nb(t)) continue;
+        ok = wait_warp(smem_u32(&b_qfull[t]), (ph_q >> t) & 1);
+        if (!ok) break;
+        ph_q ^= 1u << t;
+        tc_fence_after();
+        issue_s(t, kst, cols(it, t, 0));
+        if (it.nb(t) == 1 && lane == 0) tc_commit(smem_u32(&b_qfree[t]));
+      }
+      if (!ok) break;
+      if (lane == 0) tc_commit(smem_u32(&b_kvfree[kst]));
+      ++kv;
+      for (int j = 0; j < it.nb_max() && ok; ++j) {
+        const int vst = kv % kAttRing;
+        ok = wait_warp(smem_u32(&b_kvfull[vst]), (uint32_t)((kv / kAttRing) & 1));
+        if (!ok) break;
+        ++kv;
+        // V rows past the unit's last one, up to the 16-row step of PV,
+        // meet P = 0 and must be finite: zeros.
+        const int v0 = n - j * kBlk, v1 = min(kBlk, (v0 + 15) & ~15);
+        if (it.lim_max() == n && v0 > 0 && v0 < v1) {
+          unsigned char *V = smem + 2 * kTile + vst * kTile;
+          for (int x = lane; x < (v1 - v0) * 16; x += 32)
+            reinterpret_cast<int4 *>(V + ((x >> 3) & 1) * kHalf + (v0 + (x >> 4)) * 128)[x & 7] =
+                make_int4(0, 0, 0, 0);
+          fence_proxy_async();
+          __syncwarp();
+        }
+        bool have_k = false;
+        kst = kv % kAttRing;
+        for (int t = 0; t < 2 && ok; ++t) {
+          if (j < it.nb(t)) {
+            ok = wait_warp(smem_u32(&b_p[t]), (ph_p >> t) & 1);
+            if (!ok) break;
+            ph_p ^= 1u << t;
+            tc_fence_after();
+            if (lane == 0) {
+              const uint32_t id = idesc_bf16(kBlk, kBlk, true);
+              const uint64_t b0 = sdesc_sw128(aR + vst * kTile, kHalf, 1024);
+              const int nk = cols(it, t, j) / 16;
+              for (int k = 0; k < nk; ++k) {
+                const uint32_t aP = tm + t * kBlk + 16 * k;
+                const uint64_t b = b0 + (uint64_t)(k * 128);
+                tc_mma_ts(tm + 2 * kBlk + t * kBlk, aP, b, id, j > 0 || k > 0);
+                tc_mma_ts(tm + 2 * kBlk + t * kBlk, aP + 8, b, id, true);
+              }
+              if (j + 1 == it.nb(t)) tc_commit(smem_u32(&b_o[t]));
+            }
+          }
+          if (j + 1 < it.nb(t)) {
+            if (!have_k) {
+              ok = wait_warp(smem_u32(&b_kvfull[kst]), (uint32_t)((kv / kAttRing) & 1));
+              if (!ok) break;
+              have_k = true;
+            }
+            tc_fence_after();
+            issue_s(t, kst, cols(it, t, j + 1));
+            if (j + 2 == it.nb(t) && lane == 0) tc_commit(smem_u32(&b_qfree[t]));
+          }
+        }
+        if (!ok) break;
+        if (lane == 0) {
+          tc_commit(smem_u32(&b_kvfree[vst]));
+          if (have_k) tc_commit(smem_u32(&b_kvfree[kst]));
+        }
+        if (have_k) ++kv;
+      }
+    }
+    if (lane == 0) {
+      if (!ok) {
+        if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+        *abort = 1;
+      }
+      // Every MMA issued has completed before TMEM is freed.
+      volatile int never = 0;
+      tc_commit(smem_u32(&b_drain));
+      mbar_wait(smem_u32(&b_drain), 0, &never);
+    }
+  } else if (warp < 8) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    // Softmax warpgroup t: thread r owns query row r of tile t.
+    const int t = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
+    const uint32_t lanes = (uint32_t)(wq * 32) << 16;
+    const uint32_t tS = tm + t * kBlk + lanes, tO = tm + 2 * kBlk + t * kBlk + lanes;
+    const float scale = p.scale_log2e;
+    const uint64_t scale2 = pk2(scale, scale);
+    int ns = 0, no = 0;
+    bool ok = true;
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      AttItem it;
+      if (!att_item(p, i, n_pairs, Jt, it) || !it.nb(t)) continue;
+      const int tk = r / G;
+      const bool valid = tk < it.toks(t) && r < Jt * G;
+      // Rows the query sees (rows past the tile's tokens follow the last).
+      const int seen = it.u.m + it.tok0(t) + min(tk, it.toks(t) - 1) + 1;
+      const int seen_w = it.u.m + it.tok0(t) + min(32 * wq / G, it.toks(t) - 1) + 1;
+      float ref = 0.f, l = 0.f;
+      for (int j = 0; j < it.nb(t); ++j) {
+        ok = wait_warp(smem_u32(&b_s[t]), (uint32_t)(ns++ & 1));
+        if (!ok) break;
+        tc_fence_after();
+        const int ncol = min(kBlk, it.lim(t) - j * kBlk);  // columns of S in use
+        float e[4][32];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (32 * k < ncol) tmem_ld32(tS + 32 * k, e[k]);
+        tmem_wait_ld();
+        const int lim = seen - j * kBlk;
+        float mx = -INFINITY;
+        if (seen_w - j * kBlk >= kBlk) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int x = 0; x < 32; x += 2) mx = fmaxf(mx, fmaxf(e[k][x], e[k][x + 1]));
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (32 * k < ncol) {
+#pragma unroll
+              for (int x = 0; x < 32; ++x) {
+                e[k][x] = 32 * k + x < lim ? e[k][x] : -INFINITY;
+                mx = fmaxf(mx, e[k][x]);
+              }
+            }
+          }
+        }
+        mx *= scale;
+        if (j == 0) {
+          ref = mx == -INFINITY ? 0.f : mx;
+        } else {
+          const bool up = mx > ref + kLazy;
+          if (__any_sync(0xffffffffu, up)) {
+            // O holds the blocks before this one (S of this block was
+            // committed after their PV).
+            const float f = up ? ex2(ref - mx) : 1.f;
+            if (up) ref = mx;
+            l *= f;
+#pragma unroll 1
+            for (int k = 0; k < kBlk; k += 16) {
+              uint32_t o[16];
+              tmem_ld16(tO + k, o);
+#pragma unroll
+              for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * f);
+              tmem_st16(tO + k, o);
+            }
+          }
+        }
+        const uint64_t nref2 = pk2(-ref, -ref);
+        uint64_t sum2 = pk2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (32 * k < ncol) {
+            uint32_t w[32];
+#pragma unroll
+            for (int x = 0; x < 32; x += 2) {
+              float d0, d1;
+              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, nref2), d0, d1);
+              d0 = ex2(d0);  // exp2(-inf) = 0 for masked keys
+              d1 = ex2(d1);
+              const uint64_t p2 = pk2(d0, d1);
+              sum2 = add2(sum2, p2);
+              const __nv_bfloat162 b = __floats2bfloat162_rn(d0, d1);
+              float r0, r1;  // p - bf16(p)
+              upk2(add2(p2, pk2(-__low2float(b), -__high2float(b))), r0, r1);
+              const int at = (x >> 4) * 16 + ((x & 15) >> 1);
+              w[at] = *reinterpret_cast<const uint32_t *>(&b);
+              w[at + 8] = pack_bf16(r0, r1);
+            }
+            tmem_st32(tS + 32 * k, w);  // 8 hi then 8 lo columns each 16 keys
+          }
+        }
+        float s0, s1;
+        upk2(sum2, s0, s1);
+        l += s0 + s1;
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&b_p[t]));
+      }
+      if (!ok) break;
+      ok = wait_warp(smem_u32(&b_o[t]), (uint32_t)(no++ & 1));
+      if (!ok) break;
+      tc_fence_after();
+      // The largest term is 2^(x - ref) with ref the rounded x: about 1.
+      if (valid && !(l >= 0.5f && l < INFINITY)) atomicOr(c.err, ERR_NONFINITE);
+      const float inv = 1.f / l;
+      const size_t qrow = ((it.u.row0 + it.tok0(t) + tk) * c.H + it.u.h) * G + (r - tk * G);
+      int4 *orow = reinterpret_cast<int4 *>(p.out) + qrow * 16;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float o[32];
+        tmem_ld32(tO + 32 * k, o);
+        tmem_wait_ld();
+        if (valid) {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float *v = o + 8 * x;
+            orow[4 * k + x] =
+                make_int4(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[2] * inv, v[3] * inv),
+                          pack_bf16(v[4] * inv, v[5] * inv), pack_bf16(v[6] * inv, v[7] * inv));
+          }
+        }
+      }
+      if (valid)
+        lse[it.u.ug * (size_t)G * c.cap + (size_t)it.tok0(t) * G + r] = ref + log2f(l);
+      tc_fence_before();
+    }
+    if (!ok && lane == 0) {
+      if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+      *abort = 1;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) tmem_dealloc(tm, kTmemCols);
+}
+
+// ---- 3. score -----------------------------------------------------------------
+
+// One work item: 256 rows (two key tiles) of one unit, against every query
+// tile that sees one of them.
+struct ScoreItem {
+  LUnit u;
+  int k0, n, Jt;  // first row; rows of the unit; tokens a query tile
+  // Of key tile t: the first query tile that sees one of its rows, and its
+  // rows (<= 0: none).
+  __device__ int q0(int t) const { return max(0, k0 + t * kBlk - u.m) / Jt; }
+  __device__ int nk(int t) const { return min(kBlk, n - k0 - t * kBlk); }
+};
+
+__device__ __forceinline__ bool score_item(const AbsorbParams &p, int i, int n_kp, int Jt,
+                                           ScoreItem &it) {
+  const int x = i / n_kp, kp = (i % n_kp + x) % n_kp;
+  it.u = unit_at(p, x);
+  if (!unit_ok(p, it.u)) return false;
+  it.n = it.u.m + p.chunk;
+  it.k0 = 2 * kBlk * kp;
+  it.Jt = Jt;
+  return it.k0 < it.n;
+}
+
+__global__ void __launch_bounds__(kThr, 1)
+    long_score_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmQ, const float *lse, int n_items,
+                      int n_kp, int n_qt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
+  __shared__ __align__(8) uint64_t b_kfull[2], b_kfree[2], b_qfull[kQRing], b_qfree[kQRing],
+      b_s[2][2], b_sfree[2][2], b_drain;
+  unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+  const uint32_t aK = smem_u32(smem), aQ = aK + 4 * kTile;
+  float *s_lse = reinterpret_cast<float *>(smem + (4 + kQRing) * kTile);  // [kQRing][128]
+  const CacheView &c = p.c;
+  const int G = c.G, Jt = kBlk / G;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  volatile int *abort = &s_abort;
+  // A whole warp's bounded wait; its lanes agree on the result.
+  auto wait_warp = [&](uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) != 0;
+  };
+  if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+  if (tid == 0) {
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(smem_u32(&b_kfull[t]), 1);
+      mbar_init(smem_u32(&b_kfree[t]), 1);
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(smem_u32(&b_s[t][b]), 1);
+        mbar_init(smem_u32(&b_sfree[t][b]), 4);
+      }
+    }
+    for (int s = 0; s < kQRing; ++s) {
+      mbar_init(smem_u32(&b_qfull[s]), 1 + 32);  // the TMA issue; the lanes' normalisers
+      mbar_init(smem_u32(&b_qfree[s]), 1 + 8);   // the contractions; the softmax warps
+    }
+    mbar_init(smem_u32(&b_drain), 1);
+    s_abort = 0;
+    fence_mbar_init();
+  }
+  for (int i = tid; i < kQRing * 2 * (kBlk - Jt * G) * 8; i += kThr) {
+    const int row = Jt * G + (i >> 3) % (kBlk - Jt * G), hf = (i >> 3) / (kBlk - Jt * G);
+    reinterpret_cast<int4 *>(smem + 4 * kTile + hf * kHalf + row * 128)[i & 7] =
+        make_int4(0, 0, 0, 0);
+  }
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_begin();
+  const uint32_t tm = s_tmem;
+
+  if (warp == 8) {
+    // Producer: key tiles (two pairs in flight), query tiles and their
+    // rows' normalisers.
+    if (lane == 0) {
+      prefetch_tmap(&tmK);
+      prefetch_tmap(&tmQ);
+    }
+    const uint32_t q_bytes = 256u * (uint32_t)(G * Jt);
+    int nk = 0, nq = 0;
+    bool ok = true;
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      ScoreItem it;
+      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      const int kb = nk & 1;
+      if (nk >= 2) ok = wait_warp(smem_u32(&b_kfree[kb]), (uint32_t)((nk / 2 - 1) & 1));
+      if (!ok) break;
+      if (lane == 0) {
+        const int rows = min(2 * kBlk, it.n - it.k0), nbox = (rows + kBox - 1) / kBox;
+        const uint32_t bar = smem_u32(&b_kfull[kb]);
+        const int row = (int)(it.u.ug * (size_t)c.cap) + it.k0;
+        mbar_expect_tx(bar, (uint32_t)nbox * 2 * kBox * 128);
+        for (int b = 0; b < nbox; ++b)
+          for (int hf = 0; hf < 2; ++hf)
+            tma_load_2d(aK + (kb * 2 + b / 4) * kTile + hf * kHalf + (b & 3) * kBox * 128, &tmK,
+                        64 * hf, row + b * kBox, bar);
+      }
+      ++nk;
+      const float *lu = lse + it.u.ug * (size_t)G * c.cap;
+      for (int q = it.q0(0); q < n_qt; ++q) {
+        const int s = nq % kQRing;
+        const int base = q * Jt * G, nv = min(Jt, p.chunk - q * Jt) * G;
+        float v[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int col = 32 * x + lane;
+          v[x] = col < nv ? lu[base + col] : INFINITY;
+        }
+        if (nq >= kQRing)
+          ok = wait_warp(smem_u32(&b_qfree[s]), (uint32_t)((nq / kQRing - 1) & 1));
+        if (!ok) break;
+        const uint32_t bar = smem_u32(&b_qfull[s]);
+        if (lane == 0) {
+          mbar_expect_tx(bar, q_bytes);
+          for (int hf = 0; hf < 2; ++hf)
+            tma_load_4d(aQ + s * kTile + hf * kHalf, &tmQ, 64 * hf, 0, it.u.h,
+                        (int)it.u.row0 + q * Jt, bar);
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) s_lse[s * kBlk + 32 * x + lane] = -v[x];
+        mbar_arrive(bar);
+        ++nq;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) {
+      if (!ok) {
+        if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+        *abort = 1;
+      }
+      volatile int never = 0;
+      for (int k = max(0, nk - 2); k < nk; ++k)
+        mbar_wait(smem_u32(&b_kfull[k & 1]), (uint32_t)((k / 2) & 1), &never);
+      for (int k = max(0, nq - kQRing); k < nq; ++k)
+        mbar_wait(smem_u32(&b_qfull[k % kQRing]), (uint32_t)((k / kQRing) & 1), &never);
+    }
+  } else if (warp == 9) {
+    int nk = 0, nq = 0, ns0 = 0, ns1 = 0;
+    bool ok = true;
+    const uint32_t id = idesc_bf16(kBlk, kBlk, false);
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      ScoreItem it;
+      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      const int kb = nk & 1;
+      ok = wait_warp(smem_u32(&b_kfull[kb]), (uint32_t)((nk / 2) & 1));
+      for (int q = it.q0(0); q < n_qt && ok; ++q) {
+        const int s = nq % kQRing;
+        ok = wait_warp(smem_u32(&b_qfull[s]), (uint32_t)((nq / kQRing) & 1));
+        for (int t = 0; t < 2 && ok; ++t) {
+          if (it.nk(t) <= 0 || q < it.q0(t)) continue;
+          int &ns = t ? ns1 : ns0;
+          const int b = ns & 1;
+          if (ns >= 2) ok = wait_warp(smem_u32(&b_sfree[t][b]), (uint32_t)((ns / 2 - 1) & 1));
+          if (!ok) break;
+          ++ns;
+          tc_fence_after();
+          if (lane == 0) {
+            const uint64_t a0 = sdesc_sw128(aK + (kb * 2 + t) * kTile, 16, 1024);
+            const uint64_t b0 = sdesc_sw128(aQ + s * kTile, 16, 1024);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const uint64_t off = (uint64_t)(((k >> 2) * kHalf + (k & 3) * 32) >> 4);
+              tc_mma(tm + (t * 2 + b) * kBlk, a0 + off, b0 + off, id, k > 0);
+            }
+            tc_commit(smem_u32(&b_s[t][b]));
+          }
+        }
+        if (!ok) break;
+        if (lane == 0) tc_commit(smem_u32(&b_qfree[s]));
+        ++nq;
+      }
+      if (!ok) break;
+      if (lane == 0) tc_commit(smem_u32(&b_kfree[kb]));
+      ++nk;
+    }
+    if (lane == 0) {
+      if (!ok) {
+        if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+        *abort = 1;
+      }
+      volatile int never = 0;
+      tc_commit(smem_u32(&b_drain));
+      mbar_wait(smem_u32(&b_drain), 0, &never);
+    }
+  } else if (warp < 8) {
+    // Warpgroup t: thread r owns key row r of tile t.
+    const int t = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
+    const uint32_t tS = tm + t * 2 * kBlk + ((uint32_t)(wq * 32) << 16);
+    const uint64_t scale2 = pk2(p.scale_log2e, p.scale_log2e);
+    int nq = 0, ns = 0;
+    bool ok = true;
+    for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
+      ScoreItem it;
+      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      const int slot = it.k0 + t * kBlk + r;
+      const int tmin = max(0, slot - it.u.m);  // first token that sees the row
+      const int tmin_w = max(0, it.k0 + t * kBlk + wq * 32 + 31 - it.u.m);
+      uint64_t a0 = pk2(0.f, 0.f), a1 = a0;
+      for (int q = it.q0(0); q < n_qt; ++q) {
+        const int s = nq % kQRing;
+        const uint32_t ph_q = (uint32_t)((nq / kQRing) & 1);
+        ++nq;
+        if (it.nk(t) <= 0 || q < it.q0(t)) {
+          // Nothing to read; the arrival counts for this filling of the slot.
+          ok = wait_warp(smem_u32(&b_qfull[s]), ph_q);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+          continue;
+        }
+        const int b = ns & 1;
+        ok = wait_warp(smem_u32(&b_s[t][b]), (uint32_t)((ns / 2) & 1)) &&
+             wait_warp(smem_u32(&b_qfull[s]), ph_q);
+        if (!ok) break;
+        ++ns;
+        tc_fence_after();
+        float e[4][32];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) tmem_ld32(tS + b * kBlk + 32 * k, e[k]);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&b_sfree[t][b]));
+        const ulonglong2 *nl = reinterpret_cast<const ulonglong2 *>(s_lse + s * kBlk);
+        const int toks = p.chunk - q * Jt;  // tokens from this tile on
+        if (q * Jt >= tmin_w && toks >= Jt) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int x = 0; x < 32; x += 4) {
+              const ulonglong2 z = nl[(32 * k + x) >> 2];
+              float d0, d1, d2, d3;
+              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d0, d1);
+              upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d2, d3);
+              a0 = add2(a0, pk2(ex2(d0), ex2(d1)));
+              a1 = add2(a1, pk2(ex2(d2), ex2(d3)));
+            }
+        } else {
+          // The diagonal tiles and the last one: columns of tokens before
+          // tmin do not see the row; columns past the chunk hold no query.
+          const int c_lo = (tmin - q * Jt) * G, c_hi = min(Jt, toks) * G;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int x = 0; x < 32; x += 4) {
+              const ulonglong2 z = nl[(32 * k + x) >> 2];
+              float d[4];
+              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d[0], d[1]);
+              upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d[2], d[3]);
+#pragma unroll
+              for (int y = 0; y < 4; ++y) {
+                const int col = 32 * k + x + y;
+                d[y] = col >= c_lo && col < c_hi ? ex2(d[y]) : 0.f;
+              }
+              a0 = add2(a0, pk2(d[0], d[1]));
+              a1 = add2(a1, pk2(d[2], d[3]));
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+      }
+      if (!ok) break;
+      if (slot < it.n) {
+        float x0, x1, y0, y1;
+        upk2(a0, x0, x1);
+        upk2(a1, y0, y1);
+        c.score[it.u.ug * (size_t)c.sstride + slot] += ((x0 + x1) + (y0 + y1)) * p.inv_g;
+      }
+    }
+    if (!ok && lane == 0) {
+      if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
+      *abort = 1;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) tmem_dealloc(tm, kTmemCols);
+}
+
+}  // namespace
+
+int absorb_long_box_rows() { return kBox; }
+
+cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
+                               const CUtensorMap &tmQ, const AbsorbParams &p, int sms,
+                               cudaStream_t st) {
+  if (p.chunk < 1 || p.c.G > 8 || p.c.d != 128 || !p.c.kv_bf16 || !p.c.out_bf16)
+    return cudaErrorInvalidValue;
+  const int units = p.c.S * p.nl * p.c.H;
+  const int Jt = kBlk / p.c.G, n_qt = (p.chunk + Jt - 1) / Jt, n_pairs = (n_qt + 1) / 2;
+  const int n_kp = (p.max_rows + 2 * kBlk - 1) / (2 * kBlk);
+  cudaError_t e = cudaFuncSetAttribute(
+      long_attend_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(long_score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kScoreSmem);
+  if (e != cudaSuccess) return e;
+  // The logit scratch holds [u][G][cap] floats; a unit's normalisers take
+  // chunk * G of its G * cap.
+  float *lse = p.c.logits;
+  e = launch_pdl(long_append_kernel,
+                 dim3(units, (p.chunk + kAppendRows - 1) / kAppendRows), dim3(256), 0, st, p);
+  if (e != cudaSuccess) return e;
+  const int n_att = units * n_pairs, n_sc = units * n_kp;
+  e = launch_pdl(long_attend_kernel, dim3(n_att < sms ? n_att : sms), dim3(kThr),
+                 (size_t)kAttSmem, st, p, tmK, tmV, tmQ, lse, n_att, n_pairs);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(long_score_kernel, dim3(n_sc < sms ? n_sc : sms), dim3(kThr),
+                    (size_t)kScoreSmem, st, p, tmK, tmQ, (const float *)lse, n_sc, n_kp, n_qt);
+}
+
+}  // namespace kvr

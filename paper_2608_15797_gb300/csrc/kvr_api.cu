@@ -248,12 +248,12 @@ kvr_status check_evict(int budget, int window) {
   return KVR_OK;
 }
 
-void mirror_append(kvr_cache *c, int lb, int le) {
+void mirror_append(kvr_cache *c, int lb, int le, int rows = 1) {
   for (int s = 0; s < c->desc.n_seq; ++s)
     for (int l = lb; l < le; ++l) {
       const size_t i = (size_t)s * c->desc.n_layers + l;
-      c->len[i] += 1;
-      c->next_pos[i] += 1;
+      c->len[i] += rows;
+      c->next_pos[i] += rows;
     }
 }
 
@@ -482,6 +482,48 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
   const int grid = std::min(c->sm_count, p.n_jobs);
   *err = kvr::launch_chunk_step(maps->first, maps->second, nullptr, nullptr, p,
                                 grid, stream);
+  return true;
+}
+
+// Absorb a chunk into units of any length on tensor cores if this call
+// qualifies.  P is split into two bf16 terms there, which the outputs'
+// rounding to bf16 covers; fp32 outputs keep the token-by-token path, whose
+// probabilities are fp32.
+bool try_absorb_long(kvr_cache *c, int lb, int le, int chunk, const void *q,
+                     const void *k_new, const void *v_new, void *out,
+                     int max_rows, int budget, int window, bool evict,
+                     cudaStream_t stream, cudaError_t *err) {
+  const CacheView &v = c->view;
+  if (!c->fused || !v.kv_bf16 || !v.out_bf16 || v.d != 128 || v.G > 8)
+    return false;
+  const size_t rows = (size_t)v.S * v.L * v.H * v.cap;
+  const size_t toks = (size_t)v.S * (le - lb) * chunk;
+  if (rows >= (size_t)INT32_MAX || toks >= (size_t)INT32_MAX) return false;
+  if (!aligned16(q) || !aligned16(k_new) || !aligned16(v_new) || !aligned16(out))
+    return false;
+  if (!device_facts(c)) return false;
+  const std::pair<CUtensorMap, CUtensorMap> *maps =
+      slab_maps(c, kvr::absorb_long_box_rows());
+  CUtensorMap tmq;
+  if (!maps || !encode_q4(&tmq, q, v.G, v.H, toks)) return false;
+  kvr::AbsorbParams p{};
+  p.c = v;
+  p.q = static_cast<const __nv_bfloat16 *>(q);
+  p.k_new = static_cast<const __nv_bfloat16 *>(k_new);
+  p.v_new = static_cast<const __nv_bfloat16 *>(v_new);
+  p.out = out;
+  p.lb = lb;
+  p.nl = le - lb;
+  p.chunk = chunk;
+  p.max_rows = max_rows;
+  p.scale_log2e = v.scale * 1.4426950408889634f;
+  p.inv_g = 1.f / (float)v.G;
+  *err = kvr::launch_absorb_long(maps->first, maps->second, tmq, p, c->sm_count,
+                                 stream);
+  if (*err == cudaSuccess)
+    *err = kvr::launch_evict_generic(v, lb, p.nl, max_rows,
+                                     evict ? budget : max_rows,
+                                     evict ? window : 0, stream, chunk);
   return true;
 }
 
@@ -893,7 +935,17 @@ kvr_status kvr_absorb_chunk(kvr_cache *c, int lb, int le, int chunk,
     if (e != cudaSuccess) return cuda_fail("kvr_absorb_chunk", e);
     c->last_absorb = ran;
     c->launches += 1;
-    for (int j = 0; j < chunk; ++j) mirror_append(c, lb, le);
+    mirror_append(c, lb, le, chunk);
+    if (evict) mirror_evict(c, lb, le, budget, window);
+    return KVR_OK;
+  }
+  cudaError_t e = cudaSuccess;
+  if (try_absorb_long(c, lb, le, chunk, q, k_new, v_new, out, m + chunk, budget,
+                      window, evict != 0, as_stream(stream), &e)) {
+    if (e != cudaSuccess) return cuda_fail("kvr_absorb_chunk", e);
+    c->last_absorb = 3;
+    c->launches += 4;
+    mirror_append(c, lb, le, chunk);
     if (evict) mirror_evict(c, lb, le, budget, window);
     return KVR_OK;
   }
@@ -904,7 +956,7 @@ kvr_status kvr_absorb_chunk(kvr_cache *c, int lb, int le, int chunk,
     StepArgs a = step_args(c, lb, le, q, k_new, v_new, out);
     a.chunk = chunk;
     a.tok = j;
-    cudaError_t e = kvr::launch_attend_score_generic(c->view, a, as_stream(stream));
+    e = kvr::launch_attend_score_generic(c->view, a, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail("kvr_absorb_chunk", e);
     c->launches += 1;
     mirror_append(c, lb, le);

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreads)
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
-    evict_kernel(CacheView c, int lb, int nl, int B, int W) {
+    evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow) {
   pdl_begin();
   __shared__ unsigned hist[256];
   __shared__ unsigned long long s_prefix;
@@ -204,7 +204,15 @@ __global__ void __launch_bounds__(kThreads)
 
   const Unit x = unit_of(c, lb, nl);
   const int tid = threadIdx.x;
-  const int n = c.state[4 * x.u];
+  // `grow` rows were appended whose length is not recorded yet.
+  const int n = c.state[4 * x.u] + grow;
+  const int newest = c.state[4 * x.u + 1] + grow - 1;
+  __syncthreads();
+  if (tid == 0 && grow) {
+    c.state[4 * x.u] = n;
+    c.state[4 * x.u + 1] = newest + 1;
+    c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
+  }
   if (n <= B + W) return;
   T *Ku = reinterpret_cast<T *>(c.K) + x.u * (size_t)c.cap * D;
   T *Vu = reinterpret_cast<T *>(c.V) + x.u * (size_t)c.cap * D;
@@ -212,7 +220,7 @@ __global__ void __launch_bounds__(kThreads)
   int32_t *pu = c.pos + x.u * (size_t)c.sstride;
   // The W most recent positions are protected; a row is a candidate iff its
   // position is at most newest - W.
-  const int wlo = c.state[4 * x.u + 1] - 1 - W;
+  const int wlo = newest - W;
 
   // TopB: by rank when every row has its own thread, else by a radix
   // select of the B-th largest candidate key.
@@ -344,7 +352,7 @@ cudaError_t attend_ext_dispatch(const CacheView &c, const StepArgs &a,
 
 template <typename T, int D>
 cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
-                           int B, int W, cudaStream_t st) {
+                           int B, int W, int grow, cudaStream_t st) {
   const int nk = B + W;
   const int max_list = max(1, min(nk, max_rows - nk));
   const size_t bytes = 2 * (size_t)max_list * sizeof(int);
@@ -353,7 +361,7 @@ cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(kThreads), bytes, st, c,
-                    lb, nl, B, W);
+                    lb, nl, B, W, grow);
 }
 
 }  // namespace
@@ -400,15 +408,17 @@ cudaError_t launch_attend_score_ext_scratch(const CacheView &c,
 
 cudaError_t launch_evict_generic(const CacheView &c, int lb, int nl,
                                  int max_rows, int budget, int window,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, int grow) {
   if (c.kv_bf16)
-    return c.d == 128 ? evict_dispatch<__nv_bfloat16, 128>(c, lb, nl, max_rows,
-                                                           budget, window, st)
-                      : evict_dispatch<__nv_bfloat16, 64>(c, lb, nl, max_rows,
-                                                          budget, window, st);
-  return c.d == 128
-             ? evict_dispatch<float, 128>(c, lb, nl, max_rows, budget, window, st)
-             : evict_dispatch<float, 64>(c, lb, nl, max_rows, budget, window, st);
+    return c.d == 128
+               ? evict_dispatch<__nv_bfloat16, 128>(c, lb, nl, max_rows, budget,
+                                                    window, grow, st)
+               : evict_dispatch<__nv_bfloat16, 64>(c, lb, nl, max_rows, budget,
+                                                   window, grow, st);
+  return c.d == 128 ? evict_dispatch<float, 128>(c, lb, nl, max_rows, budget,
+                                                 window, grow, st)
+                    : evict_dispatch<float, 64>(c, lb, nl, max_rows, budget,
+                                                window, grow, st);
 }
 
 cudaError_t launch_load(const CacheView &c, int seq, const void *k,

@@ -104,9 +104,11 @@ cudaError_t launch_attend_score_ext_scratch(const CacheView &c,
 cudaError_t launch_evict_rkv(const CacheView &c, int lb, int nl, int max_rows,
                              int budget, int window, float lam,
                              cudaStream_t st);
+// grow: rows appended to every unit whose lengths and next positions this
+// launch records before it evicts.
 cudaError_t launch_evict_generic(const CacheView &c, int lb, int nl,
                                  int max_rows, int budget, int window,
-                                 cudaStream_t st);
+                                 cudaStream_t st, int grow = 0);
 cudaError_t launch_load(const CacheView &c, int seq, const void *k,
                         const void *v, int n_rows, int first_pos,
                         cudaStream_t st);
@@ -299,6 +301,16 @@ int absorb_max_rows();
 // *ran (if given): the kernel launched, 0 tcgen05 or 1 mma.sync.
 cudaError_t launch_absorb(const AbsorbParams &p, int kernel, const CUtensorMap *tmQ,
                           cudaStream_t st, int *ran = nullptr);
+
+// Absorbing a chunk into units of any length (kvr_absorb_long.cu): bf16 in
+// and out, d = 128, G <= 8.  Three launches that append the rows, write the
+// outputs and add the scores; the lengths are left to the launch_evict_generic
+// (grow = chunk) that follows.  tmK, tmV: the slab with boxes of
+// absorb_long_box_rows() rows; tmQ as for launch_absorb.
+int absorb_long_box_rows();
+cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
+                               const CUtensorMap &tmQ, const AbsorbParams &p,
+                               int sms, cudaStream_t st);
 
 // Persistent chunked step (kvr_chunked.cu): bf16, d = 128, G <= 8, at most
 // chunk_max_rows() rows per job with the new row.  A job is one unit of the

@@ -443,7 +443,7 @@ class Cache:
 
     def last_absorb_kernel(self) -> int:
         """How the last absorb ran (kvr_cache_last_absorb_kernel): 0 tcgen05,
-        1 mma.sync, 2 token by token, -1 before the first."""
+        1 mma.sync, 2 token by token, 3 in blocks, -1 before the first."""
         return int(lib.kvr_cache_last_absorb_kernel(self.handle))
 
     def set_fused(self, enable: bool):

@@ -1,0 +1,77 @@
+"""kvr_absorb_chunk beyond the one-launch kernels' limits, bf16 outputs (the
+blocked tensor-core path), against the oracle: units and chunks at the edges
+of its 128-row key blocks, 256-row score items and query tiles of 128 // G
+whole tokens."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import parity
+from paper_2608_15797_gb300 import inputs
+from tests import harness
+from tests.test_gpu_absorb import absorb_lockstep
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    torch.cuda.set_device(0)
+
+
+# (G, rows before the chunk, chunk): one and several query tiles, an odd
+# number of tiles, a last tile of one token; units ending on, one before and
+# one past a block or an item; an empty unit beside a full one; a one-token
+# chunk; G = 1 (128 tokens a tile) and 8 (16).
+SHAPES = [(7, [192, 0], 1), (7, [250, 131], 18), (7, [0, 0], 127),
+          (7, [128, 1], 128), (7, [120, 0], 136), (7, [0, 255], 257),
+          (7, [640, 640], 57), (1, [3, 300], 129), (1, [0, 128], 256),
+          (8, [129, 257], 65), (8, [0, 240], 16), (3, [500, 11], 43),
+          (5, [0, 100], 300)]
+
+
+@pytest.mark.parametrize("G,old,chunk", SHAPES)
+def test_absorb_long_shapes(G, old, chunk):
+    w = inputs.Workload("al", 2, 2, G, 128, "bf16", 48, 8, 0, 0, sigma=1.0)
+    c, o = harness.make_pair(w, 90 + G, 2, cap=max(old) + chunk + 1,
+                             prompt_lens=old, out_dtype="bf16")
+    absorb_lockstep(c, o, w, 90 + G, chunk, w.budget, w.window)
+    assert c.last_absorb_kernel() == 3
+    harness.check_guards(c)
+    harness.lockstep(c, o, w, 90 + G, 2, w.budget, w.window, step0=100)
+
+
+def test_absorb_long_without_eviction_and_budget_edges():
+    """No eviction (every unit grows), then a chunk cut to a budget of one
+    row and no window; peaked logits (scores of 3-sigma keys) move the online
+    softmax's reference between blocks."""
+    w = inputs.Workload("al", 1, 2, 7, 128, "bf16", 1, 0, 0, 0, sigma=2.0,
+                        heavy_frac=0.05)
+    c, o = harness.make_pair(w, 97, 2, cap=600, prompt_lens=[260, 30],
+                             out_dtype="bf16")
+    absorb_lockstep(c, o, w, 97, 70, 0, 0, evict=False)
+    assert c.last_absorb_kernel() == 3
+    assert c.lengths().tolist() == [[330], [100]]
+    absorb_lockstep(c, o, w, 97, 200, 1, 0, step0=30_000)
+    assert c.lengths().tolist() == [[1], [1]]
+
+
+def test_absorb_long_layer_range():
+    """Layers [1, 3) of four: the other layers' units stay as they were."""
+    w = inputs.Workload("al", 4, 2, 7, 128, "bf16", 100, 8, 0, 0, sigma=1.0)
+    c, o = harness.make_pair(w, 98, 2, cap=400, prompt_lens=[200, 180],
+                             out_dtype="bf16")
+    toks = [inputs.step_inputs(w, 98, 40_000 + j, 2) for j in range(90)]
+    q, kn, vn = (np.stack([t[i] for t in toks], axis=2) for i in range(3))
+    out = c.absorb(*(harness.dev(a[:, 1:3], "bf16") for a in (q, kn, vn)),
+                   100, 8, layers=(1, 3))
+    assert c.last_absorb_kernel() == 3
+    ref = o.absorb(q, kn, vn, B=100, W=8, evict=True)
+    torch.cuda.synchronize()
+    parity.check_out(out.float().cpu().numpy(), ref[:, 1:3])
+    assert c.lengths().tolist() == [[200, 108, 108, 200], [180, 108, 108, 180]]
+    e = c.export(0, kv=False)
+    assert (e["score"][0, :, :200] == 0).all()
+    c.sync_status()
