@@ -8,7 +8,7 @@
 // The work is a contraction: C tokens x G heads against m + C rows, causal.
 // Run token by token it was one launch a token, each reading every row again
 // (7B, two 1,000-token prompts: 140 ms; 16 sequences absorbing 57 tokens into
-// 640 rows: 39.8 ms).  Here it is four launches (1.34 ms and 0.99 ms):
+// 640 rows: 39.8 ms).  Here it is four launches (0.95 ms and 0.81 ms):
 //   1. append: the chunk's rows go to slots m.. of each unit, score 0.
 //   2. attend (tcgen05): tiles of 128 query rows (128 / G whole tokens) over
 //      128-row key blocks with an online softmax; writes the outputs and each
@@ -40,18 +40,19 @@ constexpr int kBlk = 128;            // keys a block; query rows a tile
 constexpr int kHalf = kBlk * 128;    // bytes of a 64-column half of a block
 constexpr int kTile = 2 * kHalf;     // bytes of a 128 x 128 bf16 block
 constexpr int kBox = 32;             // slab rows a TMA box
-// Two softmax warpgroups, and a third whose first two warps load and issue.
-// The softmax holds a block's 128 logits a thread: it takes registers from
-// the third (setmaxnreg: 2 x 200 + 104 = 3 x 168, the launch's allocation).
-constexpr int kThr = 384;
-constexpr int kTmemCols = 512;
-constexpr int kAttRing = 4;          // K and V blocks in flight (attend)
-constexpr int kQRing = 3;            // query tiles in flight (score)
-constexpr int kAttSmem = (2 + kAttRing) * kTile + 1024;
+constexpr int kAttThr = 320, kAttCols = 256;  // attend: two CTAs an SM
+constexpr int kAttSmem = 3 * kTile + 1024;
+static_assert(kAttSmem + 2048 <= 113 * 1024, "two CTAs an SM, with the static variables");
+// Score: one CTA an SM; four softmax warpgroups, a loading and an issuing warp.
+constexpr int kScThr = 576, kScCols = 512;
+constexpr int kProducer = 16, kIssuer = 17;
+constexpr int kQRing = 3;            // query tiles in flight
 constexpr int kScoreSmem = (4 + kQRing) * kTile + kQRing * 512 + 1024;
+static_assert(kScoreSmem + 512 <= 227 * 1024, "with the static variables");
 // Lazy rescaling: the reference of a row's exponentials moves only when a
 // logit exceeds it by 2^kLazy; sums stay far inside fp32's range.
 constexpr float kLazy = 8.f;
+constexpr uint32_t kGaveUp = 0x7FBADBADu;  // a NaN that no arithmetic returns
 
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
   uint64_t r;
@@ -106,6 +107,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t (&v)[16]) 
       "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]),
       "r"(v[14]), "r"(v[15])
       : "memory");
+}
+// 32 bytes to global memory, one whole sector a thread (32-byte aligned).
+__device__ __forceinline__ void st_global32(void *dst, const uint32_t *v) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -177,72 +184,69 @@ __global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) 
 
 // ---- 2. attend ----------------------------------------------------------------
 
-// One work item: two adjacent query tiles (2 x 128 / G tokens) of one unit.
+// One work item: a query tile (128 / G whole tokens) of one unit.
 struct AttItem {
   LUnit u;
-  int pair, Jt, chunk;
-  // Of tile t of the pair: its first token, its tokens (<= 0: no tile), the
-  // rows its last token sees, and its key blocks.
-  __device__ int tok0(int t) const { return (2 * pair + t) * Jt; }
-  __device__ int toks(int t) const { return min(Jt, chunk - tok0(t)); }
-  __device__ int lim(int t) const { return toks(t) > 0 ? u.m + tok0(t) + toks(t) : 0; }
-  __device__ int nb(int t) const { return (lim(t) + kBlk - 1) / kBlk; }
-  // Of the longer tile.
-  __device__ int lim_max() const { return max(lim(0), lim(1)); }
-  __device__ int nb_max() const { return max(nb(0), nb(1)); }
+  int tok0, toks;  // first token; tokens
+  int lim, nb;     // rows the last token sees; key blocks
 };
 
-__device__ __forceinline__ bool att_item(const AbsorbParams &p, int i, int n_pairs, int Jt,
-                                         AttItem &it) {
-  const int x = i / n_pairs;
-  // Pairs rotate with the unit, so that every CTA of the persistent grid
-  // gets early (short) and late (long) tiles alike.
-  it.pair = (i % n_pairs + x) % n_pairs;
-  it.Jt = Jt;
-  it.chunk = p.chunk;
-  it.u = unit_at(p, x);
+__device__ __forceinline__ bool att_item(const AbsorbParams &p, int i, int units, int n_qt,
+                                         int Jt, AttItem &it) {
+  // The longest tiles (the last tokens) of every unit first.
+  const int tile = n_qt - 1 - i / units;
+  it.u = unit_at(p, i % units);
+  it.tok0 = tile * Jt;
+  it.toks = min(Jt, p.chunk - it.tok0);
+  it.lim = it.u.m + it.tok0 + it.toks;
+  it.nb = (it.lim + kBlk - 1) / kBlk;
   return unit_ok(p, it.u);
 }
 
-__global__ void __launch_bounds__(kThr, 1)
+// Two CTAs an SM, each with one tile: while one waits for its loads, its
+// softmax or its outputs, the other has the tensor cores.  7B, two 1,000-token
+// prompts: 0.58 ms, against 0.80 ms for one CTA with two tiles in step that
+// share the K and V blocks (a third of it passed between items) and 0.94 ms
+// for that with one softmax warp for 32 rows instead of two.  Eight softmax
+// warps, then a loading and an issuing warp.
+__global__ void __launch_bounds__(kAttThr, 2)
     long_attend_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmK,
                        const __grid_constant__ CUtensorMap tmV,
                        const __grid_constant__ CUtensorMap tmQ, float *lse, int n_items,
-                       int n_pairs) {
+                       int n_qt, int out32) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  __shared__ __align__(8) uint64_t b_qfull[2], b_qfree[2], b_kvfull[kAttRing],
-      b_kvfree[kAttRing], b_s[2], b_p[2], b_o[2], b_drain;
+  __shared__ float s_x[2][kBlk];  // what a row's two threads tell each other
+  __shared__ __align__(8) uint64_t b_qfull, b_qfree, b_kfull, b_kfree, b_vfull, b_vfree, b_s,
+      b_p, b_o, b_drain;
   unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  const uint32_t aQ = smem_u32(smem), aR = aQ + 2 * kTile;
+  const uint32_t aQ = smem_u32(smem), aK = aQ + kTile, aV = aK + kTile;
   const CacheView &c = p.c;
-  const int G = c.G, Jt = kBlk / G;
+  const int G = c.G, Jt = kBlk / G, units = n_items / n_qt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   volatile int *abort = &s_abort;
   // A whole warp's bounded wait; its lanes agree on the result.
-  auto wait_warp = [&](uint32_t bar, uint32_t parity) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) != 0;
+  auto wait_warp = [&](uint64_t &bar, int n) {
+    return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), (uint32_t)(n & 1), abort)) != 0;
   };
-  if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+  if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kAttCols);
   if (tid == 0) {
-    for (int t = 0; t < 2; ++t) {
-      mbar_init(smem_u32(&b_qfull[t]), 1);
-      mbar_init(smem_u32(&b_qfree[t]), 1);
-      mbar_init(smem_u32(&b_s[t]), 1);
-      mbar_init(smem_u32(&b_p[t]), 4);
-      mbar_init(smem_u32(&b_o[t]), 1);
-    }
-    for (int s = 0; s < kAttRing; ++s) {
-      mbar_init(smem_u32(&b_kvfull[s]), 1);
-      mbar_init(smem_u32(&b_kvfree[s]), 1);
-    }
+    mbar_init(smem_u32(&b_qfull), 1);
+    mbar_init(smem_u32(&b_qfree), 1);
+    mbar_init(smem_u32(&b_kfull), 1);
+    mbar_init(smem_u32(&b_kfree), 1);
+    mbar_init(smem_u32(&b_vfull), 1);
+    mbar_init(smem_u32(&b_vfree), 1);
+    mbar_init(smem_u32(&b_s), 1);
+    mbar_init(smem_u32(&b_p), 8);
+    mbar_init(smem_u32(&b_o), 1);
     mbar_init(smem_u32(&b_drain), 1);
     s_abort = 0;
     fence_mbar_init();
   }
   // Query rows past the whole tokens of a tile are never loaded: zeros.
-  for (int i = tid; i < 2 * 2 * (kBlk - Jt * G) * 8; i += kThr) {
+  for (int i = tid; i < 2 * (kBlk - Jt * G) * 8; i += kAttThr) {
     const int row = Jt * G + (i >> 3) % (kBlk - Jt * G), hf = (i >> 3) / (kBlk - Jt * G);
     reinterpret_cast<int4 *>(smem + hf * kHalf + row * 128)[i & 7] = make_int4(0, 0, 0, 0);
   }
@@ -251,9 +255,8 @@ __global__ void __launch_bounds__(kThr, 1)
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const uint32_t tm = s_tmem;
+  const uint32_t tm = s_tmem, tmO = tm + kBlk;
 
-  if (warp >= 8) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
   if (warp == 8) {
     // Producer: one thread issues every load, in the order they are used.
     if (lane == 0) {
@@ -261,40 +264,42 @@ __global__ void __launch_bounds__(kThr, 1)
       prefetch_tmap(&tmV);
       prefetch_tmap(&tmQ);
       const uint32_t q_bytes = 256u * (uint32_t)(G * Jt);
-      int nq0 = 0, nq1 = 0, nkv = 0;  // loads issued
+      int nq = 0, nkv = 0;  // query tiles and blocks issued
       bool ok = true;
-      auto load_block = [&](const CUtensorMap *map, int row, int rows) {
-        const int s = nkv % kAttRing;
-        if (nkv >= kAttRing)
-          ok = mbar_wait(smem_u32(&b_kvfree[s]), (uint32_t)((nkv / kAttRing - 1) & 1), abort);
+      auto load_block = [&](const CUtensorMap *map, uint32_t dst, uint64_t &full,
+                            uint64_t &freed, int row, int rows) {
+        if (ok && nkv > 0) ok = mbar_wait(smem_u32(&freed), (uint32_t)((nkv - 1) & 1), abort);
         if (!ok) return;
         const int nbox = (rows + kBox - 1) / kBox;
-        const uint32_t bar = smem_u32(&b_kvfull[s]), dst = aR + s * kTile;
+        const uint32_t bar = smem_u32(&full);
         mbar_expect_tx(bar, (uint32_t)nbox * 2 * kBox * 128);
         for (int b = 0; b < nbox; ++b)
           for (int hf = 0; hf < 2; ++hf)
             tma_load_2d(dst + hf * kHalf + b * kBox * 128, map, 64 * hf, row + b * kBox, bar);
-        ++nkv;
       };
+      int nk = 0, nv = 0;  // loads in flight to wait for at the end
       for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
         AttItem it;
-        if (!att_item(p, i, n_pairs, Jt, it)) continue;
-        for (int t = 0; t < 2 && ok; ++t) {
-          if (!it.nb(t)) continue;
-          int &nq = t ? nq1 : nq0;
-          if (nq > 0) ok = mbar_wait(smem_u32(&b_qfree[t]), (uint32_t)((nq - 1) & 1), abort);
-          if (!ok) break;
-          mbar_expect_tx(smem_u32(&b_qfull[t]), q_bytes);
-          for (int hf = 0; hf < 2; ++hf)
-            tma_load_4d(aQ + t * kTile + hf * kHalf, &tmQ, 64 * hf, 0, it.u.h,
-                        (int)it.u.row0 + it.tok0(t), smem_u32(&b_qfull[t]));
-          ++nq;
-        }
+        if (!att_item(p, i, units, n_qt, Jt, it)) continue;
         const int row0 = (int)(it.u.ug * (size_t)c.cap);
-        for (int j = 0; j < it.nb_max() && ok; ++j) {
-          const int rows = min(kBlk, it.lim_max() - j * kBlk);
-          load_block(&tmK, row0 + j * kBlk, rows);
-          if (ok) load_block(&tmV, row0 + j * kBlk, rows);
+        for (int j = 0; j < it.nb && ok; ++j) {
+          const int rows = min(kBlk, it.lim - j * kBlk);
+          load_block(&tmK, aK, b_kfull, b_kfree, row0 + j * kBlk, rows);
+          if (!ok) break;
+          ++nk;
+          if (j == 0) {
+            if (nq > 0) ok = mbar_wait(smem_u32(&b_qfree), (uint32_t)((nq - 1) & 1), abort);
+            if (!ok) break;
+            mbar_expect_tx(smem_u32(&b_qfull), q_bytes);
+            for (int hf = 0; hf < 2; ++hf)
+              tma_load_4d(aQ + hf * kHalf, &tmQ, 64 * hf, 0, it.u.h, (int)it.u.row0 + it.tok0,
+                          smem_u32(&b_qfull));
+            ++nq;
+          }
+          load_block(&tmV, aV, b_vfull, b_vfree, row0 + j * kBlk, rows);
+          if (!ok) break;
+          ++nv;
+          ++nkv;
         }
       }
       if (!ok) {
@@ -304,109 +309,67 @@ __global__ void __launch_bounds__(kThr, 1)
       // Whether or not another role gave up: every load issued lands
       // (bounded) before the CTA's shared memory is given back.
       volatile int never = 0;
-      if (nq0) mbar_wait(smem_u32(&b_qfull[0]), (uint32_t)((nq0 - 1) & 1), &never);
-      if (nq1) mbar_wait(smem_u32(&b_qfull[1]), (uint32_t)((nq1 - 1) & 1), &never);
-      for (int k = max(0, nkv - kAttRing); k < nkv; ++k)
-        mbar_wait(smem_u32(&b_kvfull[k % kAttRing]), (uint32_t)((k / kAttRing) & 1), &never);
+      if (nq) mbar_wait(smem_u32(&b_qfull), (uint32_t)((nq - 1) & 1), &never);
+      if (nk) mbar_wait(smem_u32(&b_kfull), (uint32_t)((nk - 1) & 1), &never);
+      if (nv) mbar_wait(smem_u32(&b_vfull), (uint32_t)((nv - 1) & 1), &never);
     }
   } else if (warp == 9) {
-    // Issuer: S_t(j) = Q_t K_j^T, then O_t += P_t(j) V_j once the softmax
-    // has put P in place of S.  One thread issues, and its MMAs run in the
-    // order of issue, so S_t(j + 1) may follow PV_t(j), whose P it replaces;
-    // each tile's softmax runs under the other tile's contractions.
-    int kv = 0;
-    uint32_t ph_q = 0, ph_p = 0;  // phases to wait for, bit t
+    // Issuer: S(j) = Q K_j^T, then O += P(j) V_j once the softmax has put P
+    // in place of S.  One thread issues, and its MMAs run in the order of
+    // issue, so S(j + 1) may follow PV(j), whose P it replaces.
+    int nk = 0, nv = 0, nq = 0;
     bool ok = true;
-    auto issue_s = [&](int t, int kst, int N) {
-      if (lane == 0) {
-        const uint32_t id = idesc_bf16(kBlk, N, false);
-        const uint64_t a0 = sdesc_sw128(aQ + t * kTile, 16, 1024);
-        const uint64_t b0 = sdesc_sw128(aR + kst * kTile, 16, 1024);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint64_t off = (uint64_t)(((k >> 2) * kHalf + (k & 3) * 32) >> 4);
-          tc_mma(tm + t * kBlk, a0 + off, b0 + off, id, k > 0);
-        }
-        tc_commit(smem_u32(&b_s[t]));
-      }
-    };
-    auto cols = [&](const AttItem &it, int t, int j) {
-      return min(kBlk, (it.lim(t) - j * kBlk + 15) & ~15);
-    };
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       AttItem it;
-      if (!att_item(p, i, n_pairs, Jt, it)) continue;
+      if (!att_item(p, i, units, n_qt, Jt, it)) continue;
       const int n = it.u.m + p.chunk;
-      int kst = kv % kAttRing;
-      ok = wait_warp(smem_u32(&b_kvfull[kst]), (uint32_t)((kv / kAttRing) & 1));
-      for (int t = 0; t < 2 && ok; ++t) {
-        if (!it.nb(t)) continue;
-        ok = wait_warp(smem_u32(&b_qfull[t]), (ph_q >> t) & 1);
+      for (int j = 0; j < it.nb; ++j) {
+        const int ncol = min(kBlk, (it.lim - j * kBlk + 15) & ~15);
+        ok = wait_warp(b_kfull, nk++) && (j > 0 || wait_warp(b_qfull, nq++));
         if (!ok) break;
-        ph_q ^= 1u << t;
         tc_fence_after();
-        issue_s(t, kst, cols(it, t, 0));
-        if (it.nb(t) == 1 && lane == 0) tc_commit(smem_u32(&b_qfree[t]));
-      }
-      if (!ok) break;
-      if (lane == 0) tc_commit(smem_u32(&b_kvfree[kst]));
-      ++kv;
-      for (int j = 0; j < it.nb_max() && ok; ++j) {
-        const int vst = kv % kAttRing;
-        ok = wait_warp(smem_u32(&b_kvfull[vst]), (uint32_t)((kv / kAttRing) & 1));
+        if (lane == 0) {
+          const uint32_t id = idesc_bf16(kBlk, ncol, false);
+          const uint64_t a0 = sdesc_sw128(aQ, 16, 1024), b0 = sdesc_sw128(aK, 16, 1024);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const uint64_t off = (uint64_t)(((k >> 2) * kHalf + (k & 3) * 32) >> 4);
+            tc_mma(tm, a0 + off, b0 + off, id, k > 0);
+          }
+          tc_commit(smem_u32(&b_s));
+          tc_commit(smem_u32(&b_kfree));
+          if (j + 1 == it.nb) tc_commit(smem_u32(&b_qfree));
+        }
+        ok = wait_warp(b_vfull, nv);
         if (!ok) break;
-        ++kv;
         // V rows past the unit's last one, up to the 16-row step of PV,
         // meet P = 0 and must be finite: zeros.
         const int v0 = n - j * kBlk, v1 = min(kBlk, (v0 + 15) & ~15);
-        if (it.lim_max() == n && v0 > 0 && v0 < v1) {
-          unsigned char *V = smem + 2 * kTile + vst * kTile;
+        if (it.lim == n && v0 > 0 && v0 < v1) {
+          unsigned char *V = smem + 2 * kTile;
           for (int x = lane; x < (v1 - v0) * 16; x += 32)
             reinterpret_cast<int4 *>(V + ((x >> 3) & 1) * kHalf + (v0 + (x >> 4)) * 128)[x & 7] =
                 make_int4(0, 0, 0, 0);
           fence_proxy_async();
           __syncwarp();
         }
-        bool have_k = false;
-        kst = kv % kAttRing;
-        for (int t = 0; t < 2 && ok; ++t) {
-          if (j < it.nb(t)) {
-            ok = wait_warp(smem_u32(&b_p[t]), (ph_p >> t) & 1);
-            if (!ok) break;
-            ph_p ^= 1u << t;
-            tc_fence_after();
-            if (lane == 0) {
-              const uint32_t id = idesc_bf16(kBlk, kBlk, true);
-              const uint64_t b0 = sdesc_sw128(aR + vst * kTile, kHalf, 1024);
-              const int nk = cols(it, t, j) / 16;
-              for (int k = 0; k < nk; ++k) {
-                const uint32_t aP = tm + t * kBlk + 16 * k;
-                const uint64_t b = b0 + (uint64_t)(k * 128);
-                tc_mma_ts(tm + 2 * kBlk + t * kBlk, aP, b, id, j > 0 || k > 0);
-                tc_mma_ts(tm + 2 * kBlk + t * kBlk, aP + 8, b, id, true);
-              }
-              if (j + 1 == it.nb(t)) tc_commit(smem_u32(&b_o[t]));
-            }
-          }
-          if (j + 1 < it.nb(t)) {
-            if (!have_k) {
-              ok = wait_warp(smem_u32(&b_kvfull[kst]), (uint32_t)((kv / kAttRing) & 1));
-              if (!ok) break;
-              have_k = true;
-            }
-            tc_fence_after();
-            issue_s(t, kst, cols(it, t, j + 1));
-            if (j + 2 == it.nb(t) && lane == 0) tc_commit(smem_u32(&b_qfree[t]));
-          }
-        }
+        ok = wait_warp(b_p, nv++);
         if (!ok) break;
+        tc_fence_after();
         if (lane == 0) {
-          tc_commit(smem_u32(&b_kvfree[vst]));
-          if (have_k) tc_commit(smem_u32(&b_kvfree[kst]));
+          const uint32_t id = idesc_bf16(kBlk, kBlk, true);
+          const uint64_t b0 = sdesc_sw128(aV, kHalf, 1024);
+          for (int k = 0; k < ncol / 16; ++k) {
+            const uint64_t b = b0 + (uint64_t)(k * 128);
+            tc_mma_ts(tmO, tm + 16 * k, b, id, j > 0 || k > 0);
+            tc_mma_ts(tmO, tm + 16 * k + 8, b, id, true);
+          }
+          tc_commit(smem_u32(&b_vfree));
+          if (j + 1 == it.nb) tc_commit(smem_u32(&b_o));
         }
-        if (have_k) ++kv;
       }
     }
+    __syncwarp();
     if (lane == 0) {
       if (!ok) {
         if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
@@ -417,94 +380,128 @@ __global__ void __launch_bounds__(kThr, 1)
       tc_commit(smem_u32(&b_drain));
       mbar_wait(smem_u32(&b_drain), 0, &never);
     }
-  } else if (warp < 8) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
-    // Softmax warpgroup t: thread r owns query row r of tile t.
-    const int t = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
+  } else {
+    // Softmax: two warpgroups, each with half of a block's columns; thread r
+    // of either owns query row r.  The warps of the two that share 32 rows
+    // agree on the rows' reference over a named barrier.
+    const int hf = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
     const uint32_t lanes = (uint32_t)(wq * 32) << 16;
-    const uint32_t tS = tm + t * kBlk + lanes, tO = tm + 2 * kBlk + t * kBlk + lanes;
+    const int c0 = hf * 64;
+    const uint32_t tS = tm + c0 + lanes, tO = tmO + c0 + lanes;
+    const int pair_bar = 1 + wq;
+    float *mine = &s_x[hf][r];
+    const float *theirs = &s_x[hf ^ 1][r];
+    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory"); };
+    auto pair_any = [&](bool x) {
+      int y;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+          "barrier.cta.red.or.pred q, %2, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+          : "=r"(y)
+          : "r"((int)x), "r"(pair_bar)
+          : "memory");
+      return y != 0;
+    };
+    // Tell the partner v; a warp whose wait ran out says so instead, and both
+    // leave (no warp is left at the pair's barrier).
+    auto exchange = [&](bool good, float v) {
+      *mine = good ? v : __uint_as_float(kGaveUp);
+      pair_sync();
+      return good && __float_as_uint(*theirs) != kGaveUp;
+    };
     const float scale = p.scale_log2e;
-    const uint64_t scale2 = pk2(scale, scale);
+    const uint64_t scale2 = pk2(scale, scale), minus2 = pk2(-1.f, -1.f);
+    const int tk = r / G;
     int ns = 0, no = 0;
     bool ok = true;
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       AttItem it;
-      if (!att_item(p, i, n_pairs, Jt, it) || !it.nb(t)) continue;
-      const int tk = r / G;
-      const bool valid = tk < it.toks(t) && r < Jt * G;
-      // Rows the query sees (rows past the tile's tokens follow the last).
-      const int seen = it.u.m + it.tok0(t) + min(tk, it.toks(t) - 1) + 1;
-      const int seen_w = it.u.m + it.tok0(t) + min(32 * wq / G, it.toks(t) - 1) + 1;
+      if (!att_item(p, i, units, n_qt, Jt, it)) continue;
+      const bool valid = tk < it.toks && r < Jt * G;
+      // Rows the query sees (rows past the tile's tokens follow the last),
+      // and the first query of this warp; of this half's columns.
+      const int first = it.u.m + it.tok0 + 1 - c0;
+      const int seen = first + min(tk, it.toks - 1);
+      const int seen_w = first + min(32 * wq / G, it.toks - 1);
       float ref = 0.f, l = 0.f;
-      for (int j = 0; j < it.nb(t); ++j) {
-        ok = wait_warp(smem_u32(&b_s[t]), (uint32_t)(ns++ & 1));
-        if (!ok) break;
+      for (int j = 0; j < it.nb; ++j) {
+        ok = wait_warp(b_s, ns++);
         tc_fence_after();
-        const int ncol = min(kBlk, it.lim(t) - j * kBlk);  // columns of S in use
-        float e[4][32];
+        // This half's columns in use, 32 at a time: a first reading for the
+        // maximum, a second for the exponentials (TMEM reads are cheap; the
+        // registers to keep 64 logits are not there).
+        const int ncol = it.lim - c0 - j * kBlk, lim = seen - j * kBlk,
+                  lim_w = seen_w - j * kBlk;
+        auto load_s = [&](int k, float(&e)[32]) {
+          tmem_ld32(tS + 32 * k, e);
+          tmem_wait_ld();
+          if (lim_w < 32 * k + 32) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (32 * k < ncol) tmem_ld32(tS + 32 * k, e[k]);
-        tmem_wait_ld();
-        const int lim = seen - j * kBlk;
+            for (int x = 0; x < 32; ++x) e[x] = 32 * k + x < lim ? e[x] : -INFINITY;
+          }
+        };
         float mx = -INFINITY;
-        if (seen_w - j * kBlk >= kBlk) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < 2; ++k) {
+          if (ok && 32 * k < ncol) {
+            float e[32];
+            load_s(k, e);
 #pragma unroll
-            for (int x = 0; x < 32; x += 2) mx = fmaxf(mx, fmaxf(e[k][x], e[k][x + 1]));
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (32 * k < ncol) {
-#pragma unroll
-              for (int x = 0; x < 32; ++x) {
-                e[k][x] = 32 * k + x < lim ? e[k][x] : -INFINITY;
-                mx = fmaxf(mx, e[k][x]);
-              }
-            }
+            for (int x = 0; x < 32; x += 2) mx = fmaxf(mx, fmaxf(e[x], e[x + 1]));
           }
         }
         mx *= scale;
         if (j == 0) {
+          if (!exchange(ok, mx)) {
+            ok = false;
+            break;
+          }
+          mx = fmaxf(mx, *theirs);
           ref = mx == -INFINITY ? 0.f : mx;
-        } else {
+        } else if (pair_any(!ok || mx > ref + kLazy)) {
+          if (!exchange(ok, mx)) {
+            ok = false;
+            break;
+          }
+          mx = fmaxf(mx, *theirs);
           const bool up = mx > ref + kLazy;
-          if (__any_sync(0xffffffffu, up)) {
-            // O holds the blocks before this one (S of this block was
-            // committed after their PV).
-            const float f = up ? ex2(ref - mx) : 1.f;
-            if (up) ref = mx;
-            l *= f;
+          // O holds the blocks before this one (S of this block was
+          // committed after their PV).
+          const float f = up ? ex2(ref - mx) : 1.f;
+          if (up) ref = mx;
+          l *= f;
 #pragma unroll 1
-            for (int k = 0; k < kBlk; k += 16) {
-              uint32_t o[16];
-              tmem_ld16(tO + k, o);
+          for (int k = 0; k < 64; k += 16) {
+            uint32_t o[16];
+            tmem_ld16(tO + k, o);
 #pragma unroll
-              for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * f);
-              tmem_st16(tO + k, o);
-            }
+            for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * f);
+            tmem_st16(tO + k, o);
           }
         }
         const uint64_t nref2 = pk2(-ref, -ref);
         uint64_t sum2 = pk2(0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2; ++k) {
           if (32 * k < ncol) {
+            float e[32];
+            load_s(k, e);
             uint32_t w[32];
 #pragma unroll
             for (int x = 0; x < 32; x += 2) {
               float d0, d1;
-              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, nref2), d0, d1);
-              d0 = ex2(d0);  // exp2(-inf) = 0 for masked keys
-              d1 = ex2(d1);
-              const uint64_t p2 = pk2(d0, d1);
+              upk2(fma2(pk2(e[x], e[x + 1]), scale2, nref2), d0, d1);
+              const uint64_t p2 = pk2(ex2(d0), ex2(d1));  // exp2(-inf) = 0 for masked keys
               sum2 = add2(sum2, p2);
-              const __nv_bfloat162 b = __floats2bfloat162_rn(d0, d1);
-              float r0, r1;  // p - bf16(p)
-              upk2(add2(p2, pk2(-__low2float(b), -__high2float(b))), r0, r1);
+              float p0, p1, r0, r1;
+              upk2(p2, p0, p1);
+              const uint32_t b = pack_bf16(p0, p1);
+              // p - bf16(p), exact
+              upk2(fma2(pk2(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u)),
+                        minus2, p2),
+                   r0, r1);
               const int at = (x >> 4) * 16 + ((x & 15) >> 1);
-              w[at] = *reinterpret_cast<const uint32_t *>(&b);
+              w[at] = b;
               w[at + 8] = pack_bf16(r0, r1);
             }
             tmem_st32(tS + 32 * k, w);  // 8 hi then 8 lo columns each 16 keys
@@ -516,35 +513,45 @@ __global__ void __launch_bounds__(kThr, 1)
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&b_p[t]));
+        if (lane == 0) mbar_arrive(smem_u32(&b_p));
       }
       if (!ok) break;
-      ok = wait_warp(smem_u32(&b_o[t]), (uint32_t)(no++ & 1));
-      if (!ok) break;
+      ok = wait_warp(b_o, no++);
+      if (!exchange(ok, l)) {
+        ok = false;
+        break;
+      }
+      l += *theirs;
       tc_fence_after();
       // The largest term is 2^(x - ref) with ref the rounded x: about 1.
       if (valid && !(l >= 0.5f && l < INFINITY)) atomicOr(c.err, ERR_NONFINITE);
       const float inv = 1.f / l;
-      const size_t qrow = ((it.u.row0 + it.tok0(t) + tk) * c.H + it.u.h) * G + (r - tk * G);
-      int4 *orow = reinterpret_cast<int4 *>(p.out) + qrow * 16;
+      const size_t qrow = ((it.u.row0 + it.tok0 + tk) * c.H + it.u.h) * G + (r - tk * G);
+      unsigned char *orow = reinterpret_cast<unsigned char *>(p.out) + qrow * 256 + 128 * hf;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < 2; ++k) {
         float o[32];
         tmem_ld32(tO + 32 * k, o);
         tmem_wait_ld();
         if (valid) {
+          uint32_t w[16];
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            const float *v = o + 8 * x;
-            orow[4 * k + x] =
-                make_int4(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[2] * inv, v[3] * inv),
-                          pack_bf16(v[4] * inv, v[5] * inv), pack_bf16(v[6] * inv, v[7] * inv));
+          for (int x = 0; x < 16; ++x) w[x] = pack_bf16(o[2 * x] * inv, o[2 * x + 1] * inv);
+          if (out32) {
+            st_global32(orow + 64 * k, w);
+            st_global32(orow + 64 * k + 32, w + 8);
+          } else {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              reinterpret_cast<int4 *>(orow + 64 * k)[x] =
+                  make_int4(w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
           }
         }
       }
-      if (valid)
-        lse[it.u.ug * (size_t)G * c.cap + (size_t)it.tok0(t) * G + r] = ref + log2f(l);
+      if (valid && hf == 0)
+        lse[it.u.ug * (size_t)G * c.cap + (size_t)it.tok0 * G + r] = ref + log2f(l);
       tc_fence_before();
+      pair_sync();  // the partner has read this row's sum
     }
     if (!ok && lane == 0) {
       if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
@@ -553,7 +560,7 @@ __global__ void __launch_bounds__(kThr, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) tmem_dealloc(tm, kTmemCols);
+  if (warp == 8) tmem_dealloc(tm, kAttCols);
 }
 
 // ---- 3. score -----------------------------------------------------------------
@@ -569,10 +576,11 @@ struct ScoreItem {
   __device__ int nk(int t) const { return min(kBlk, n - k0 - t * kBlk); }
 };
 
-__device__ __forceinline__ bool score_item(const AbsorbParams &p, int i, int n_kp, int Jt,
+__device__ __forceinline__ bool score_item(const AbsorbParams &p, int i, int Jt,
                                            ScoreItem &it) {
-  const int x = i / n_kp, kp = (i % n_kp + x) % n_kp;
-  it.u = unit_at(p, x);
+  // The first rows, which every token sees, of every unit first.
+  const int units = p.c.S * p.nl * p.c.H, kp = i / units;
+  it.u = unit_at(p, i % units);
   if (!unit_ok(p, it.u)) return false;
   it.n = it.u.m + p.chunk;
   it.k0 = 2 * kBlk * kp;
@@ -580,10 +588,10 @@ __device__ __forceinline__ bool score_item(const AbsorbParams &p, int i, int n_k
   return it.k0 < it.n;
 }
 
-__global__ void __launch_bounds__(kThr, 1)
+__global__ void __launch_bounds__(kScThr, 1)
     long_score_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmQ, const float *lse, int n_items,
-                      int n_kp, int n_qt) {
+                      int n_qt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
@@ -600,7 +608,7 @@ __global__ void __launch_bounds__(kThr, 1)
   auto wait_warp = [&](uint32_t bar, uint32_t parity) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) != 0;
   };
-  if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+  if (warp == kProducer) tmem_alloc(smem_u32(&s_tmem), kScCols);
   if (tid == 0) {
     for (int t = 0; t < 2; ++t) {
       mbar_init(smem_u32(&b_kfull[t]), 1);
@@ -618,7 +626,7 @@ __global__ void __launch_bounds__(kThr, 1)
     s_abort = 0;
     fence_mbar_init();
   }
-  for (int i = tid; i < kQRing * 2 * (kBlk - Jt * G) * 8; i += kThr) {
+  for (int i = tid; i < kQRing * 2 * (kBlk - Jt * G) * 8; i += kScThr) {
     const int row = Jt * G + (i >> 3) % (kBlk - Jt * G), hf = (i >> 3) / (kBlk - Jt * G);
     reinterpret_cast<int4 *>(smem + 4 * kTile + hf * kHalf + row * 128)[i & 7] =
         make_int4(0, 0, 0, 0);
@@ -630,7 +638,7 @@ __global__ void __launch_bounds__(kThr, 1)
   pdl_begin();
   const uint32_t tm = s_tmem;
 
-  if (warp == 8) {
+  if (warp == kProducer) {
     // Producer: key tiles (two pairs in flight), query tiles and their
     // rows' normalisers.
     if (lane == 0) {
@@ -642,7 +650,7 @@ __global__ void __launch_bounds__(kThr, 1)
     bool ok = true;
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       ScoreItem it;
-      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      if (!score_item(p, i, Jt, it)) continue;
       const int kb = nk & 1;
       if (nk >= 2) ok = wait_warp(smem_u32(&b_kfree[kb]), (uint32_t)((nk / 2 - 1) & 1));
       if (!ok) break;
@@ -695,13 +703,13 @@ __global__ void __launch_bounds__(kThr, 1)
       for (int k = max(0, nq - kQRing); k < nq; ++k)
         mbar_wait(smem_u32(&b_qfull[k % kQRing]), (uint32_t)((k / kQRing) & 1), &never);
     }
-  } else if (warp == 9) {
+  } else if (warp == kIssuer) {
     int nk = 0, nq = 0, ns0 = 0, ns1 = 0;
     bool ok = true;
     const uint32_t id = idesc_bf16(kBlk, kBlk, false);
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       ScoreItem it;
-      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      if (!score_item(p, i, Jt, it)) continue;
       const int kb = nk & 1;
       ok = wait_warp(smem_u32(&b_kfull[kb]), (uint32_t)((nk / 2) & 1));
       for (int q = it.q0(0); q < n_qt && ok; ++q) {
@@ -743,89 +751,113 @@ __global__ void __launch_bounds__(kThr, 1)
       tc_commit(smem_u32(&b_drain));
       mbar_wait(smem_u32(&b_drain), 0, &never);
     }
-  } else if (warp < 8) {
-    // Warpgroup t: thread r owns key row r of tile t.
-    const int t = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
-    const uint32_t tS = tm + t * 2 * kBlk + ((uint32_t)(wq * 32) << 16);
+  } else if (warp < kProducer) {
+    // Two warpgroups a key tile, which take its S buffers in turn; thread r
+    // of either owns key row r.
+    const int t = warp >> 3, b = (warp >> 2) & 1, wq = warp & 3, r = wq * 32 + lane;
+    const uint32_t tS = tm + (t * 2 + b) * kBlk + ((uint32_t)(wq * 32) << 16);
     const uint64_t scale2 = pk2(p.scale_log2e, p.scale_log2e);
     int nq = 0, ns = 0;
     bool ok = true;
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       ScoreItem it;
-      if (!score_item(p, i, n_kp, Jt, it)) continue;
+      if (!score_item(p, i, Jt, it)) continue;
       const int slot = it.k0 + t * kBlk + r;
       const int tmin = max(0, slot - it.u.m);  // first token that sees the row
       const int tmin_w = max(0, it.k0 + t * kBlk + wq * 32 + 31 - it.u.m);
+      const int q1 = it.nk(t) > 0 ? it.q0(t) : n_qt;
       uint64_t a0 = pk2(0.f, 0.f), a1 = a0;
       for (int q = it.q0(0); q < n_qt; ++q) {
         const int s = nq % kQRing;
         const uint32_t ph_q = (uint32_t)((nq / kQRing) & 1);
         ++nq;
-        if (it.nk(t) <= 0 || q < it.q0(t)) {
-          // Nothing to read; the arrival counts for this filling of the slot.
-          ok = wait_warp(smem_u32(&b_qfull[s]), ph_q);
-          if (!ok) break;
-          if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+        // One of the tile's two warpgroups releases each query tile: the one
+        // that reads it, or the first where the tile has nothing to read (its
+        // arrival must count for this filling of the slot, hence the wait).
+        if (q < q1) {
+          if (b == 0) {
+            ok = wait_warp(smem_u32(&b_qfull[s]), ph_q);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+          }
           continue;
         }
-        const int b = ns & 1;
-        ok = wait_warp(smem_u32(&b_s[t][b]), (uint32_t)((ns / 2) & 1)) &&
+        const int n = ns++;
+        if ((n & 1) != b) continue;
+        ok = wait_warp(smem_u32(&b_s[t][b]), (uint32_t)((n / 2) & 1)) &&
              wait_warp(smem_u32(&b_qfull[s]), ph_q);
         if (!ok) break;
-        ++ns;
         tc_fence_after();
-        float e[4][32];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) tmem_ld32(tS + b * kBlk + 32 * k, e[k]);
-        tmem_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&b_sfree[t][b]));
-        const ulonglong2 *nl = reinterpret_cast<const ulonglong2 *>(s_lse + s * kBlk);
         const int toks = p.chunk - q * Jt;  // tokens from this tile on
-        if (q * Jt >= tmin_w && toks >= Jt) {
+        const bool all = q * Jt >= tmin_w && toks >= Jt;
+        // Columns of tokens before tmin do not see the row; columns past the
+        // chunk hold no query.
+        const int c_lo = (tmin - q * Jt) * G, c_hi = min(Jt, toks) * G;
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
+        for (int hf = 0; hf < 2; ++hf) {
+          float e[2][32];
+          tmem_ld32(tS + 64 * hf, e[0]);
+          tmem_ld32(tS + 64 * hf + 32, e[1]);
+          tmem_wait_ld();
+          if (hf == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&b_sfree[t][b]));
+          }
+          const ulonglong2 *nl = reinterpret_cast<const ulonglong2 *>(s_lse + s * kBlk + 64 * hf);
+          if (all) {
 #pragma unroll
-            for (int x = 0; x < 32; x += 4) {
-              const ulonglong2 z = nl[(32 * k + x) >> 2];
-              float d0, d1, d2, d3;
-              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d0, d1);
-              upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d2, d3);
-              a0 = add2(a0, pk2(ex2(d0), ex2(d1)));
-              a1 = add2(a1, pk2(ex2(d2), ex2(d3)));
-            }
-        } else {
-          // The diagonal tiles and the last one: columns of tokens before
-          // tmin do not see the row; columns past the chunk hold no query.
-          const int c_lo = (tmin - q * Jt) * G, c_hi = min(Jt, toks) * G;
+            for (int k = 0; k < 2; ++k)
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int x = 0; x < 32; x += 4) {
-              const ulonglong2 z = nl[(32 * k + x) >> 2];
-              float d[4];
-              upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d[0], d[1]);
-              upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d[2], d[3]);
-#pragma unroll
-              for (int y = 0; y < 4; ++y) {
-                const int col = 32 * k + x + y;
-                d[y] = col >= c_lo && col < c_hi ? ex2(d[y]) : 0.f;
+              for (int x = 0; x < 32; x += 4) {
+                const ulonglong2 z = nl[(32 * k + x) >> 2];
+                float d0, d1, d2, d3;
+                upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d0, d1);
+                upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d2, d3);
+                a0 = add2(a0, pk2(ex2(d0), ex2(d1)));
+                a1 = add2(a1, pk2(ex2(d2), ex2(d3)));
               }
-              a0 = add2(a0, pk2(d[0], d[1]));
-              a1 = add2(a1, pk2(d[2], d[3]));
-            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+              for (int x = 0; x < 32; x += 4) {
+                const ulonglong2 z = nl[(32 * k + x) >> 2];
+                float d[4];
+                upk2(fma2(pk2(e[k][x], e[k][x + 1]), scale2, z.x), d[0], d[1]);
+                upk2(fma2(pk2(e[k][x + 2], e[k][x + 3]), scale2, z.y), d[2], d[3]);
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                  const int col = 64 * hf + 32 * k + x + y;
+                  d[y] = col >= c_lo && col < c_hi ? ex2(d[y]) : 0.f;
+                }
+                a0 = add2(a0, pk2(d[0], d[1]));
+                a1 = add2(a1, pk2(d[2], d[3]));
+              }
+          }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
       }
-      if (!ok) break;
-      if (slot < it.n) {
-        float x0, x1, y0, y1;
-        upk2(a0, x0, x1);
-        upk2(a1, y0, y1);
-        c.score[it.u.ug * (size_t)c.sstride + slot] += ((x0 + x1) + (y0 + y1)) * p.inv_g;
+      // The two warpgroups' sums, added one after the other.
+      float x0, x1, y0, y1;
+      upk2(a0, x0, x1);
+      upk2(a1, y0, y1);
+      const float sum = ((x0 + x1) + (y0 + y1)) * p.inv_g;
+      float *su = c.score + it.u.ug * (size_t)c.sstride + slot;
+      if (b == 0 && ok && slot < it.n) *su += sum;
+      int bad;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+          "barrier.cta.red.or.pred q, %2, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+          : "=r"(bad)
+          : "r"(ok ? 0 : 1), "r"(1 + t)
+          : "memory");
+      if (bad) {
+        ok = false;
+        break;
       }
+      if (b == 1 && slot < it.n) *su += sum;
     }
     if (!ok && lane == 0) {
       if (!*abort) atomicOr(c.err, ERR_TIMEOUT);
@@ -834,7 +866,7 @@ __global__ void __launch_bounds__(kThr, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) tmem_dealloc(tm, kTmemCols);
+  if (warp == kProducer) tmem_dealloc(tm, kScCols);
 }
 
 }  // namespace
@@ -847,7 +879,7 @@ cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
   if (p.chunk < 1 || p.c.G > 8 || p.c.d != 128 || !p.c.kv_bf16 || !p.c.out_bf16)
     return cudaErrorInvalidValue;
   const int units = p.c.S * p.nl * p.c.H;
-  const int Jt = kBlk / p.c.G, n_qt = (p.chunk + Jt - 1) / Jt, n_pairs = (n_qt + 1) / 2;
+  const int Jt = kBlk / p.c.G, n_qt = (p.chunk + Jt - 1) / Jt;
   const int n_kp = (p.max_rows + 2 * kBlk - 1) / (2 * kBlk);
   cudaError_t e = cudaFuncSetAttribute(
       long_attend_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
@@ -861,12 +893,13 @@ cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
   e = launch_pdl(long_append_kernel,
                  dim3(units, (p.chunk + kAppendRows - 1) / kAppendRows), dim3(256), 0, st, p);
   if (e != cudaSuccess) return e;
-  const int n_att = units * n_pairs, n_sc = units * n_kp;
-  e = launch_pdl(long_attend_kernel, dim3(n_att < sms ? n_att : sms), dim3(kThr),
-                 (size_t)kAttSmem, st, p, tmK, tmV, tmQ, lse, n_att, n_pairs);
+  const int n_att = units * n_qt, n_sc = units * n_kp;
+  e = launch_pdl(long_attend_kernel, dim3(n_att < 2 * sms ? n_att : 2 * sms), dim3(kAttThr),
+                 (size_t)kAttSmem, st, p, tmK, tmV, tmQ, lse, n_att, n_qt,
+                 reinterpret_cast<uintptr_t>(p.out) % 32 == 0 ? 1 : 0);
   if (e != cudaSuccess) return e;
-  return launch_pdl(long_score_kernel, dim3(n_sc < sms ? n_sc : sms), dim3(kThr),
-                    (size_t)kScoreSmem, st, p, tmK, tmQ, (const float *)lse, n_sc, n_kp, n_qt);
+  return launch_pdl(long_score_kernel, dim3(n_sc < sms ? n_sc : sms), dim3(kScThr),
+                    (size_t)kScoreSmem, st, p, tmK, tmQ, (const float *)lse, n_sc, n_qt);
 }
 
 }  // namespace kvr
