@@ -426,7 +426,8 @@ bool try_stream(kvr_cache *c, const StepArgs &a, bool evict, int budget,
 // of up to n_max rows: the first of (4,2) (3,3) (3,2) (2,3) (2,2) (1,3)
 // (1,2) that fits in shared memory (more groups first: measured), or the
 // tuned choice.
-bool chunk_config(const kvr_cache *c, int n_max, int *groups, int *stages) {
+bool chunk_config(const kvr_cache *c, int n_max, int *groups, int *stages,
+                  bool rkv = false) {
   static const int order[7][2] = {{4, 2}, {3, 3}, {3, 2}, {2, 3},
                                   {2, 2}, {1, 3}, {1, 2}};
   const size_t limit = (size_t)c->smem_optin - 512;
@@ -434,7 +435,7 @@ bool chunk_config(const kvr_cache *c, int n_max, int *groups, int *stages) {
   for (const auto &o : order) {
     const int g = tg > 0 ? tg : o[0], s = ts > 0 ? ts : o[1];
     if (g > kvr::chunk_max_groups() || s > kvr::chunk_max_stages()) continue;
-    if (kvr::chunk_smem_bytes(n_max, g, s) <= limit) {
+    if (kvr::chunk_smem_bytes(n_max, g, s, rkv) <= limit) {
       *groups = g;
       *stages = s;
       return true;
@@ -445,7 +446,8 @@ bool chunk_config(const kvr_cache *c, int n_max, int *groups, int *stages) {
 
 // Launch the chunked step for plain units if this call qualifies.
 bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
-                 int window, cudaStream_t stream, cudaError_t *err) {
+                 int window, cudaStream_t stream, cudaError_t *err,
+                 bool rkv = false, float lam = 0.f) {
   const CacheView &v = c->view;
   if (!c->fused || c->chunk_groups < 0 || !v.kv_bf16 || v.d != 128 ||
       v.G > 8)
@@ -460,11 +462,13 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
     return false;
   if (!device_facts(c)) return false;
   kvr::ChunkParams p{};
-  if (!chunk_config(c, a.max_rows, &p.n_groups, &p.n_stages)) return false;
+  if (!chunk_config(c, a.max_rows, &p.n_groups, &p.n_stages, rkv)) return false;
   const std::pair<CUtensorMap, CUtensorMap> *maps =
       slab_maps(c, kvr::chunk_box_rows());
   if (!maps) return false;
   p.c = v;
+  p.rkv = rkv ? 1 : 0;
+  p.lam = lam;
   p.fork = 0;
   p.q = static_cast<const __nv_bfloat16 *>(a.q);
   p.k_new = static_cast<const __nv_bfloat16 *>(a.k_new);
@@ -482,6 +486,44 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
   const int grid = std::min(c->sm_count, p.n_jobs);
   *err = kvr::launch_chunk_step(maps->first, maps->second, nullptr, nullptr, p,
                                 grid, stream);
+  return true;
+}
+
+// Launch the clustered step (units of any length, no eviction) if this call
+// qualifies.
+bool try_long_step(kvr_cache *c, const StepArgs &a, cudaStream_t stream,
+                   cudaError_t *err) {
+  const CacheView &v = c->view;
+  if (!c->fused || !v.kv_bf16 || v.d != 128 || v.G > 8) return false;
+  const size_t rows = (size_t)v.S * v.L * v.H * v.cap;
+  const long long units = (long long)v.S * a.nl * v.H;
+  if (rows >= (size_t)INT32_MAX || units > 65535) return false;
+  if (!aligned16(a.q) || !aligned16(a.k_new) || !aligned16(a.v_new) ||
+      !aligned16(a.out))
+    return false;
+  const std::pair<CUtensorMap, CUtensorMap> *maps =
+      slab_maps(c, kvr::split_rows_per_stage());
+  if (!maps) return false;
+  kvr::SplitParams p{};
+  p.c = v;
+  p.q = static_cast<const __nv_bfloat16 *>(a.q);
+  p.k_new = static_cast<const __nv_bfloat16 *>(a.k_new);
+  p.v_new = static_cast<const __nv_bfloat16 *>(a.v_new);
+  p.lb = a.lb;
+  p.nl = a.nl;
+  p.scale_log2e = v.scale * 1.4426950408889634f;
+  // The longest sequences start first, so that the launch does not end with
+  // a few CTAs streaming the longest unit.
+  kvr::SeqOrder order{};
+  if (v.S <= kvr::kMaxOrder) {
+    for (int s = 0; s < v.S; ++s) order.seq[s] = (uint16_t)s;
+    const int L = v.L;
+    std::stable_sort(order.seq, order.seq + v.S, [&](uint16_t x, uint16_t y) {
+      return c->len[(size_t)x * L + a.lb] > c->len[(size_t)y * L + a.lb];
+    });
+  }
+  *err = kvr::launch_long_step(maps->first, maps->second, p, order, a.max_rows,
+                               a.out, stream);
   return true;
 }
 
@@ -695,7 +737,8 @@ kvr_status kvr_decode_attend_score(kvr_cache *c, int lb, int le, const void *q,
   cudaError_t e = cudaSuccess;
   if (!try_fused(c, a, false, 0, 0, as_stream(stream), &e) &&
       !try_chunked(c, a, false, 0, 0, as_stream(stream), &e) &&
-      !try_stream(c, a, false, 0, 0, as_stream(stream), &e))
+      !try_stream(c, a, false, 0, 0, as_stream(stream), &e) &&
+      !try_long_step(c, a, as_stream(stream), &e))
     e = kvr::launch_attend_score_generic(c->view, a, as_stream(stream));
   if (e != cudaSuccess) return cuda_fail("kvr_decode_attend_score", e);
   c->launches += 1;
@@ -999,10 +1042,12 @@ kvr_status kvr_decode_step_rkv(kvr_cache *c, int lb, int le, const void *q,
     return fail(KVR_EINVAL, "mix weight %g outside [0, 1]", (double)lambda);
   StepArgs a = step_args(c, lb, le, q, k_new, v_new, out);
   cudaError_t e = cudaSuccess;
-  if (try_fused(c, a, true, budget, window, as_stream(stream), &e, true,
-                lambda)) {
+  const bool one = try_fused(c, a, true, budget, window, as_stream(stream), &e,
+                             true, lambda);
+  if (one || try_chunked(c, a, true, budget, window, as_stream(stream), &e, true,
+                         lambda)) {
     if (e != cudaSuccess) return cuda_fail("kvr_decode_step_rkv", e);
-    c->launches += 1;
+    c->launches += one ? 1 : 2;
     mirror_append(c, lb, le);
     mirror_evict(c, lb, le, budget, window);
     return KVR_OK;

@@ -9,9 +9,14 @@
 //   they fit, else in the cache's per-unit logit scratch; K and V are each
 //   read once.
 // evict_kernel: TopB of Eq. 1 with the protected recent window of Sec. 4.1:
-//   a block radix select of the B-th best (score, -position) key among the
-//   non-window rows, then an in-place compaction that moves the survivors
-//   lying beyond the new length into the freed slots below it.
+//   by rank where every row has a thread, else a histogram select of the B-th
+//   best score among the non-window rows (ties to the lower position), then an
+//   in-place compaction that moves the survivors lying beyond the new length
+//   into the freed slots below it.  Long units are bound by the passes over
+//   their rows: scores are kept in shared memory, the lists take two passes
+//   and one exchange of counts (448 units of 700 to 16,384 rows: 152 us with
+//   64-bit keys read from global memory eight times and block-wide list
+//   building, 55 now; 1,792 units of 697 rows: 96 and 62).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -192,15 +197,99 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
-    evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow) {
+// The need-th largest of v(i) over the rows i in [0, n) with v(i) != kNone, by
+// passes over a 2,048-bin histogram, each over the range that the last one
+// left: first the values' own range (scores share their leading bits, and
+// bins by those would take all the additions), three passes at most.  Returns
+// the value; *rest is how many of the rows that equal it belong to the `need`,
+// *ties how many rows equal it.  need >= 1 and at least `need` such rows must
+// exist.  lo, hi: the least and greatest value among the rows that this thread
+// has seen (kNone, 0 for none); every row must have been seen by some thread.
+// Every thread must call it.
+constexpr unsigned kNone = 0xFFFFFFFFu;
+struct SelectSmem {
+  unsigned hist[2048];
+  unsigned wsum[32], wmax[32];
+  unsigned digit, above, count;
+};
+template <int NT, typename Val>
+__device__ unsigned select_desc(int n, unsigned need, Val v, unsigned lo, unsigned hi,
+                                SelectSmem &m, unsigned *rest, unsigned *ties) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kPer = 2048 / NT;  // bins a thread scans
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    m.wsum[warp] = lo;
+    m.wmax[warp] = hi;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    lo = min(lo, m.wsum[w]);
+    hi = max(hi, m.wmax[w]);
+  }
+  int shift = max(0, 32 - __clz((int)(hi - lo)) - 11);
+  unsigned bins = 2048;  // of the range left
+  for (bool last = false; !last;) {
+    last = shift == 0;
+    for (int i = tid; i < 2048; i += NT) m.hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NT) {
+      const unsigned x = v(i), bin = (x - lo) >> shift;
+      if (x != kNone && bin < bins) atomicAdd(&m.hist[bin], 1u);
+    }
+    __syncthreads();
+    // Inclusive counts from the top bin down; thread t owns kPer bins.
+    unsigned c[kPer], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      c[k] = m.hist[2047 - (tid * kPer + k)];
+      s += c[k];
+    }
+    unsigned inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) m.wsum[warp] = inc;
+    __syncthreads();
+    unsigned above = inc - s;
+    for (int w = 0; w < warp; ++w) above += m.wsum[w];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (above < need && above + c[k] >= need) {
+        m.digit = 2047 - (tid * kPer + k);
+        m.above = above;
+        m.count = c[k];
+      }
+      above += c[k];
+    }
+    __syncthreads();
+    lo += m.digit << shift;
+    need -= m.above;
+    *ties = m.count;
+    bins = 1u << min(shift, 11);
+    shift = max(0, shift - 11);
+    __syncthreads();
+  }
+  *rest = need;
+  return lo;
+}
+
+// Cut every unit longer than B + W back to B + W rows.  kByRank: units of at
+// most NT rows, one row a thread, kept by rank; otherwise the B-th best score
+// is selected over the unit's scores, which shared memory holds once
+// (`cached`; else they are read from global memory on every pass).
+template <typename T, int D, int NT, bool kByRank>
+__global__ void __launch_bounds__(NT)
+    evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow, int max_list,
+                 int cached) {
   pdl_begin();
-  __shared__ unsigned hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_need, s_base, s_count;
-  __shared__ int s_wsum[kWarps];
-  extern __shared__ int lists[];  // holes | movers, each max_list entries
+  extern __shared__ int lists[];  // holes | movers [max_list each] | scores
+  __shared__ unsigned s_wsum[NT / 32];
+  __shared__ int2 s_cnt[NT / 32];
 
   const Unit x = unit_of(c, lb, nl);
   const int tid = threadIdx.x;
@@ -221,70 +310,144 @@ __global__ void __launch_bounds__(kThreads)
   // The W most recent positions are protected; a row is a candidate iff its
   // position is at most newest - W.
   const int wlo = newest - W;
-
-  // TopB: by rank when every row has its own thread, else by a radix
-  // select of the B-th largest candidate key.
-  __shared__ unsigned long long s_key[kThreads];
-  __shared__ unsigned char s_keep[kThreads];
-  const bool by_rank = n <= kThreads;
-  unsigned long long thr = ~0ull;
-  if (by_rank)
+  const int nk = B + W;
+  int *holes = lists, *movers = lists + max_list;
+  auto finish = [&](auto keep) {
+    // The freed slots below nk and the survivors above, both in ascending
+    // order: each warp takes a contiguous run of rows, counts, and after one
+    // exchange of counts writes its part of the lists.
+    constexpr int kNW = NT / 32;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int seg = (n + kNW * 32 - 1) / (kNW * 32) * 32;
+    const int r0 = min(n, warp * seg), r1 = min(n, r0 + seg);
+    int ch = 0, cm = 0;
+    for (int base = r0; base < r1; base += 32) {
+      const int i = base + lane;
+      const bool in = i < r1, k = in && keep(i);
+      ch += __popc(__ballot_sync(0xffffffffu, in && i < nk && !k));
+      cm += __popc(__ballot_sync(0xffffffffu, in && i >= nk && k));
+    }
+    if (lane == 0) s_cnt[warp] = make_int2(ch, cm);
+    __syncthreads();
+    int oh = 0, om = 0, nh = 0, nm = 0;
+#pragma unroll
+    for (int w = 0; w < kNW; ++w) {
+      const int2 x = s_cnt[w];
+      if (w < warp) {
+        oh += x.x;
+        om += x.y;
+      }
+      nh += x.x;
+      nm += x.y;
+    }
+    // As many survivors above nk as free slots below: the window is intact
+    // and B + W rows stay.
+    if (nh != nm || nh > max_list) {
+      if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+      return;
+    }
+    const unsigned below = (1u << lane) - 1u;
+    for (int base = r0; base < r1; base += 32) {
+      const int i = base + lane;
+      const bool in = i < r1, k = in && keep(i);
+      const bool h = in && i < nk && !k, m = in && i >= nk && k;
+      const unsigned bh = __ballot_sync(0xffffffffu, h), bm = __ballot_sync(0xffffffffu, m);
+      if (h) holes[oh + __popc(bh & below)] = i;
+      if (m) movers[om + __popc(bm & below)] = i;
+      oh += __popc(bh);
+      om += __popc(bm);
+    }
+    __syncthreads();
+    // Move every survivor beyond nk into a freed slot below it (disjoint).
+    constexpr int kChunks = D * (int)sizeof(T) / 16;
+    for (int j = warp; j < nh; j += kNW) {
+      const int dst = holes[j], src = movers[j];
+      const int4 *ks = reinterpret_cast<const int4 *>(Ku + (size_t)src * D);
+      const int4 *vs = reinterpret_cast<const int4 *>(Vu + (size_t)src * D);
+      int4 *kd = reinterpret_cast<int4 *>(Ku + (size_t)dst * D);
+      int4 *vd = reinterpret_cast<int4 *>(Vu + (size_t)dst * D);
+      for (int q = lane; q < kChunks; q += 32) {
+        kd[q] = ks[q];
+        vd[q] = vs[q];
+      }
+      if (lane == 0) {
+        su[dst] = su[src];
+        pu[dst] = pu[src];
+      }
+    }
+    if (tid == 0) {
+      c.state[4 * x.u] = nk;
+      c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
+    }
+  };
+  if constexpr (kByRank) {
+    __shared__ unsigned long long s_key[NT];
+    __shared__ unsigned char s_keep[NT];
     block_rank_keep(
         n, B, [&](int i) { return pu[i] <= wlo; },
         [&](int i) { return rank_key(su[i], pu[i]); }, s_key, s_keep);
-  else if (B > 0)
-    thr = block_select(
-        n, B, [&](int i) { return pu[i] <= wlo; },
-        [&](int i) { return rank_key(su[i], pu[i]); }, hist, &s_prefix,
-        &s_need);
-  auto keep = [&](int i) {
-    if (by_rank) return s_keep[i] != 0;
-    const int32_t p = pu[i];
-    return p > wlo || (B > 0 && rank_key(su[i], p) >= thr);
-  };
-
-  // New length = number of kept rows (B + W whenever the window is intact).
-  if (tid == 0) s_count = 0;
-  __syncthreads();
-  int mine = 0;
-  for (int i = tid; i < n; i += kThreads) mine += keep(i) ? 1 : 0;
-  atomicAdd(&s_count, mine);
-  __syncthreads();
-  const int nk = s_count;
-  if (nk != B + W) {
-    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
-    return;
-  }
-  const int max_list = min(nk, n - nk);
-  int *holes = lists, *movers = lists + max_list;
-  const int nh = block_collect(0, nk, [&](int i) { return !keep(i); }, holes,
-                               s_wsum, &s_base);
-  const int nm = block_collect(nk, n, keep, movers, s_wsum, &s_base);
-  if (nh != nm) {
-    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
-    return;
-  }
-  // Move every survivor beyond nk into a freed slot below it (disjoint).
-  const int lane = tid & 31, warp = tid >> 5;
-  constexpr int kChunks = D * (int)sizeof(T) / 16;
-  for (int j = warp; j < nh; j += kWarps) {
-    const int dst = holes[j], src = movers[j];
-    const int4 *ks = reinterpret_cast<const int4 *>(Ku + (size_t)src * D);
-    const int4 *vs = reinterpret_cast<const int4 *>(Vu + (size_t)src * D);
-    int4 *kd = reinterpret_cast<int4 *>(Ku + (size_t)dst * D);
-    int4 *vd = reinterpret_cast<int4 *>(Vu + (size_t)dst * D);
-    for (int q = lane; q < kChunks; q += 32) {
-      kd[q] = ks[q];
-      vd[q] = vs[q];
+    finish([&](int i) { return s_keep[i] != 0; });
+  } else {
+    __shared__ SelectSmem m;
+    unsigned *sv = reinterpret_cast<unsigned *>(lists + 2 * max_list);
+    // A candidate's score bits (scores are >= 0: they order like the values),
+    // kNone for the window's rows.
+    auto bits = [&](int i) {
+      return pu[i] <= wlo ? min(__float_as_uint(su[i]), kNone - 1) : kNone;
+    };
+    int have = 0;
+    unsigned lo = kNone, hi = 0;
+    for (int i0 = tid; i0 < n; i0 += 4 * NT) {  // four rows' loads in flight
+      int32_t ps[4];
+      float sc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k * NT;
+        ps[k] = i < n ? pu[i] : INT32_MAX;
+        sc[k] = i < n ? su[i] : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k * NT;
+        const bool cand = i < n && ps[k] <= wlo;
+        const unsigned b = cand ? min(__float_as_uint(sc[k]), kNone - 1) : kNone;
+        if (cached && i < n) sv[i] = b;
+        lo = min(lo, b);
+        if (cand) hi = max(hi, b);
+        have += cand ? 1 : 0;
+      }
     }
-    if (lane == 0) {
-      su[dst] = su[src];
-      pu[dst] = pu[src];
+    have = __reduce_add_sync(0xffffffffu, have);
+    if ((tid & 31) == 0) s_wsum[tid >> 5] = have;
+    __syncthreads();
+    have = 0;
+    for (int w = 0; w < NT / 32; ++w) have += (int)s_wsum[w];
+    __syncthreads();
+    auto val = [&](int i) { return cached ? sv[i] : bits(i); };
+    unsigned thr = 0, last = 0;  // scores above thr stay; ties at positions up to ~last
+    if (B > 0 && have > B) {
+      unsigned rest, ties;
+      thr = select_desc<NT>(n, (unsigned)B, val, lo, hi, m, &rest, &ties);
+      if (rest < ties) {
+        // Equal scores: the lower positions stay.
+        unsigned r2, t2;
+        auto low_pos = [&](int i) { return val(i) == thr ? ~(unsigned)pu[i] - 1u : kNone; };
+        lo = kNone;
+        hi = 0;
+        for (int i = tid; i < n; i += NT) {
+          const unsigned b = low_pos(i);
+          lo = min(lo, b);
+          if (b != kNone) hi = max(hi, b);
+        }
+        last = select_desc<NT>(n, rest, low_pos, lo, hi, m, &r2, &t2);
+      }
     }
-  }
-  if (tid == 0) {
-    c.state[4 * x.u] = nk;
-    c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
+    finish([&](int i) {
+      const unsigned b = val(i);
+      if (b == kNone) return true;
+      if (B == 0) return false;
+      return b > thr || (b == thr && ~(unsigned)pu[i] - 1u >= last);
+    });
   }
 }
 
@@ -350,18 +513,34 @@ cudaError_t attend_ext_dispatch(const CacheView &c, const StepArgs &a,
                     a, 0, ext);
 }
 
-template <typename T, int D>
-cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
-                           int B, int W, int grow, cudaStream_t st) {
+// Rows a CTA of the radix select keeps in shared memory, and the rows from
+// which a unit takes 1,024 threads instead of 256 (few units, long scans).
+constexpr int kCachedRows = 49152, kWideRows = 2048;
+
+template <typename T, int D, int NT, bool kByRank>
+cudaError_t evict_launch(const CacheView &c, int lb, int nl, int max_rows, int B, int W,
+                         int grow, cudaStream_t st) {
   const int nk = B + W;
   const int max_list = max(1, min(nk, max_rows - nk));
-  const size_t bytes = 2 * (size_t)max_list * sizeof(int);
-  auto kern = evict_kernel<T, D>;
+  const int cached = !kByRank && max_rows <= kCachedRows &&
+                     (2 * (size_t)max_list + max_rows) * sizeof(int) <= 200 * 1024;
+  const size_t bytes = (2 * (size_t)max_list + (cached ? max_rows : 0)) * sizeof(int);
+  auto kern = evict_kernel<T, D, NT, kByRank>;
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(kThreads), bytes, st, c,
-                    lb, nl, B, W, grow);
+  return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(NT), bytes, st, c, lb, nl, B, W, grow,
+                    max_list, cached);
+}
+
+template <typename T, int D>
+cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
+                           int B, int W, int grow, cudaStream_t st) {
+  if (max_rows <= kThreads)
+    return evict_launch<T, D, kThreads, true>(c, lb, nl, max_rows, B, W, grow, st);
+  if (max_rows <= kWideRows)
+    return evict_launch<T, D, kThreads, false>(c, lb, nl, max_rows, B, W, grow, st);
+  return evict_launch<T, D, 1024, false>(c, lb, nl, max_rows, B, W, grow, st);
 }
 
 }  // namespace

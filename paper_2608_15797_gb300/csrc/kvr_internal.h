@@ -193,6 +193,19 @@ cudaError_t launch_split_attend(const CUtensorMap &tmK, const CUtensorMap &tmV,
                                 const SplitParams &p, void *out,
                                 cudaStream_t st);
 
+// A decode step with scores and no eviction over units of any length
+// (kvr_split.cu): bf16, d = 128, G <= 8; takes p without ws and n_splits, and
+// the maps of split_rows_per_stage()-row boxes.  order: the sequences, longest
+// first (read for caches of at most kMaxOrder sequences); max_rows: the
+// longest unit's rows.
+constexpr int kMaxOrder = 128;
+struct SeqOrder {
+  uint16_t seq[kMaxOrder];
+};
+cudaError_t launch_long_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
+                             const SplitParams &p, const SeqOrder &order,
+                             int max_rows, void *out, cudaStream_t st);
+
 // Candidates of one cache (kvr_fork.cu).  A candidate unit cu = c * units + u.
 struct ForkView {
   CacheView p;       // the parent: its live rows are every candidate's prefix
@@ -329,12 +342,17 @@ struct ChunkParams {
   int n_groups, n_stages;      // consumer groups; ring stages per group
   int budget, window, evict;
   float scale_log2e, inv_g;
+  // R-KV eviction (App. C) instead of the accumulated-attention TopB, plain
+  // units only; two launches, the first of which sums the keys of units that
+  // have no current sum.
+  int rkv;
+  float lam;
 };
 int chunk_box_rows();
 int chunk_max_rows();
 int chunk_max_groups();
 int chunk_max_stages();
-size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages);
+size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, bool rkv = false);
 cudaError_t launch_chunk_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                               const CUtensorMap *tmTK, const CUtensorMap *tmTV,
                               const ChunkParams &p, int grid, cudaStream_t st);
