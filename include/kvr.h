@@ -151,7 +151,10 @@ kvr_status kvr_decode_step(kvr_cache *cache, int layer_begin, int layer_end,
  * reading of R-KV.  Where every unit holds at most 160 rows after the
  * append and at most one is evicted (bf16, head_dim 128, G <= 8) it is one
  * launch: the redundancy of each row comes from the keys already staged
- * for attention, so no key is read twice; otherwise it runs the two calls.
+ * for attention, so no key is read twice.  Up to 1,024 rows it is the same in
+ * two launches, the first of which sums the keys of units that hold no
+ * current sum (kvr_cache_scores, state word 2) and is empty otherwise.  Any
+ * other call runs the two calls.
  * Arguments as kvr_decode_step, plus 0 <= lambda <= 1 (KVR_EINVAL
  * otherwise). */
 kvr_status kvr_decode_step_rkv(kvr_cache *cache, int layer_begin,

@@ -30,6 +30,15 @@
 //    states and partial outputs, compute every row's exact probability from
 //    the kept logits for the score update, agree on the evicted row, and
 //    write back.
+//  - R-KV (kRkv; plain units): the row's redundancy comes from the K tile
+//    that the QK product has in registers: its dot with the unit's kept sum
+//    of normalised keys S (a B operand of three bf16 terms) and its squared
+//    norm (the diagonal of the tile's Gram block), so that no key is read
+//    twice.  One more exchange of sums at the end of a job gives z.  Units
+//    with no current S get one from rkv_sum_kernel, launched before.  7B, 16
+//    sequences, 641-row units: 148 us against 113 for the plain step; the
+//    separate eviction pass it replaces (two readings of the keys, a radix
+//    select) took 337 us after the 113.
 //  - Launched with programmatic stream serialization; every mbarrier wait is
 //    bounded (about 2 s) and on timeout sets ERR_TIMEOUT and drains its own
 //    copies.
@@ -38,6 +47,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "kvr_device.cuh"
 #include "kvr_internal.h"
 #include "kvr_ptx.cuh"
 
@@ -45,6 +55,7 @@ namespace kvr {
 namespace {
 
 using namespace ptx;
+using dev::rkv_key;
 
 // Packed fp32 pairs (round to nearest, no flush).
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
@@ -91,21 +102,26 @@ struct ChunkStage {
                             v1 = 3 * kCR * 128, q = 4 * kCR * 128,
                             kn = q + 8 * kQPitch, vn = kn + 256, sc = vn + 256,
                             ps = sc + 4 * kCR, hdr = ps + 4 * kCR,
-                            bytes = ((hdr + 4 * H_WORDS) + 1023) / 1024 * 1024;
+                            bytes = ((hdr + 4 * H_WORDS) + 1023) / 1024 * 1024,
+                            // R-KV stages: the unit's kept key sum follows
+                            rs = bytes, rkv_bytes = bytes + 1024;
 };
+__host__ __device__ constexpr uint32_t stage_bytes(bool rkv) {
+  return rkv ? ChunkStage::rkv_bytes : ChunkStage::bytes;
+}
 
 // Byte offsets inside one group's area (after the rings).
 struct ChunkGroup {
   uint32_t xs, ox, lg, sc, ps, ns, bytes;
   __host__ __device__ explicit ChunkGroup(int n_max) {
     const int n = round_up16(n_max);
-    xs = 0;                      // [kU][5] 16-byte slots
+    xs = 0;                      // [kU][5] 16-byte slots; R-KV: [kU] more
     ox = 256;                    // [kU][4][32] float4 partial outputs: the
                                  // 4 head-dim tiles the other warp owns
     lg = ox + kU * 4 * 32 * 16;  // [n][8] scaled logits
     sc = lg + n * 8 * 4;         // [n] old scores
     ps = sc + n * 4;             // [n] positions
-    ns = ps + n * 4;             // [n] new scores
+    ns = ps + n * 4;             // [n] new scores (R-KV: mean cosines)
     bytes = ((ns + n * 4) + 127) / 128 * 128;
   }
 };
@@ -127,12 +143,38 @@ __device__ __forceinline__ Job job_of(const ChunkParams &p, int idx) {
   return j;
 }
 
+// Elements 4 lane .. 4 lane + 3 of a bf16 row.
+__device__ __forceinline__ void key4(const unsigned char *row, int lane, float (&v)[4]) {
+  const uint2 x = reinterpret_cast<const uint2 *>(row)[lane];
+  v[0] = __uint_as_float(x.x << 16);
+  v[1] = __uint_as_float(x.x & 0xFFFF0000u);
+  v[2] = __uint_as_float(x.y << 16);
+  v[3] = __uint_as_float(x.y & 0xFFFF0000u);
+}
+// 1 / |k| of the row that the warp holds four elements a lane (0 for a zero
+// row): the arithmetic by which a key enters the kept sum and leaves it.
+__device__ __forceinline__ float inv_norm(const float (&v)[4]) {
+  float ss = fmaf(v[0], v[0], fmaf(v[1], v[1], fmaf(v[2], v[2], v[3] * v[3])));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  return ss > 0.f ? rsqrtf(ss) : 0.f;
+}
+// Term `t` (0-2; 0 beyond) of a pair split into three bf16 terms.
+__device__ __forceinline__ uint32_t s_term(float2 v, int t) {
+  const uint32_t h = pack_bf16(v.x, v.y);
+  const float rx = v.x - __uint_as_float(h << 16), ry = v.y - __uint_as_float(h & 0xFFFF0000u);
+  const uint32_t m = pack_bf16(rx, ry);
+  const uint32_t l = pack_bf16(rx - __uint_as_float(m << 16),
+                               ry - __uint_as_float(m & 0xFFFF0000u));
+  return t == 0 ? h : t == 1 ? m : t == 2 ? l : 0u;
+}
+
 __device__ __forceinline__ void group_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // Producer warp of one group: every chunk of the group's jobs, in order.
-template <bool kFork>
+template <bool kFork, bool kRkv>
 __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
                         const CUtensorMap *tmV, const CUtensorMap *tmTK,
                         const CUtensorMap *tmTV, unsigned char *ring,
@@ -177,7 +219,7 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
         return;
       }
       __syncwarp();
-      unsigned char *st = ring + s * ChunkStage::bytes;
+      unsigned char *st = ring + s * stage_bytes(kRkv);
       const uint32_t s0 = smem_u32(st);
       const uint32_t bar = smem_u32(&full[s]);
       const bool segA = ci < cA;
@@ -220,7 +262,10 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
             cp_async16(s0 + ChunkStage::q + (i >> 4) * kQPitch + (i & 15) * 16,
                        q + i * 16);
         }
-        if (has_new)
+        if (kRkv && ci == 0)  // the kept sum of the live rows' normalised keys
+          cp_async16(s0 + ChunkStage::rs + lane * 16,
+                     c.rsum + jb.ug * 128 + lane * 4);
+        if (has_new || (kRkv && ci == 0))
           cp_async16(s0 + (lane < 16 ? ChunkStage::kn : ChunkStage::vn) +
                          (lane & 15) * 16,
                      reinterpret_cast<const unsigned char *>(
@@ -250,7 +295,44 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
   }
 }
 
-template <bool kFork, bool kOutBf16>
+// R-KV: the sum of a unit's normalised keys, where the unit has none that is
+// current (state word 2); one CTA a unit, a warp a row.  In the steady state
+// every unit has one and this is the launch of an empty kernel.
+__global__ void __launch_bounds__(128) rkv_sum_kernel(CacheView c, int lb, int nl) {
+  pdl_begin();
+  __shared__ float4 s_S[4][32];
+  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int h = b % c.H, lr = (b / c.H) % nl, sq = b / (c.H * nl);
+  const size_t u = ((size_t)sq * c.L + lb + lr) * c.H + h;
+  const int n = c.state[4 * u];
+  if (c.state[4 * u + 2] == 1 || n < 0 || n > c.cap) return;
+  const unsigned char *K = reinterpret_cast<const unsigned char *>(c.K) + u * (size_t)c.cap * 256;
+  float S[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int i = warp; i < n; i += 4) {
+    float k[4];
+    key4(K + (size_t)i * 256, lane, k);
+    const float inv = inv_norm(k);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) S[x] = fmaf(k[x], inv, S[x]);
+  }
+  s_S[warp][lane] = make_float4(S[0], S[1], S[2], S[3]);
+  __syncthreads();
+  if (warp == 0) {
+    float4 t = s_S[0][lane];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) {
+      t.x += s_S[w][lane].x;
+      t.y += s_S[w][lane].y;
+      t.z += s_S[w][lane].z;
+      t.w += s_S[w][lane].w;
+    }
+    reinterpret_cast<float4 *>(c.rsum + u * 128)[lane] = t;
+    if (lane == 0) c.state[4 * u + 2] = 1;
+  }
+}
+
+template <bool kFork, bool kOutBf16, bool kRkv>
 __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
     chunk_step_kernel(const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV,
@@ -274,7 +356,9 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
                        : 0;
   const int consumers = p.n_groups * kU;
   const ChunkGroup GL(p.n_max);
-  const uint32_t ring_bytes = p.n_stages * ChunkStage::bytes;
+  static_assert(!(kFork && kRkv), "candidates evict at the commit");
+  constexpr uint32_t kStage = stage_bytes(kRkv);
+  const uint32_t ring_bytes = p.n_stages * kStage;
 
   if (threadIdx.x == 0) {
     prefetch_tmap(&tmK);
@@ -300,7 +384,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
     const int st = i / (8 * (kQPitch / 16)), r = i % (8 * (kQPitch / 16));
     const int g = st / p.n_stages, s = st % p.n_stages;
     if (r >= G * (kQPitch / 16))
-      reinterpret_cast<int4 *>(smem + g * ring_bytes + s * ChunkStage::bytes +
+      reinterpret_cast<int4 *>(smem + g * ring_bytes + s * kStage +
                                ChunkStage::q)[r] = make_int4(0, 0, 0, 0);
   }
   fence_proxy_async();
@@ -310,7 +394,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   if (warp >= consumers) {
     const int g = warp - consumers;
     if (g < p.n_groups)
-      produce<kFork>(p, &tmK, &tmV, &tmTK, &tmTV, smem + g * ring_bytes,
+      produce<kFork, kRkv>(p, &tmK, &tmV, &tmTK, &tmTV, smem + g * ring_bytes,
                      full_bar[g], empty_bar[g], g, mine, lane, &s_abort,
                      &issued_n[g]);
   } else {
@@ -333,6 +417,10 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
 #pragma unroll
       for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
       uint32_t qb[8][2];
+      // R-KV: the key sum S with the new key, elements 4 lane .. 4 lane + 3, and
+      // S as the B operand of K S (columns 0-2: three bf16 terms, exact).
+      float S4[4] = {0.f, 0.f, 0.f, 0.f}, inv_n1 = 0.f;
+      uint32_t sq[8][2];
       int idx = 0, t = 0, ntot = 0, nA = 0;
       int4 nrow = make_int4(0, 0, 0, 0);  // warp 0: the new k (lanes 0-15) / v row
       bool skip = false;
@@ -356,7 +444,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           break;
         }
         mbar_try_wait(smem_u32(&full_bar[g][s]), ph);  // acquire for this thread
-        unsigned char *st = ring + s * ChunkStage::bytes;
+        unsigned char *st = ring + s * kStage;
         const int *h = reinterpret_cast<const int *>(st + ChunkStage::hdr);
         const int flags = h[H_FLAGS], base = h[H_BASE], valid = h[H_VALID];
         const int loaded = h[H_LOADED];
@@ -373,6 +461,31 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
                     qb[2 * i + 1][1]);
         }
         skip = (flags & F_SKIP) != 0;
+        if constexpr (kRkv) {
+          if ((flags & F_FIRST) && !skip) {
+            const float4 rs = reinterpret_cast<const float4 *>(st + ChunkStage::rs)[lane];
+            float kn[4];
+            key4(st + ChunkStage::kn, lane, kn);
+            const float inv = inv_norm(kn);
+            S4[0] = fmaf(kn[0], inv, rs.x);
+            S4[1] = fmaf(kn[1], inv, rs.y);
+            S4[2] = fmaf(kn[2], inv, rs.z);
+            S4[3] = fmaf(kn[3], inv, rs.w);
+            inv_n1 = ntot > 1 ? 1.f / (float)(ntot - 1) : 0.f;
+            // Through this warp's part of the (now idle) output exchange.
+            float *sx = reinterpret_cast<float *>(OX + w * 4 * 32);
+            reinterpret_cast<float4 *>(sx)[lane] = make_float4(S4[0], S4[1], S4[2], S4[3]);
+            __syncwarp();
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh) {
+                const float2 v = *reinterpret_cast<const float2 *>(sx + 16 * ks + 8 * hh + c2);
+                sq[ks][hh] = s_term(v, lane >> 2);
+              }
+            __syncwarp();
+          }
+        }
         unsigned char *K0 = st + ChunkStage::k0, *K1 = st + ChunkStage::k1;
         unsigned char *V0 = st + ChunkStage::v0, *V1 = st + ChunkStage::v1;
         const int tr0 = kBox * w;
@@ -410,6 +523,8 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           }
           __syncwarp();
           float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+          float sd[4] = {0.f, 0.f, 0.f, 0.f}, g0[4] = {0.f, 0.f, 0.f, 0.f},
+                g1[4] = {0.f, 0.f, 0.f, 0.f};
           {
             const int row = tr0 + (lane & 7) + ((lane >> 3) & 1) * 8;
             const uint32_t b0 = smem_u32(K0) + row * 128, b1 = smem_u32(K1) + row * 128;
@@ -421,6 +536,14 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
               ldsm_x4(addr, a0, a1, a2, a3);
               if (ks & 1) mma_bf16(sb, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
               else mma_bf16(sa, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+              if constexpr (kRkv) {
+                // K S, and the Gram blocks of the tile's two row halves,
+                // whose diagonals are the squared norms (a K tile is the
+                // row-major B operand as it stands).
+                mma_bf16(sd, a0, a1, a2, a3, sq[ks][0], sq[ks][1]);
+                mma_bf16(g0, a0, a1, a2, a3, a0, a2);
+                mma_bf16(g1, a0, a1, a2, a3, a1, a3);
+              }
             }
           }
           const int ra = tr0 + r0l, rb = ra + 8;  // stage rows
@@ -435,6 +558,23 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           if (rb < valid)
             *reinterpret_cast<float2 *>(LG + (base + rb) * 8 + c2) =
                 make_float2(s4[2], s4[3]);
+          if constexpr (kRkv) {
+            // Mean cosine of rows ra and rb with the other live rows.
+            float da = sd[0] + sd[1], db = sd[2] + sd[3];
+            da += __shfl_xor_sync(0xffffffffu, da, 1);
+            db += __shfl_xor_sync(0xffffffffu, db, 1);
+            const int own = (lane & ~3) | (r0l >> 1);  // holds the diagonals
+            const float na =
+                __shfl_sync(0xffffffffu, (r0l & 1) ? g0[1] : g0[0], own);
+            const float nb =
+                __shfl_sync(0xffffffffu, (r0l & 1) ? g1[3] : g1[2], own);
+            if ((lane & 3) == 0) {
+              if (ra < valid)
+                GNS[base + ra] = na > 0.f ? (da * rsqrtf(na) - 1.f) * inv_n1 : 0.f;
+              if (rb < valid)
+                GNS[base + rb] = nb > 0.f ? (db * rsqrtf(nb) - 1.f) * inv_n1 : 0.f;
+            }
+          }
           float x0 = fmaxf(s4[0], s4[2]), x1 = fmaxf(s4[1], s4[3]);
 #pragma unroll
           for (int off = 4; off < 32; off <<= 1) {
@@ -594,6 +734,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
       const bool evict = !kFork && p.evict && ntot > p.budget + p.window;
       unsigned long long best = ~0ull;
       int bi = -1;
+      float ssum = 0.f, esum = 0.f;
       for (int r = tid; r < ntot; r += 32 * kU) {
         const float4 la = *reinterpret_cast<const float4 *>(LG + r * 8);
         const float4 lb = *reinterpret_cast<const float4 *>(LG + r * 8 + 4);
@@ -603,8 +744,18 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
         for (int gg = 0; gg < 8; ++gg)
           if (gg < G) acc += ex2(lg8[gg] - Mh[gg]) * iZ[gg];
         const float sc = GSC[r] + acc * p.inv_g;
-        GNS[r] = sc;
-        if (evict) {
+        if constexpr (kRkv) {
+          GSC[r] = sc;
+          // The candidates' sums: of the scores, and of exp(mean cosine) (a
+          // cosine needs no maximum taken off).
+          if (evict && GPS[r] <= wlo) {
+            ssum += sc;
+            esum += expf(GNS[r]);
+          }
+        } else {
+          GNS[r] = sc;
+        }
+        if (evict && !kRkv) {
           const int pr = GPS[r];
           if (pr <= wlo) {
             const unsigned long long key =
@@ -613,6 +764,32 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
             if (key < best) {
               best = key;
               bi = r;
+            }
+          }
+        }
+      }
+      if constexpr (kRkv) {
+        if (evict) {
+#pragma unroll
+          for (int o2 = 16; o2 > 0; o2 >>= 1) {
+            ssum += __shfl_xor_sync(0xffffffffu, ssum, o2);
+            esum += __shfl_xor_sync(0xffffffffu, esum, o2);
+          }
+          if (lane == 0) XS4[kU * 5 + w] = make_float4(ssum, esum, 0.f, 0.f);
+          group_bar(bar_id, 32 * kU);
+          const float4 x0 = XS4[kU * 5], x1 = XS4[kU * 5 + 1];
+          const float ss = x0.x + x1.x;
+          const float ci = ss > 0.f ? p.lam / ss : 0.f;
+          const float cr = (1.f - p.lam) / (x0.y + x1.y);
+          for (int r = tid; r < ntot; r += 32 * kU) {
+            const int pr = GPS[r];
+            if (pr <= wlo) {
+              const unsigned long long key =
+                  rkv_key(GSC[r] * ci - cr * expf(GNS[r]), pr);
+              if (key < best) {
+                best = key;
+                bi = r;
+              }
             }
           }
         }
@@ -669,9 +846,34 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
       } else {
         const int m = ntot - 1;  // live rows before the append
         float *gsc = c.score + jb.ug * c.sstride;
+        const float *NS = kRkv ? GSC : GNS;  // the new scores
+        uint2 vk = make_uint2(0u, 0u);  // the victim's key, before its slot is written
+        if (kRkv && w == 0 && victim >= 0 && victim < m)
+          vk = reinterpret_cast<const uint2 *>(
+              reinterpret_cast<const __nv_bfloat16 *>(c.K) +
+              (jb.ug * (size_t)c.cap + victim) * 128)[lane];
         for (int r = tid; r < m; r += 32 * kU)
-          gsc[r] = r == victim ? GNS[m] : GNS[r];
+          gsc[r] = r == victim ? NS[m] : NS[r];
         const int slot = victim < 0 ? m : (victim < m ? victim : -1);
+        if (kRkv && w == 0) {
+          // The sum of the rows that stay, for the next step.
+          if (victim == m) {  // the new row itself: lanes 0-15 hold its key
+            const int src = lane >> 1;
+            const int x = __shfl_sync(0xffffffffu, nrow.x, src);
+            const int y = __shfl_sync(0xffffffffu, nrow.y, src);
+            const int z = __shfl_sync(0xffffffffu, nrow.z, src);
+            const int u = __shfl_sync(0xffffffffu, nrow.w, src);
+            vk = (lane & 1) ? make_uint2((uint32_t)z, (uint32_t)u)
+                            : make_uint2((uint32_t)x, (uint32_t)y);
+          }
+          float kv[4];
+          key4(reinterpret_cast<const unsigned char *>(&vk), 0, kv);
+          const float inv = inv_norm(kv);
+          reinterpret_cast<float4 *>(c.rsum + jb.ug * 128)[lane] =
+              make_float4(fmaf(kv[0], -inv, S4[0]), fmaf(kv[1], -inv, S4[1]),
+                          fmaf(kv[2], -inv, S4[2]), fmaf(kv[3], -inv, S4[3]));
+          __syncwarp();  // the victim's key has been read
+        }
         if (w == 0) {
           if (slot >= 0) {
             __nv_bfloat16 *dst =
@@ -680,13 +882,13 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
             reinterpret_cast<int4 *>(dst)[lane & 15] = nrow;
             if (lane == 0) {
               c.pos[jb.ug * c.sstride + slot] = t;
-              if (slot == m) gsc[m] = GNS[m];
+              if (slot == m) gsc[m] = NS[m];
             }
           }
           if (lane == 0) {
             c.state[4 * jb.ug] = victim < 0 ? m + 1 : m;
             c.state[4 * jb.ug + 1] = t + 1;
-            c.state[4 * jb.ug + 2] = 0;  // R-KV key sum no longer valid
+            c.state[4 * jb.ug + 2] = kRkv ? 1 : 0;  // the kept R-KV key sum
           }
         }
       }
@@ -704,13 +906,13 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   }
 }
 
-template <bool kFork>
+template <bool kFork, bool kRkv>
 cudaError_t launch_k(const CUtensorMap &tmK, const CUtensorMap &tmV,
                      const CUtensorMap &tmTK, const CUtensorMap &tmTV,
                      const ChunkParams &p, int grid, size_t smem,
                      cudaStream_t st) {
-  auto kern = p.c.out_bf16 ? chunk_step_kernel<kFork, true>
-                           : chunk_step_kernel<kFork, false>;
+  auto kern = p.c.out_bf16 ? chunk_step_kernel<kFork, true, kRkv>
+                           : chunk_step_kernel<kFork, false, kRkv>;
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -724,9 +926,9 @@ int chunk_box_rows() { return kBox; }
 int chunk_max_rows() { return kMaxRowsChunk; }
 int chunk_max_groups() { return kMaxGroups; }
 int chunk_max_stages() { return kMaxStages; }
-size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages) {
+size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, bool rkv) {
   return (size_t)n_groups *
-             ((size_t)n_stages * ChunkStage::bytes + ChunkGroup(n_max).bytes) +
+             ((size_t)n_stages * stage_bytes(rkv) + ChunkGroup(n_max).bytes) +
          1024;
 }
 
@@ -736,12 +938,20 @@ cudaError_t launch_chunk_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                               cudaStream_t st) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.n_stages < 2 ||
       p.n_stages > kMaxStages || p.n_max < 1 || p.n_max > kMaxRowsChunk ||
-      p.c.G > 8 || (p.fork && (!tmTK || !tmTV)))
+      p.c.G > 8 || (p.fork && (!tmTK || !tmTV || p.rkv)))
     return cudaErrorInvalidValue;
-  const size_t smem = chunk_smem_bytes(p.n_max, p.n_groups, p.n_stages);
+  const size_t smem = chunk_smem_bytes(p.n_max, p.n_groups, p.n_stages, p.rkv != 0);
   if (p.fork)
-    return launch_k<true>(tmK, tmV, *tmTK, *tmTV, p, grid, smem, st);
-  return launch_k<false>(tmK, tmV, tmK, tmV, p, grid, smem, st);
+    return launch_k<true, false>(tmK, tmV, *tmTK, *tmTV, p, grid, smem, st);
+  if (p.rkv) {
+    // Units whose kept key sum another call has left stale, first.
+    const int units = p.c.S * p.nl * p.c.H;
+    const cudaError_t e =
+        launch_pdl(rkv_sum_kernel, dim3(units), dim3(128), 0, st, p.c, p.lb, p.nl);
+    if (e != cudaSuccess) return e;
+    return launch_k<false, true>(tmK, tmV, tmK, tmV, p, grid, smem, st);
+  }
+  return launch_k<false, false>(tmK, tmV, tmK, tmV, p, grid, smem, st);
 }
 
 }  // namespace kvr
