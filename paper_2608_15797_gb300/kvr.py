@@ -101,26 +101,36 @@ def _check(status: int, where: str):
         raise KvrError(status, where, kvr_last_error())
 
 
+# A call's marshalling is most of what a small step costs on the host (one
+# sequence, one call a layer, 28 calls: 304 us a token with c_void_p objects
+# and torch.cuda.current_stream(), 184 without), so pointers go to ctypes as plain integers and
+# the current stream is read without building a torch.cuda.Stream.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _ptr(t):
-    if t is None:
-        return None
     if isinstance(t, torch.Tensor):
         if not t.is_contiguous():
             raise ValueError("tensors passed to libkvr must be contiguous")
-        return ctypes.c_void_p(t.data_ptr())
+        return t.data_ptr()
+    if t is None:
+        return None
     if isinstance(t, np.ndarray):
         if not t.flags["C_CONTIGUOUS"]:
             raise ValueError("arrays passed to libkvr must be C-contiguous")
         return t.ctypes.data_as(ctypes.c_void_p)
-    return ctypes.c_void_p(int(t))
+    return int(t)
 
 
 def make_desc(n_seq, n_layers, n_kv_heads, group, head_dim, capacity,
