@@ -466,8 +466,9 @@ void kvr_entropy_destroy(kvr_entropy *det);
  * v_new and out; other calls run in blocks on the tensor cores where the
  * outputs are bf16, else token by token).  Results agree within rounding:
  * 0 = 5th-generation tensor cores with the logits, probabilities and outputs
- * in tensor memory, for units of at most 144 rows after the chunk (larger
- * ones run kernel 1; the default), 1 = mma.sync with register accumulators. */
+ * in tensor memory, for units of at most 144 rows after the chunk (the
+ * default; larger ones run in blocks where the outputs are bf16 and that is
+ * the faster, else kernel 1), 1 = mma.sync with register accumulators. */
 kvr_status kvr_cache_set_absorb_kernel(kvr_cache *cache, int kernel);
 
 /* How the cache's last kvr_absorb_chunk ran: 0 = the tensor-memory kernel,

@@ -904,6 +904,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 int absorb_max_chunk() { return kMaxChunk; }
 int absorb_max_rows() { return kMaxRows; }
+int absorb_tc_max_rows() { return kTcMaxRows; }
 
 cudaError_t launch_absorb(const AbsorbParams &p, int kernel, const CUtensorMap *tmQ,
                           cudaStream_t st, int *ran) {

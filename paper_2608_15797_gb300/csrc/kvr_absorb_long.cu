@@ -8,7 +8,7 @@
 // The work is a contraction: C tokens x G heads against m + C rows, causal.
 // Run token by token it was one launch a token, each reading every row again
 // (7B, two 1,000-token prompts: 140 ms; 16 sequences absorbing 57 tokens into
-// 640 rows: 39.8 ms).  Here it is four launches (0.95 ms and 0.81 ms):
+// 640 rows: 39.8 ms).  Here it is four launches (0.91 ms and 0.75 ms):
 //   1. append: the chunk's rows go to slots m.. of each unit, score 0.
 //   2. attend (tcgen05): tiles of 128 query rows (128 / G whole tokens) over
 //      128-row key blocks with an online softmax; writes the outputs and each
@@ -47,8 +47,15 @@ static_assert(kAttSmem + 2048 <= 113 * 1024, "two CTAs an SM, with the static va
 constexpr int kScThr = 576, kScCols = 512;
 constexpr int kProducer = 16, kIssuer = 17;
 constexpr int kQRing = 3;            // query tiles in flight
-constexpr int kScoreSmem = (4 + kQRing) * kTile + kQRing * 512 + 1024;
-static_assert(kScoreSmem + 512 <= 227 * 1024, "with the static variables");
+constexpr int kLRing = 4;            // their rows' normalisers
+struct ScoreBars {
+  uint64_t kfull[2], kfree[2], qfull[kQRing], qfree[kQRing], lfull[kLRing], lfree[kLRing],
+      s[2][2], sfree[2][2], drain;
+  uint32_t tmem;
+  int abort;
+};
+constexpr int kScoreSmem = (4 + kQRing) * kTile + kLRing * 512 + (int)sizeof(ScoreBars);
+static_assert(kScoreSmem <= 227 * 1024, "one CTA an SM");
 // Lazy rescaling: the reference of a row's exponentials moves only when a
 // logit exceeds it by 2^kLazy; sums stay far inside fp32's range.
 constexpr float kLazy = 8.f;
@@ -441,13 +448,22 @@ __global__ void __launch_bounds__(kAttThr, 2)
           }
         };
         float mx = -INFINITY;
+        if (ok && lim_w >= 64) {  // every column is seen: both loads in flight
+          float e0[32], e1[32];
+          tmem_ld32(tS, e0);
+          tmem_ld32(tS + 32, e1);
+          tmem_wait_ld();
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (ok && 32 * k < ncol) {
-            float e[32];
-            load_s(k, e);
+          for (int x = 0; x < 32; ++x) mx = fmaxf(mx, fmaxf(e0[x], e1[x]));
+        } else {
 #pragma unroll
-            for (int x = 0; x < 32; x += 2) mx = fmaxf(mx, fmaxf(e[x], e[x + 1]));
+          for (int k = 0; k < 2; ++k) {
+            if (ok && 32 * k < ncol) {
+              float e[32];
+              load_s(k, e);
+#pragma unroll
+              for (int x = 0; x < 32; x += 2) mx = fmaxf(mx, fmaxf(e[x], e[x + 1]));
+            }
           }
         }
         mx *= scale;
@@ -592,38 +608,40 @@ __global__ void __launch_bounds__(kScThr, 1)
     long_score_kernel(const AbsorbParams p, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmQ, const float *lse, int n_items,
                       int n_qt) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_abort;
-  __shared__ __align__(8) uint64_t b_kfull[2], b_kfree[2], b_qfull[kQRing], b_qfree[kQRing],
-      b_s[2][2], b_sfree[2][2], b_drain;
-  unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+  // (No static shared memory: the tiles need 1,024-byte alignment and all the
+  // rest of the SM's shared memory.)
+  extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t aK = smem_u32(smem), aQ = aK + 4 * kTile;
-  float *s_lse = reinterpret_cast<float *>(smem + (4 + kQRing) * kTile);  // [kQRing][128]
+  float *s_lse = reinterpret_cast<float *>(smem + (4 + kQRing) * kTile);  // [kLRing][128]
+  ScoreBars &B = *reinterpret_cast<ScoreBars *>(s_lse + kLRing * kBlk);
   const CacheView &c = p.c;
   const int G = c.G, Jt = kBlk / G;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  volatile int *abort = &s_abort;
-  // A whole warp's bounded wait; its lanes agree on the result.
-  auto wait_warp = [&](uint32_t bar, uint32_t parity) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) != 0;
+  volatile int *abort = &B.abort;
+  // A whole warp's bounded wait for completion n of a barrier.
+  auto wait_warp = [&](uint64_t &bar, int n) {
+    return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), (uint32_t)(n & 1), abort)) != 0;
   };
-  if (warp == kProducer) tmem_alloc(smem_u32(&s_tmem), kScCols);
+  if (warp == kProducer) tmem_alloc(smem_u32(&B.tmem), kScCols);
   if (tid == 0) {
     for (int t = 0; t < 2; ++t) {
-      mbar_init(smem_u32(&b_kfull[t]), 1);
-      mbar_init(smem_u32(&b_kfree[t]), 1);
+      mbar_init(smem_u32(&B.kfull[t]), 1);
+      mbar_init(smem_u32(&B.kfree[t]), 1);
       for (int b = 0; b < 2; ++b) {
-        mbar_init(smem_u32(&b_s[t][b]), 1);
-        mbar_init(smem_u32(&b_sfree[t][b]), 4);
+        mbar_init(smem_u32(&B.s[t][b]), 1);
+        mbar_init(smem_u32(&B.sfree[t][b]), 4);
       }
     }
     for (int s = 0; s < kQRing; ++s) {
-      mbar_init(smem_u32(&b_qfull[s]), 1 + 32);  // the TMA issue; the lanes' normalisers
-      mbar_init(smem_u32(&b_qfree[s]), 1 + 8);   // the contractions; the softmax warps
+      mbar_init(smem_u32(&B.qfull[s]), 1);
+      mbar_init(smem_u32(&B.qfree[s]), 1);
     }
-    mbar_init(smem_u32(&b_drain), 1);
-    s_abort = 0;
+    for (int s = 0; s < kLRing; ++s) {
+      mbar_init(smem_u32(&B.lfull[s]), 32);
+      mbar_init(smem_u32(&B.lfree[s]), 8);
+    }
+    mbar_init(smem_u32(&B.drain), 1);
+    B.abort = 0;
     fence_mbar_init();
   }
   for (int i = tid; i < kQRing * 2 * (kBlk - Jt * G) * 8; i += kScThr) {
@@ -636,7 +654,7 @@ __global__ void __launch_bounds__(kScThr, 1)
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const uint32_t tm = s_tmem;
+  const uint32_t tm = B.tmem;
 
   if (warp == kProducer) {
     // Producer: key tiles (two pairs in flight), query tiles and their
@@ -652,11 +670,11 @@ __global__ void __launch_bounds__(kScThr, 1)
       ScoreItem it;
       if (!score_item(p, i, Jt, it)) continue;
       const int kb = nk & 1;
-      if (nk >= 2) ok = wait_warp(smem_u32(&b_kfree[kb]), (uint32_t)((nk / 2 - 1) & 1));
+      if (nk >= 2) ok = wait_warp(B.kfree[kb], nk / 2 - 1);
       if (!ok) break;
       if (lane == 0) {
         const int rows = min(2 * kBlk, it.n - it.k0), nbox = (rows + kBox - 1) / kBox;
-        const uint32_t bar = smem_u32(&b_kfull[kb]);
+        const uint32_t bar = smem_u32(&B.kfull[kb]);
         const int row = (int)(it.u.ug * (size_t)c.cap) + it.k0;
         mbar_expect_tx(bar, (uint32_t)nbox * 2 * kBox * 128);
         for (int b = 0; b < nbox; ++b)
@@ -675,20 +693,26 @@ __global__ void __launch_bounds__(kScThr, 1)
           const int col = 32 * x + lane;
           v[x] = col < nv ? lu[base + col] : INFINITY;
         }
-        if (nq >= kQRing)
-          ok = wait_warp(smem_u32(&b_qfree[s]), (uint32_t)((nq / kQRing - 1) & 1));
+        if (nq >= kQRing) ok = wait_warp(B.qfree[s], nq / kQRing - 1);
         if (!ok) break;
-        const uint32_t bar = smem_u32(&b_qfull[s]);
         if (lane == 0) {
+          const uint32_t bar = smem_u32(&B.qfull[s]);
           mbar_expect_tx(bar, q_bytes);
           for (int hf = 0; hf < 2; ++hf)
             tma_load_4d(aQ + s * kTile + hf * kHalf, &tmQ, 64 * hf, 0, it.u.h,
                         (int)it.u.row0 + q * Jt, bar);
         }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) s_lse[s * kBlk + 32 * x + lane] = -v[x];
-        mbar_arrive(bar);
+        // The normalisers have slots of their own: the softmax still reads
+        // them when the contraction has long released the query tile.  (In
+        // one slot with it, the three query tiles in flight waited for the
+        // softmax: 249 us against 227, 7B, two 1,000-token prompts.)
+        const int sl = nq % kLRing;
         ++nq;
+        if (nq > kLRing) ok = wait_warp(B.lfree[sl], (nq - 1) / kLRing - 1);
+        if (!ok) break;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) s_lse[sl * kBlk + 32 * x + lane] = -v[x];
+        mbar_arrive(smem_u32(&B.lfull[sl]));
       }
     }
     __syncwarp();
@@ -699,9 +723,9 @@ __global__ void __launch_bounds__(kScThr, 1)
       }
       volatile int never = 0;
       for (int k = max(0, nk - 2); k < nk; ++k)
-        mbar_wait(smem_u32(&b_kfull[k & 1]), (uint32_t)((k / 2) & 1), &never);
+        mbar_wait(smem_u32(&B.kfull[k & 1]), (uint32_t)((k / 2) & 1), &never);
       for (int k = max(0, nq - kQRing); k < nq; ++k)
-        mbar_wait(smem_u32(&b_qfull[k % kQRing]), (uint32_t)((k / kQRing) & 1), &never);
+        mbar_wait(smem_u32(&B.qfull[k % kQRing]), (uint32_t)((k / kQRing) & 1), &never);
     }
   } else if (warp == kIssuer) {
     int nk = 0, nq = 0, ns0 = 0, ns1 = 0;
@@ -711,15 +735,15 @@ __global__ void __launch_bounds__(kScThr, 1)
       ScoreItem it;
       if (!score_item(p, i, Jt, it)) continue;
       const int kb = nk & 1;
-      ok = wait_warp(smem_u32(&b_kfull[kb]), (uint32_t)((nk / 2) & 1));
+      ok = wait_warp(B.kfull[kb], nk / 2);
       for (int q = it.q0(0); q < n_qt && ok; ++q) {
         const int s = nq % kQRing;
-        ok = wait_warp(smem_u32(&b_qfull[s]), (uint32_t)((nq / kQRing) & 1));
+        ok = wait_warp(B.qfull[s], nq / kQRing);
         for (int t = 0; t < 2 && ok; ++t) {
           if (it.nk(t) <= 0 || q < it.q0(t)) continue;
           int &ns = t ? ns1 : ns0;
           const int b = ns & 1;
-          if (ns >= 2) ok = wait_warp(smem_u32(&b_sfree[t][b]), (uint32_t)((ns / 2 - 1) & 1));
+          if (ns >= 2) ok = wait_warp(B.sfree[t][b], ns / 2 - 1);
           if (!ok) break;
           ++ns;
           tc_fence_after();
@@ -731,15 +755,15 @@ __global__ void __launch_bounds__(kScThr, 1)
               const uint64_t off = (uint64_t)(((k >> 2) * kHalf + (k & 3) * 32) >> 4);
               tc_mma(tm + (t * 2 + b) * kBlk, a0 + off, b0 + off, id, k > 0);
             }
-            tc_commit(smem_u32(&b_s[t][b]));
+            tc_commit(smem_u32(&B.s[t][b]));
           }
         }
         if (!ok) break;
-        if (lane == 0) tc_commit(smem_u32(&b_qfree[s]));
+        if (lane == 0) tc_commit(smem_u32(&B.qfree[s]));
         ++nq;
       }
       if (!ok) break;
-      if (lane == 0) tc_commit(smem_u32(&b_kfree[kb]));
+      if (lane == 0) tc_commit(smem_u32(&B.kfree[kb]));
       ++nk;
     }
     if (lane == 0) {
@@ -748,8 +772,8 @@ __global__ void __launch_bounds__(kScThr, 1)
         *abort = 1;
       }
       volatile int never = 0;
-      tc_commit(smem_u32(&b_drain));
-      mbar_wait(smem_u32(&b_drain), 0, &never);
+      tc_commit(smem_u32(&B.drain));
+      mbar_wait(smem_u32(&B.drain), 0, &never);
     }
   } else if (warp < kProducer) {
     // Two warpgroups a key tile, which take its S buffers in turn; thread r
@@ -766,26 +790,27 @@ __global__ void __launch_bounds__(kScThr, 1)
       const int tmin = max(0, slot - it.u.m);  // first token that sees the row
       const int tmin_w = max(0, it.k0 + t * kBlk + wq * 32 + 31 - it.u.m);
       const int q1 = it.nk(t) > 0 ? it.q0(t) : n_qt;
-      uint64_t a0 = pk2(0.f, 0.f), a1 = a0;
+      // The row's sum: of each query tile's 128 terms apart, then over the
+      // tiles.  (What is left of the scores' error, 1.3e-7 to 1.7e-7 relative,
+      // is the contraction's accumulation: compensated sums did not move it.)
+      float sum = 0.f;
       for (int q = it.q0(0); q < n_qt; ++q) {
-        const int s = nq % kQRing;
-        const uint32_t ph_q = (uint32_t)((nq / kQRing) & 1);
+        const int s = nq % kLRing, ph_l = nq / kLRing;
         ++nq;
-        // One of the tile's two warpgroups releases each query tile: the one
+        // One of the tile's two warpgroups releases each tile's normalisers: the one
         // that reads it, or the first where the tile has nothing to read (its
         // arrival must count for this filling of the slot, hence the wait).
         if (q < q1) {
           if (b == 0) {
-            ok = wait_warp(smem_u32(&b_qfull[s]), ph_q);
+            ok = wait_warp(B.lfull[s], ph_l);
             if (!ok) break;
-            if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+            if (lane == 0) mbar_arrive(smem_u32(&B.lfree[s]));
           }
           continue;
         }
         const int n = ns++;
         if ((n & 1) != b) continue;
-        ok = wait_warp(smem_u32(&b_s[t][b]), (uint32_t)((n / 2) & 1)) &&
-             wait_warp(smem_u32(&b_qfull[s]), ph_q);
+        ok = wait_warp(B.s[t][b], n / 2) && wait_warp(B.lfull[s], ph_l);
         if (!ok) break;
         tc_fence_after();
         const int toks = p.chunk - q * Jt;  // tokens from this tile on
@@ -793,6 +818,7 @@ __global__ void __launch_bounds__(kScThr, 1)
         // Columns of tokens before tmin do not see the row; columns past the
         // chunk hold no query.
         const int c_lo = (tmin - q * Jt) * G, c_hi = min(Jt, toks) * G;
+        uint64_t a0 = pk2(0.f, 0.f), a1 = a0;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           float e[2][32];
@@ -802,7 +828,7 @@ __global__ void __launch_bounds__(kScThr, 1)
           if (hf == 1) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&b_sfree[t][b]));
+            if (lane == 0) mbar_arrive(smem_u32(&B.sfree[t][b]));
           }
           const ulonglong2 *nl = reinterpret_cast<const ulonglong2 *>(s_lse + s * kBlk + 64 * hf);
           if (all) {
@@ -836,14 +862,15 @@ __global__ void __launch_bounds__(kScThr, 1)
               }
           }
         }
+        float x0, x1, y0, y1;
+        upk2(a0, x0, x1);
+        upk2(a1, y0, y1);
+        sum += (x0 + x1) + (y0 + y1);
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&b_qfree[s]));
+        if (lane == 0) mbar_arrive(smem_u32(&B.lfree[s]));
       }
       // The two warpgroups' sums, added one after the other.
-      float x0, x1, y0, y1;
-      upk2(a0, x0, x1);
-      upk2(a1, y0, y1);
-      const float sum = ((x0 + x1) + (y0 + y1)) * p.inv_g;
+      sum *= p.inv_g;
       float *su = c.score + it.u.ug * (size_t)c.sstride + slot;
       if (b == 0 && ok && slot < it.n) *su += sum;
       int bad;

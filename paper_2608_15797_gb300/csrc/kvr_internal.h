@@ -307,6 +307,7 @@ struct AbsorbParams {
 };
 int absorb_max_chunk();
 int absorb_max_rows();
+int absorb_tc_max_rows();  // of the tensor-memory kernel
 // kernel: 0 the tensor-memory (tcgen05) kernel (units of at most 144 rows
 // after the chunk, given tmQ; otherwise the other), 1 the mma.sync kernel.
 // tmQ: q as a 4-D tensor {128, G, H, S * nl * chunk tokens} with boxes
