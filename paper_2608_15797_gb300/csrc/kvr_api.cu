@@ -1033,6 +1033,20 @@ kvr_status kvr_decode_step(kvr_cache *c, int lb, int le, const void *q,
     mirror_evict(c, lb, le, budget, window);
     return KVR_OK;
   }
+  // Shapes that only the generic kernels take (fp32, head_dim 64): one launch
+  // where every row of a unit has a thread to rank it.
+  if (c->fused && (!c->view.kv_bf16 || c->view.d != 128) &&
+      a.max_rows <= kvr::generic_evict_rows()) {
+    a.evict = 1;
+    a.budget = budget;
+    a.window = window;
+    e = kvr::launch_attend_score_generic(c->view, a, as_stream(stream));
+    if (e != cudaSuccess) return cuda_fail("kvr_decode_step", e);
+    c->launches += 1;
+    mirror_append(c, lb, le);
+    mirror_evict(c, lb, le, budget, window);
+    return KVR_OK;
+  }
   st = kvr_decode_attend_score(c, lb, le, q, k_new, v_new, out, stream);
   if (st != KVR_OK) return st;
   return kvr_evict_compact(c, lb, le, budget, window, stream);

@@ -44,6 +44,166 @@ __device__ __forceinline__ Unit unit_of(const CacheView &c, int lb, int nl) {
   return x;
 }
 
+// The need-th largest of v(i) over the rows i in [0, n) with v(i) != kNone, by
+// passes over a 2,048-bin histogram, each over the range that the last one
+// left: first the values' own range (scores share their leading bits, and
+// bins by those would take all the additions), three passes at most.  Returns
+// the value; *rest is how many of the rows that equal it belong to the `need`,
+// *ties how many rows equal it.  need >= 1 and at least `need` such rows must
+// exist.  lo, hi: the least and greatest value among the rows that this thread
+// has seen (kNone, 0 for none); every row must have been seen by some thread.
+// Every thread must call it.
+constexpr unsigned kNone = 0xFFFFFFFFu;
+struct SelectSmem {
+  unsigned hist[2048];
+  unsigned wsum[32], wmax[32];
+  unsigned digit, above, count;
+};
+template <int NT, typename Val>
+__device__ unsigned select_desc(int n, unsigned need, Val v, unsigned lo, unsigned hi,
+                                SelectSmem &m, unsigned *rest, unsigned *ties) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kPer = 2048 / NT;  // bins a thread scans
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    m.wsum[warp] = lo;
+    m.wmax[warp] = hi;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    lo = min(lo, m.wsum[w]);
+    hi = max(hi, m.wmax[w]);
+  }
+  int shift = max(0, 32 - __clz((int)(hi - lo)) - 11);
+  unsigned bins = 2048;  // of the range left
+  for (bool last = false; !last;) {
+    last = shift == 0;
+    for (int i = tid; i < 2048; i += NT) m.hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NT) {
+      const unsigned x = v(i), bin = (x - lo) >> shift;
+      if (x != kNone && bin < bins) atomicAdd(&m.hist[bin], 1u);
+    }
+    __syncthreads();
+    // Inclusive counts from the top bin down; thread t owns kPer bins.
+    unsigned c[kPer], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      c[k] = m.hist[2047 - (tid * kPer + k)];
+      s += c[k];
+    }
+    unsigned inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) m.wsum[warp] = inc;
+    __syncthreads();
+    unsigned above = inc - s;
+    for (int w = 0; w < warp; ++w) above += m.wsum[w];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (above < need && above + c[k] >= need) {
+        m.digit = 2047 - (tid * kPer + k);
+        m.above = above;
+        m.count = c[k];
+      }
+      above += c[k];
+    }
+    __syncthreads();
+    lo += m.digit << shift;
+    need -= m.above;
+    *ties = m.count;
+    bins = 1u << min(shift, 11);
+    shift = max(0, shift - 11);
+    __syncthreads();
+  }
+  *rest = need;
+  return lo;
+}
+
+// The end of an eviction: the rows that keep(i) names, nk of unit u's n, stay;
+// lists has room for 2 * max_list entries.  Every thread must call it.
+template <typename T, int D, int NT, typename Keep>
+__device__ void compact_unit(const CacheView &c, size_t u, int n, int nk, Keep keep, int *lists,
+                             int max_list, int2 *s_cnt) {
+  const int tid = threadIdx.x;
+  T *Ku = reinterpret_cast<T *>(c.K) + u * (size_t)c.cap * D;
+  T *Vu = reinterpret_cast<T *>(c.V) + u * (size_t)c.cap * D;
+  float *su = c.score + u * (size_t)c.sstride;
+  int32_t *pu = c.pos + u * (size_t)c.sstride;
+  int *holes = lists, *movers = lists + max_list;
+  // The freed slots below nk and the survivors above, both in ascending
+  // order: each warp takes a contiguous run of rows, counts, and after one
+  // exchange of counts writes its part of the lists.
+  constexpr int kNW = NT / 32;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int seg = (n + kNW * 32 - 1) / (kNW * 32) * 32;
+  const int r0 = min(n, warp * seg), r1 = min(n, r0 + seg);
+  int ch = 0, cm = 0;
+  for (int base = r0; base < r1; base += 32) {
+    const int i = base + lane;
+    const bool in = i < r1, k = in && keep(i);
+    ch += __popc(__ballot_sync(0xffffffffu, in && i < nk && !k));
+    cm += __popc(__ballot_sync(0xffffffffu, in && i >= nk && k));
+  }
+  if (lane == 0) s_cnt[warp] = make_int2(ch, cm);
+  __syncthreads();
+  int oh = 0, om = 0, nh = 0, nm = 0;
+#pragma unroll
+  for (int w = 0; w < kNW; ++w) {
+    const int2 x = s_cnt[w];
+    if (w < warp) {
+      oh += x.x;
+      om += x.y;
+    }
+    nh += x.x;
+    nm += x.y;
+  }
+  // As many survivors above nk as free slots below: the window is intact
+  // and B + W rows stay.
+  if (nh != nm || nh > max_list) {
+    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+    return;
+  }
+  const unsigned below = (1u << lane) - 1u;
+  for (int base = r0; base < r1; base += 32) {
+    const int i = base + lane;
+    const bool in = i < r1, k = in && keep(i);
+    const bool h = in && i < nk && !k, m = in && i >= nk && k;
+    const unsigned bh = __ballot_sync(0xffffffffu, h), bm = __ballot_sync(0xffffffffu, m);
+    if (h) holes[oh + __popc(bh & below)] = i;
+    if (m) movers[om + __popc(bm & below)] = i;
+    oh += __popc(bh);
+    om += __popc(bm);
+  }
+  __syncthreads();
+  // Move every survivor beyond nk into a freed slot below it (disjoint).
+  constexpr int kChunks = D * (int)sizeof(T) / 16;
+  for (int j = warp; j < nh; j += kNW) {
+    const int dst = holes[j], src = movers[j];
+    const int4 *ks = reinterpret_cast<const int4 *>(Ku + (size_t)src * D);
+    const int4 *vs = reinterpret_cast<const int4 *>(Vu + (size_t)src * D);
+    int4 *kd = reinterpret_cast<int4 *>(Ku + (size_t)dst * D);
+    int4 *vd = reinterpret_cast<int4 *>(Vu + (size_t)dst * D);
+    for (int q = lane; q < kChunks; q += 32) {
+      kd[q] = ks[q];
+      vd[q] = vs[q];
+    }
+    if (lane == 0) {
+      su[dst] = su[src];
+      pu[dst] = pu[src];
+    }
+  }
+  if (tid == 0) {
+    c.state[4 * u] = nk;
+    c.state[4 * u + 2] = 0;  // the R-KV key sum no longer matches
+  }
+}
+
 // Dynamic shared memory of attend_score_kernel (floats).
 __host__ __device__ constexpr int attend_fixed_floats(int D) {
   return kMaxG * D                           // q
@@ -52,8 +212,11 @@ __host__ __device__ constexpr int attend_fixed_floats(int D) {
 }
 
 // kExtScratch: logits always go to `ext`, one [G][max_rows] block per CTA,
-// instead of shared memory or the cache's own scratch area.
-template <typename T, typename O, int D, bool kExtScratch = false>
+// instead of shared memory or the cache's own scratch area.  kEvict: the CTA
+// also cuts its unit (at most kThreads rows with the new one) back to budget +
+// window rows, by rank, as evict_kernel would: one launch where a step's cost
+// is launches (one layer, 2 units, fp32: 9.0 us a step in two, 6.9 in one).
+template <typename T, typename O, int D, bool kExtScratch = false, bool kEvict = false>
 __global__ void __launch_bounds__(kThreads)
     attend_score_kernel(CacheView c, StepArgs a, int logits_in_smem,
                         float *ext) {
@@ -195,87 +358,24 @@ __global__ void __launch_bounds__(kThreads)
     c.state[4 * x.u + 1] = newest + 1;
     c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
   }
-}
-
-// The need-th largest of v(i) over the rows i in [0, n) with v(i) != kNone, by
-// passes over a 2,048-bin histogram, each over the range that the last one
-// left: first the values' own range (scores share their leading bits, and
-// bins by those would take all the additions), three passes at most.  Returns
-// the value; *rest is how many of the rows that equal it belong to the `need`,
-// *ties how many rows equal it.  need >= 1 and at least `need` such rows must
-// exist.  lo, hi: the least and greatest value among the rows that this thread
-// has seen (kNone, 0 for none); every row must have been seen by some thread.
-// Every thread must call it.
-constexpr unsigned kNone = 0xFFFFFFFFu;
-struct SelectSmem {
-  unsigned hist[2048];
-  unsigned wsum[32], wmax[32];
-  unsigned digit, above, count;
-};
-template <int NT, typename Val>
-__device__ unsigned select_desc(int n, unsigned need, Val v, unsigned lo, unsigned hi,
-                                SelectSmem &m, unsigned *rest, unsigned *ties) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kPer = 2048 / NT;  // bins a thread scans
-  lo = __reduce_min_sync(0xffffffffu, lo);
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) {
-    m.wsum[warp] = lo;
-    m.wmax[warp] = hi;
+  if constexpr (kEvict) {
+    const int nk = a.budget + a.window;
+    if (n <= nk) return;
+    if (n > kThreads) {  // the host sized the launch from its mirror
+      if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+      return;
+    }
+    __shared__ unsigned long long s_key[kThreads];
+    __shared__ unsigned char s_keep[kThreads];
+    __shared__ int s_lists[2 * kThreads];
+    __shared__ int2 s_cnt[kWarps];
+    const int wlo = newest - a.window;
+    block_rank_keep(
+        n, a.budget, [&](int i) { return pu[i] <= wlo; },
+        [&](int i) { return rank_key(su[i], pu[i]); }, s_key, s_keep);
+    compact_unit<T, D, kThreads>(
+        c, x.u, n, nk, [&](int i) { return s_keep[i] != 0; }, s_lists, kThreads, s_cnt);
   }
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < NT / 32; ++w) {
-    lo = min(lo, m.wsum[w]);
-    hi = max(hi, m.wmax[w]);
-  }
-  int shift = max(0, 32 - __clz((int)(hi - lo)) - 11);
-  unsigned bins = 2048;  // of the range left
-  for (bool last = false; !last;) {
-    last = shift == 0;
-    for (int i = tid; i < 2048; i += NT) m.hist[i] = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += NT) {
-      const unsigned x = v(i), bin = (x - lo) >> shift;
-      if (x != kNone && bin < bins) atomicAdd(&m.hist[bin], 1u);
-    }
-    __syncthreads();
-    // Inclusive counts from the top bin down; thread t owns kPer bins.
-    unsigned c[kPer], s = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      c[k] = m.hist[2047 - (tid * kPer + k)];
-      s += c[k];
-    }
-    unsigned inc = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) m.wsum[warp] = inc;
-    __syncthreads();
-    unsigned above = inc - s;
-    for (int w = 0; w < warp; ++w) above += m.wsum[w];
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      if (above < need && above + c[k] >= need) {
-        m.digit = 2047 - (tid * kPer + k);
-        m.above = above;
-        m.count = c[k];
-      }
-      above += c[k];
-    }
-    __syncthreads();
-    lo += m.digit << shift;
-    need -= m.above;
-    *ties = m.count;
-    bins = 1u << min(shift, 11);
-    shift = max(0, shift - 11);
-    __syncthreads();
-  }
-  *rest = need;
-  return lo;
 }
 
 // Cut every unit longer than B + W back to B + W rows.  kByRank: units of at
@@ -303,82 +403,13 @@ __global__ void __launch_bounds__(NT)
     c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
   }
   if (n <= B + W) return;
-  T *Ku = reinterpret_cast<T *>(c.K) + x.u * (size_t)c.cap * D;
-  T *Vu = reinterpret_cast<T *>(c.V) + x.u * (size_t)c.cap * D;
   float *su = c.score + x.u * (size_t)c.sstride;
   int32_t *pu = c.pos + x.u * (size_t)c.sstride;
   // The W most recent positions are protected; a row is a candidate iff its
   // position is at most newest - W.
   const int wlo = newest - W;
-  const int nk = B + W;
-  int *holes = lists, *movers = lists + max_list;
   auto finish = [&](auto keep) {
-    // The freed slots below nk and the survivors above, both in ascending
-    // order: each warp takes a contiguous run of rows, counts, and after one
-    // exchange of counts writes its part of the lists.
-    constexpr int kNW = NT / 32;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int seg = (n + kNW * 32 - 1) / (kNW * 32) * 32;
-    const int r0 = min(n, warp * seg), r1 = min(n, r0 + seg);
-    int ch = 0, cm = 0;
-    for (int base = r0; base < r1; base += 32) {
-      const int i = base + lane;
-      const bool in = i < r1, k = in && keep(i);
-      ch += __popc(__ballot_sync(0xffffffffu, in && i < nk && !k));
-      cm += __popc(__ballot_sync(0xffffffffu, in && i >= nk && k));
-    }
-    if (lane == 0) s_cnt[warp] = make_int2(ch, cm);
-    __syncthreads();
-    int oh = 0, om = 0, nh = 0, nm = 0;
-#pragma unroll
-    for (int w = 0; w < kNW; ++w) {
-      const int2 x = s_cnt[w];
-      if (w < warp) {
-        oh += x.x;
-        om += x.y;
-      }
-      nh += x.x;
-      nm += x.y;
-    }
-    // As many survivors above nk as free slots below: the window is intact
-    // and B + W rows stay.
-    if (nh != nm || nh > max_list) {
-      if (tid == 0) atomicOr(c.err, ERR_LENGTH);
-      return;
-    }
-    const unsigned below = (1u << lane) - 1u;
-    for (int base = r0; base < r1; base += 32) {
-      const int i = base + lane;
-      const bool in = i < r1, k = in && keep(i);
-      const bool h = in && i < nk && !k, m = in && i >= nk && k;
-      const unsigned bh = __ballot_sync(0xffffffffu, h), bm = __ballot_sync(0xffffffffu, m);
-      if (h) holes[oh + __popc(bh & below)] = i;
-      if (m) movers[om + __popc(bm & below)] = i;
-      oh += __popc(bh);
-      om += __popc(bm);
-    }
-    __syncthreads();
-    // Move every survivor beyond nk into a freed slot below it (disjoint).
-    constexpr int kChunks = D * (int)sizeof(T) / 16;
-    for (int j = warp; j < nh; j += kNW) {
-      const int dst = holes[j], src = movers[j];
-      const int4 *ks = reinterpret_cast<const int4 *>(Ku + (size_t)src * D);
-      const int4 *vs = reinterpret_cast<const int4 *>(Vu + (size_t)src * D);
-      int4 *kd = reinterpret_cast<int4 *>(Ku + (size_t)dst * D);
-      int4 *vd = reinterpret_cast<int4 *>(Vu + (size_t)dst * D);
-      for (int q = lane; q < kChunks; q += 32) {
-        kd[q] = ks[q];
-        vd[q] = vs[q];
-      }
-      if (lane == 0) {
-        su[dst] = su[src];
-        pu[dst] = pu[src];
-      }
-    }
-    if (tid == 0) {
-      c.state[4 * x.u] = nk;
-      c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
-    }
+    compact_unit<T, D, NT>(c, x.u, n, B + W, keep, lists, max_list, s_cnt);
   };
   if constexpr (kByRank) {
     __shared__ unsigned long long s_key[NT];
@@ -492,7 +523,8 @@ cudaError_t attend_dispatch(const CacheView &c, const StepArgs &a,
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int in_smem = fixed + lg <= (size_t)optin ? 1 : 0;
   const size_t bytes = fixed + (in_smem ? lg : 0);
-  auto kern = attend_score_kernel<T, O, D>;
+  auto kern = a.evict ? attend_score_kernel<T, O, D, false, true>
+                      : attend_score_kernel<T, O, D>;
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
@@ -544,6 +576,8 @@ cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
 }
 
 }  // namespace
+
+int generic_evict_rows() { return kThreads; }
 
 cudaError_t launch_attend_score_generic(const CacheView &c, const StepArgs &a,
                                         cudaStream_t st) {

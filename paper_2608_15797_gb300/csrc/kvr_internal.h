@@ -92,6 +92,9 @@ struct StepArgs {
 };
 
 // Generic kernels (any d in {64,128}, G <= 8, fp32 or bf16): one CTA per unit.
+// With a.evict the launch also evicts (units of at most generic_evict_rows()
+// rows after the append).
+int generic_evict_rows();
 cudaError_t launch_attend_score_generic(const CacheView &c, const StepArgs &a,
                                         cudaStream_t st);
 // The attend kernel with its logits always in `ext` (one [G][max_rows] fp32
