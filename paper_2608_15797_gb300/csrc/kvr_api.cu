@@ -14,7 +14,6 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <array>
 #include <vector>
 
 #include "../../include/kvr.h"
@@ -165,21 +164,33 @@ bool encode_tails3(CUtensorMap *m, void *base, size_t rows_per_cand, int n_cand,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The N candidates' tails as a 4-D tensor {128 elements, nt rows, units, N}
-// (a unit's tail is tcap rows apart, a candidate's units * tcap): a box
-// {64, round_up16(nt), 1, min(N, 2)} fetches the first nt rows of one unit's
-// tails for two candidates and fills the rest of the box with zeros.
-bool encode_tails4(CUtensorMap *m, void *base, int nt, int tcap, size_t units,
-                   int n_cand) {
+// The N candidates' tails as {128 elements, nt rows, units, N} with boxes of T
+// rows of one unit for every candidate; rows past nt are filled with zeros.
+bool encode_tail_tile(CUtensorMap *m, void *base, int nt, int tcap, size_t units,
+                      int n_cand, int T) {
   auto fn = encode_tiled();
   if (!fn || nt < 1) return false;
   cuuint64_t dims[4] = {128, (cuuint64_t)nt, (cuuint64_t)units, (cuuint64_t)n_cand};
   cuuint64_t strides[3] = {256, (cuuint64_t)tcap * 256, (cuuint64_t)units * tcap * 256};
-  cuuint32_t box[4] = {64, (cuuint32_t)kvr::round_up16(nt), 1,
-                       (cuuint32_t)std::min(n_cand, 2)};
+  cuuint32_t box[4] = {64, (cuuint32_t)T, 1, (cuuint32_t)n_cand};
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The candidates' queries as {128 elements, G heads, units of the call, N}:
+// a box holds two candidates' rows of one unit.
+bool encode_cand_q(CUtensorMap *m, const void *base, int G, size_t units, int n_cand) {
+  auto fn = encode_tiled();
+  if (!fn) return false;
+  cuuint64_t dims[4] = {128, (cuuint64_t)G, (cuuint64_t)units, (cuuint64_t)n_cand};
+  cuuint64_t strides[3] = {256, (cuuint64_t)G * 256, (cuuint64_t)units * G * 256};
+  cuuint32_t box[4] = {64, (cuuint32_t)G, 1, 2};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides,
+            box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1297,10 +1308,6 @@ struct kvr_fork {
   CUtensorMap tmTK, tmTV;     // 16-row boxes
   bool batch_maps = false;    // 3-D tail maps (candidate-batched kernel)
   CUtensorMap tmTK3, tmTV3;
-  // Tail maps of the tensor-memory kernel, per tail length nt (encoded on
-  // first use): 0 not yet, 1 encoded, -1 cannot be encoded.
-  std::vector<signed char> tc_state;
-  std::vector<std::array<CUtensorMap, 2>> tc_tails;
   int kernel = 0;             // kvr_fork_set_kernel choice
   int last_kernel = 0;        // the kernel that ran the last step (1..5)
 };
@@ -1414,8 +1421,6 @@ kvr_status kvr_fork_candidates(kvr_cache *p, int n_cand, int tail_cap,
         T > 0 &&
         encode_tails3(&f->tmTK3, v.TK, units * (size_t)tail_cap, n_cand, T) &&
         encode_tails3(&f->tmTV3, v.TV, units * (size_t)tail_cap, n_cand, T);
-    f->tc_state.assign(std::min(tail_cap, kvr::fork_tc_max_tail()) + 1, 0);
-    f->tc_tails.resize(f->tc_state.size());
   }
   p->forks += 1;
   *out = f;
@@ -1465,37 +1470,37 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
   const CacheView &pv = p->view;
   const std::pair<CUtensorMap, CUtensorMap> *maps = nullptr, *maps128 = nullptr;
   const int want = p->fused ? f->kernel : 4;  // 0 auto, 1..5 one kernel
-  // The tensor-memory kernel (chosen explicitly only: the candidate-batched
-  // kernel is faster at the sizes measured) wants every unit of the call at
-  // the same tail length (its tail maps end there).
+  // The tile kernel wants every unit of the call at the same tail length (its
+  // tail maps end there).
   bool nt_same = true;
   for (int s = 0; s < p->desc.n_seq && nt_same; ++s)
     for (int l = lb; l < le; ++l)
       nt_same = nt_same && f->tlen[(size_t)s * p->desc.n_layers + l] == nt_max;
-  const CUtensorMap *tails = nullptr;
-  if (want == 5 && nt_same && (size_t)nt_max < f->tc_state.size()) {
-    signed char &st8 = f->tc_state[nt_max];
-    if (st8 == 0) {
-      const size_t units = (size_t)pv.S * pv.L * pv.H;
-      const int rows = std::max(nt_max, 1);
-      st8 = encode_tails4(&f->tc_tails[nt_max][0], f->view.TK, rows, f->view.tcap, units,
-                          f->view.N) &&
-                    encode_tails4(&f->tc_tails[nt_max][1], f->view.TV, rows, f->view.tcap,
-                                  units, f->view.N)
-                ? 1
-                : -1;
-    }
-    if (st8 == 1) tails = f->tc_tails[nt_max].data();
-  }
-  const bool tc_ok =
-      want == 5 && p->fused && tails && pv.G <= 8 &&
-      f->view.N <= kvr::fork_tc_max_cand() && device_facts(p) &&
-      kvr::fork_tc_smem_bytes() <= (size_t)p->smem_optin &&
-      max_prefix <= kvr::fork_tc_max_prefix() && nt_max <= kvr::fork_tc_max_tail() &&
+  // By itself the library takes tiles on the tensor cores for four candidates
+  // and more where every SM gets several units: a tile costs the same for any
+  // number of candidates, and its long chain of steps wants other units to
+  // hide behind.  72B geometry, 64 + 8 rows, a fork of 16 tokens and commit,
+  // against one warp a candidate: 640 units, N = 8: 637 and 774 us, N = 4: 576
+  // and 598, N = 2: 566 and 542; 2,560 units, N = 8: 1,786 and 2,482, N = 4: 1,640
+  // and 1,915; 448 units (7B), N = 8: 490 and 511, N = 4: 455 and 405.  Asked for
+  // (kernel 5), within the limits that choice has.
+  const int call_units = pv.S * (le - lb) * pv.H;
+  CUtensorMap tile_q, tile_k, tile_v;
+  const bool tile_ok =
+      (want == 0 || (want == 5 && max_prefix <= 128 && nt_max <= 64)) && p->fused && pv.kv_bf16 && pv.d == 128 && nt_same && pv.G <= 8 &&
+      f->view.N <= kvr::fork_tile_max_cand() && device_facts(p) &&
+      (want == 5 || (f->view.N >= 4 && call_units >= 4 * p->sm_count)) &&
       (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
       aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
-      (maps = slab_maps(p, kvr::fork_tc_box_rows())) != nullptr;
-  const bool batch_ok = !tc_ok &&
+      (maps = slab_maps(p, kvr::fork_tile_box_rows())) != nullptr &&
+      encode_cand_q(&tile_q, q, pv.G, (size_t)call_units, f->view.N) &&
+      encode_tail_tile(&tile_k, f->view.TK, std::max(nt_max, 1), f->view.tcap,
+                       (size_t)pv.S * pv.L * pv.H, f->view.N,
+                       kvr::fork_tile_tail_rows(f->view.N)) &&
+      encode_tail_tile(&tile_v, f->view.TV, std::max(nt_max, 1), f->view.tcap,
+                       (size_t)pv.S * pv.L * pv.H, f->view.N,
+                       kvr::fork_tile_tail_rows(f->view.N));
+  const bool batch_ok = !tile_ok &&
       (want == 0 || want == 1) && p->fused && f->batch_maps && pv.G <= 8 &&
       f->view.N <= kvr::fork_batch_max_cand() && device_facts(p) &&
       kvr::fork_batch_smem_bytes(n_max, f->view.N) + 512 <=
@@ -1505,14 +1510,14 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr &&
       (maps128 = slab_maps(p, kvr::fork_batch_prefix_box_rows())) != nullptr;
   kvr::ChunkParams cp{};
-  const bool chunk_ok = !batch_ok && (want == 0 || want == 2) &&
+  const bool chunk_ok = !batch_ok && !tile_ok && (want == 0 || want == 2) &&
       p->fused && p->chunk_groups >= 0 && f->tail_maps && pv.G <= 8 &&
       n_max <= kvr::chunk_max_rows() && device_facts(p) &&
       chunk_config(p, n_max, &cp.n_groups, &cp.n_stages) &&
       (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
       aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr;
-  const bool mma_ok = !batch_ok && !chunk_ok && (want == 0 || want == 3) &&
+  const bool mma_ok = !batch_ok && !tile_ok && !chunk_ok && (want == 0 || want == 3) &&
       p->fused && f->tail_maps && pv.G <= 8 &&
       f->view.N <= kvr::fork_mma_max_cand() && device_facts(p) &&
       kvr::fork_mma_smem_bytes(max_prefix, nt_max, f->view.N) + 512 <=
@@ -1520,8 +1525,8 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
       (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
       aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
       (maps = slab_maps(p, kvr::fork_mma_box_rows())) != nullptr;
-  if (tc_ok) {
-    kvr::ForkTcParams tp{};
+  if (tile_ok) {
+    kvr::ForkTileParams tp{};
     tp.f = f->view;
     tp.q = static_cast<const __nv_bfloat16 *>(q);
     tp.k_new = static_cast<const __nv_bfloat16 *>(k_new);
@@ -1529,13 +1534,11 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
     tp.out = out;
     tp.lb = lb;
     tp.nl = le - lb;
+    tp.nt = nt_max;
     tp.scale_log2e = pv.scale * 1.4426950408889634f;
     tp.inv_g = 1.f / (float)pv.G;
-    const int units = pv.S * (le - lb) * pv.H;
-    tp.nt = nt_max;
-    tp.np_max = max_prefix;
-    e = kvr::launch_fork_tc(maps->first, maps->second, &tails[0], &tails[1], tp,
-                            std::min(p->sm_count, units), as_stream(stream));
+    e = kvr::launch_fork_tile(maps->first, maps->second, tile_k, tile_v, tile_q, tp,
+                              p->sm_count, as_stream(stream));
   } else if (batch_ok) {
     kvr::ForkBatchParams bp{};
     bp.f = f->view;
@@ -1588,7 +1591,7 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
                                 as_stream(stream));
   }
   if (e != cudaSuccess) return cuda_fail("kvr_fork_decode_attend_score", e);
-  f->last_kernel = tc_ok ? 5 : batch_ok ? 1 : chunk_ok ? 2 : mma_ok ? 3 : 4;
+  f->last_kernel = tile_ok ? 5 : batch_ok ? 1 : chunk_ok ? 2 : mma_ok ? 3 : 4;
   p->launches += 1;
   for (int s = 0; s < p->desc.n_seq; ++s)
     for (int l = lb; l < le; ++l) f->tlen[(size_t)s * p->desc.n_layers + l] += 1;
