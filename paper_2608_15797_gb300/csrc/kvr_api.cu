@@ -433,22 +433,56 @@ bool try_stream(kvr_cache *c, const StepArgs &a, bool evict, int budget,
   return true;
 }
 
-// Consumer groups and ring stages per group of the chunked kernel for jobs
-// of up to n_max rows: the first of (4,2) (3,3) (3,2) (2,3) (2,2) (1,3)
-// (1,2) that fits in shared memory (more groups first: measured), or the
-// tuned choice.
-bool chunk_config(const kvr_cache *c, int n_max, int *groups, int *stages,
-                  bool rkv = false) {
+// Whether plain units run in groups of four warps (64-row chunks) in the
+// chunked kernel, for `per` units an SM and units of up to n_max rows.  A
+// group of four takes about two thirds of a pair's time for a unit, so what
+// counts is how many rounds of units an SM needs.  us a step on one GB300:
+//   one unit an SM: 18.1 against 21.0 with two or three pairs (521 rows),
+//     23.0 against 32.3 (909 rows); R-KV 22.0 against 30.9 (521 rows);
+//   two: 17.7 against 21.7 (521 rows);
+//   more, where four pairs do not fit (more than about 330 rows): two groups
+//     of four take 2/3 of the time of three pairs, and 0.64 of it beyond 416
+//     rows (R-KV: 480), where the last 64-row chunk is better filled:
+//     4 units an SM 34.3 against 45.4 (489 rows), 48: 355.7 against 367.8
+//     (521 rows); 3 units an SM 34.9 against 30.2, which stay with pairs, and
+//     6: 43.3 against 41.7 (389 rows), which do too.
+bool chunk_wide(const kvr_cache *c, int n_max, int per, bool rkv, int *groups,
+                int *stages) {
+  const size_t limit = (size_t)c->smem_optin - 512;
+  *groups = per <= 1 ? 1 : 2;
+  *stages = per <= 1 ? 3 : 2;
+  if (kvr::chunk_smem_bytes(n_max, *groups, *stages, 4, rkv) > limit)
+    return false;
+  if (per <= 2) return true;
+  if (kvr::chunk_smem_bytes(n_max, 4, 2, 2, rkv) <= limit) return false;
+  const int two = 2 * ((per + 1) / 2), three = 3 * ((per + 2) / 3);
+  return n_max > (rkv ? 480 : 416) ? two <= three : 51 * two <= 50 * three;
+}
+
+// Consumer groups, ring stages per group and warps a group of the chunked
+// kernel for `units` jobs of up to n_max rows: groups of four warps
+// (chunk_wide), or the first of (4,2) (3,3) (3,2) (2,3) (2,2) (1,3) (1,2)
+// with two warps that fits in shared memory (more groups first: measured), or
+// the tuned choice.
+bool chunk_config(const kvr_cache *c, int n_max, int units,
+                  kvr::ChunkParams *p) {
   static const int order[7][2] = {{4, 2}, {3, 3}, {3, 2}, {2, 3},
                                   {2, 2}, {1, 3}, {1, 2}};
   const size_t limit = (size_t)c->smem_optin - 512;
   const int tg = c->chunk_groups, ts = c->chunk_stages;
+  const bool rkv = p->rkv != 0;
+  const int per = (units + c->sm_count - 1) / c->sm_count;
+  p->warps = 4;
+  if (!p->fork && tg <= 0 && ts <= 0 &&
+      chunk_wide(c, n_max, per, rkv, &p->n_groups, &p->n_stages))
+    return true;
+  p->warps = 2;
   for (const auto &o : order) {
     const int g = tg > 0 ? tg : o[0], s = ts > 0 ? ts : o[1];
     if (g > kvr::chunk_max_groups() || s > kvr::chunk_max_stages()) continue;
-    if (kvr::chunk_smem_bytes(n_max, g, s, rkv) <= limit) {
-      *groups = g;
-      *stages = s;
+    if (kvr::chunk_smem_bytes(n_max, g, s, 2, rkv) <= limit) {
+      p->n_groups = g;
+      p->n_stages = s;
       return true;
     }
   }
@@ -473,13 +507,13 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
     return false;
   if (!device_facts(c)) return false;
   kvr::ChunkParams p{};
-  if (!chunk_config(c, a.max_rows, &p.n_groups, &p.n_stages, rkv)) return false;
+  p.rkv = rkv ? 1 : 0;
+  p.lam = lam;
+  if (!chunk_config(c, a.max_rows, v.S * a.nl * v.H, &p)) return false;
   const std::pair<CUtensorMap, CUtensorMap> *maps =
       slab_maps(c, kvr::chunk_box_rows());
   if (!maps) return false;
   p.c = v;
-  p.rkv = rkv ? 1 : 0;
-  p.lam = lam;
   p.fork = 0;
   p.q = static_cast<const __nv_bfloat16 *>(a.q);
   p.k_new = static_cast<const __nv_bfloat16 *>(a.k_new);
@@ -1510,10 +1544,11 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr &&
       (maps128 = slab_maps(p, kvr::fork_batch_prefix_box_rows())) != nullptr;
   kvr::ChunkParams cp{};
+  cp.fork = 1;
   const bool chunk_ok = !batch_ok && !tile_ok && (want == 0 || want == 2) &&
       p->fused && p->chunk_groups >= 0 && f->tail_maps && pv.G <= 8 &&
       n_max <= kvr::chunk_max_rows() && device_facts(p) &&
-      chunk_config(p, n_max, &cp.n_groups, &cp.n_stages) &&
+      chunk_config(p, n_max, 0, &cp) &&
       (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
       aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr;

@@ -1,5 +1,5 @@
-// kvr_chunked.cu -- the persistent decode step for units streamed in 32-row
-// chunks: units longer than the staged kernel of kvr_fused.cu takes (the
+// kvr_chunked.cu -- the persistent decode step for units streamed in 32-
+// or 64-row chunks: units longer than the staged kernel of kvr_fused.cu takes (the
 // B = 128..512 sweep), and the candidate-batched step of stepwise best-of-N
 // (Sec. 2.2 Eq. 2), where a job is one candidate of one unit and its rows are
 // the parent's live rows (a shared, read-only prefix) followed by the
@@ -11,12 +11,18 @@
 //
 // Design (GB300, sm_103a):
 //  - Persistent CTAs, one per SM.  A CTA runs n_groups independent consumer
-//    groups of two warps, each with its own ring of n_stages chunk stages and
-//    its own producer warp, so no group ever waits for another group's rows.
+//    groups of two warps (or four), each with its own ring of n_stages chunk
+//    stages and its own producer warp, so no group ever waits for another
+//    group's rows.  A unit is a serial chain of chunks, and at 520 rows a
+//    group's area (logits of every row) leaves room for three pairs only, six
+//    consumer warps: the chain, not the bytes, is what bounds the step.  Two
+//    groups of four warps put eight to work and halve the chain: 64 sequences
+//    of 7B, 521-row units, 366 us (5.6 TB/s) with three pairs, 354 (5.8) with
+//    two groups of four; 56 units of 521 rows 20.6 and 16.5.
 //  - A job's rows are segment A (plain units: none; candidates: the prefix,
 //    from the parent slab) then segment B (the unit's rows, or the
 //    candidate's tail) then the new row.  Each segment streams in chunks of
-//    32 rows, loaded by TMA as 16-row 128B-swizzled boxes (so at most 15
+//    32 rows (64 for four warps), loaded by TMA as 16-row 128B-swizzled boxes (so at most 15
 //    rows past a segment's end are read); the new row is inserted into the
 //    last chunk of B from the inputs.  The producer warp's 32 lanes fetch the
 //    small inputs (query rows, new k/v row, old scores and positions of the
@@ -26,7 +32,7 @@
 //    bf16 mma.sync (m16n8k16, fp32 accumulate, P split hi + lo) with an
 //    online softmax across the job's chunks, and it keeps the scaled logits,
 //    old scores and positions of its rows in the group's area, then releases
-//    the stage.  After the last chunk the two warps merge their softmax
+//    the stage.  After the last chunk the warps merge their softmax
 //    states and partial outputs, compute every row's exact probability from
 //    the kept logits for the score update, agree on the evicted row, and
 //    write back.
@@ -36,7 +42,7 @@
 //    norm (the diagonal of the tile's Gram block), so that no key is read
 //    twice.  One more exchange of sums at the end of a job gives z.  Units
 //    with no current S get one from rkv_sum_kernel, launched before.  7B, 16
-//    sequences, 641-row units: 148 us against 113 for the plain step; the
+//    sequences, 641-row units: 145 us against 113 for the plain step; the
 //    separate eviction pass it replaces (two readings of the keys, a radix
 //    select) took 337 us after the 113.
 //  - Launched with programmatic stream serialization; every mbarrier wait is
@@ -72,11 +78,15 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   return d;
 }
 
-constexpr int kCR = 32;       // rows per chunk
 constexpr int kBox = 16;      // rows per TMA box (and per MMA tile)
-constexpr int kU = 2;         // consumer warps per group, one tile each
-static_assert(kU == 2, "the partial-output exchange pairs two warps");
 constexpr int kMaxGroups = 4;
+// U consumer warps a group (2, or 4 in at most kWideGroups groups), one tile of
+// every chunk each: a chunk is 16 U rows.
+constexpr int kWideGroups = 2;
+template <int U>
+__host__ __device__ constexpr int chunk_rows() {
+  return kBox * U;
+}
 constexpr int kMaxStages = 4; // per group
 constexpr int kQPitch = 272;  // bytes per staged query row (256 + 16 padding)
 constexpr int kMaxRowsChunk = 1024;
@@ -97,28 +107,31 @@ enum : int {
 enum : int { F_FIRST = 1, F_LAST = 2, F_NEW = 4, F_SKIP = 8 };
 
 // Byte offsets inside one stage.
+template <int U>
 struct ChunkStage {
-  static constexpr uint32_t k0 = 0, k1 = kCR * 128, v0 = 2 * kCR * 128,
-                            v1 = 3 * kCR * 128, q = 4 * kCR * 128,
+  static constexpr uint32_t rows = kBox * U, k0 = 0, k1 = rows * 128, v0 = 2 * rows * 128,
+                            v1 = 3 * rows * 128, q = 4 * rows * 128,
                             kn = q + 8 * kQPitch, vn = kn + 256, sc = vn + 256,
-                            ps = sc + 4 * kCR, hdr = ps + 4 * kCR,
+                            ps = sc + 4 * rows, hdr = ps + 4 * rows,
                             bytes = ((hdr + 4 * H_WORDS) + 1023) / 1024 * 1024,
                             // R-KV stages: the unit's kept key sum follows
                             rs = bytes, rkv_bytes = bytes + 1024;
 };
+template <int U>
 __host__ __device__ constexpr uint32_t stage_bytes(bool rkv) {
-  return rkv ? ChunkStage::rkv_bytes : ChunkStage::bytes;
+  return rkv ? ChunkStage<U>::rkv_bytes : ChunkStage<U>::bytes;
 }
 
 // Byte offsets inside one group's area (after the rings).
+template <int U>
 struct ChunkGroup {
   uint32_t xs, ox, lg, sc, ps, ns, bytes;
   __host__ __device__ explicit ChunkGroup(int n_max) {
     const int n = round_up16(n_max);
-    xs = 0;                      // [kU][5] 16-byte slots; R-KV: [kU] more
-    ox = 256;                    // [kU][4][32] float4 partial outputs: the
-                                 // 4 head-dim tiles the other warp owns
-    lg = ox + kU * 4 * 32 * 16;  // [n][8] scaled logits
+    xs = 0;                      // [U][5] 16-byte slots; R-KV: [U] more
+    ox = U == 2 ? 256 : 512;     // [U][4][32] float4 partial outputs: the
+                                 // 4 head-dim tiles that another warp takes
+    lg = ox + U * 4 * 32 * 16;   // [n][8] scaled logits
     sc = lg + n * 8 * 4;         // [n] old scores
     ps = sc + n * 4;             // [n] positions
     ns = ps + n * 4;             // [n] new scores (R-KV: mean cosines)
@@ -174,12 +187,14 @@ __device__ __forceinline__ void group_bar(int id, int threads) {
 }
 
 // Producer warp of one group: every chunk of the group's jobs, in order.
-template <bool kFork, bool kRkv>
+template <bool kFork, bool kRkv, int U>
 __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
                         const CUtensorMap *tmV, const CUtensorMap *tmTK,
                         const CUtensorMap *tmTV, unsigned char *ring,
                         uint64_t *full, uint64_t *empty, int g, int mine,
                         int lane, volatile int *abort, int *issued) {
+  using Stage = ChunkStage<U>;
+  constexpr int kCR = chunk_rows<U>();
   const CacheView &c = p.c;
   // Test hook: group 0 of CTA 0 never loads its first job (no copy is
   // issued, so there is nothing to drain); its consumers' wait runs out.
@@ -219,17 +234,17 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
         return;
       }
       __syncwarp();
-      unsigned char *st = ring + s * stage_bytes(kRkv);
+      unsigned char *st = ring + s * stage_bytes<U>(kRkv);
       const uint32_t s0 = smem_u32(st);
       const uint32_t bar = smem_u32(&full[s]);
       const bool segA = ci < cA;
-      const int first = 32 * (segA ? ci : ci - cA);  // row within the segment
+      const int first = kCR * (segA ? ci : ci - cA);  // row within the segment
       const int nseg = segA ? nA : nB;
       const int loaded = ok ? max(0, min(kCR, nseg - first)) : 0;
       const bool has_new = ok && !segA && nB - first < kCR;
       const int boxes = (loaded + kBox - 1) / kBox;
       if (lane == 0) {
-        int *h = reinterpret_cast<int *>(st + ChunkStage::hdr);
+        int *h = reinterpret_cast<int *>(st + Stage::hdr);
         h[H_JOB] = idx;
         h[H_BASE] = (segA ? 0 : nA) + first;
         h[H_VALID] = loaded + (has_new ? 1 : 0);
@@ -248,10 +263,10 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
         for (int bx = 0; bx < boxes; ++bx) {
           const int y = (int)(y0 + first + bx * kBox);
           const uint32_t off = bx * kBox * 128;
-          tma_load_2d(s0 + ChunkStage::k0 + off, mk, 0, y, bar);
-          tma_load_2d(s0 + ChunkStage::k1 + off, mk, 64, y, bar);
-          tma_load_2d(s0 + ChunkStage::v0 + off, mv, 0, y, bar);
-          tma_load_2d(s0 + ChunkStage::v1 + off, mv, 64, y, bar);
+          tma_load_2d(s0 + Stage::k0 + off, mk, 0, y, bar);
+          tma_load_2d(s0 + Stage::k1 + off, mk, 64, y, bar);
+          tma_load_2d(s0 + Stage::v0 + off, mv, 0, y, bar);
+          tma_load_2d(s0 + Stage::v1 + off, mv, 64, y, bar);
         }
       }
       if (ok) {
@@ -259,14 +274,14 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
           const unsigned char *q = reinterpret_cast<const unsigned char *>(
               p.q + jb.orow * c.G * 128);
           for (int i = lane; i < c.G * 16; i += 32)
-            cp_async16(s0 + ChunkStage::q + (i >> 4) * kQPitch + (i & 15) * 16,
+            cp_async16(s0 + Stage::q + (i >> 4) * kQPitch + (i & 15) * 16,
                        q + i * 16);
         }
         if (kRkv && ci == 0)  // the kept sum of the live rows' normalised keys
-          cp_async16(s0 + ChunkStage::rs + lane * 16,
+          cp_async16(s0 + Stage::rs + lane * 16,
                      c.rsum + jb.ug * 128 + lane * 4);
         if (has_new || (kRkv && ci == 0))
-          cp_async16(s0 + (lane < 16 ? ChunkStage::kn : ChunkStage::vn) +
+          cp_async16(s0 + (lane < 16 ? Stage::kn : Stage::vn) +
                          (lane & 15) * 16,
                      reinterpret_cast<const unsigned char *>(
                          (lane < 16 ? p.k_new : p.v_new) + jb.orow * 128) +
@@ -284,9 +299,9 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
         }
         const int pieces = (loaded + 3) / 4;
         if (lane < pieces)
-          cp_async16(s0 + ChunkStage::sc + lane * 16, sc + first + 4 * lane);
+          cp_async16(s0 + Stage::sc + lane * 16, sc + first + 4 * lane);
         else if (!kFork && lane >= 16 && lane - 16 < pieces)
-          cp_async16(s0 + ChunkStage::ps + (lane - 16) * 16,
+          cp_async16(s0 + Stage::ps + (lane - 16) * 16,
                      ps + first + 4 * (lane - 16));
       }
       cp_async_arrive_noinc(bar);
@@ -332,8 +347,8 @@ __global__ void __launch_bounds__(128) rkv_sum_kernel(CacheView c, int lb, int n
   }
 }
 
-template <bool kFork, bool kOutBf16, bool kRkv>
-__global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
+template <bool kFork, bool kOutBf16, bool kRkv, int U>
+__global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) * 32, 1)
     chunk_step_kernel(const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmTK,
@@ -344,7 +359,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   __shared__ __align__(8) uint64_t empty_bar[kMaxGroups][kMaxStages];
   __shared__ int issued_n[kMaxGroups], consumed_n[kMaxGroups];
   __shared__ volatile int s_abort;
-  __shared__ volatile int s_ok[kMaxGroups];
+  __shared__ volatile int s_ok[kMaxGroups][2];  // by chunk parity
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const CacheView &c = p.c;
@@ -354,10 +369,11 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   const int mine = (int)blockIdx.x < n_jobs
                        ? (n_jobs - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
                        : 0;
-  const int consumers = p.n_groups * kU;
-  const ChunkGroup GL(p.n_max);
+  const int consumers = p.n_groups * U;
+  const ChunkGroup<U> GL(p.n_max);
   static_assert(!(kFork && kRkv), "candidates evict at the commit");
-  constexpr uint32_t kStage = stage_bytes(kRkv);
+  using Stage = ChunkStage<U>;
+  constexpr uint32_t kStage = stage_bytes<U>(kRkv);
   const uint32_t ring_bytes = p.n_stages * kStage;
 
   if (threadIdx.x == 0) {
@@ -370,7 +386,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
     for (int g = 0; g < p.n_groups; ++g) {
       for (int s = 0; s < p.n_stages; ++s) {
         mbar_init(smem_u32(&full_bar[g][s]), 1 + 32);  // TMA + producer lanes
-        mbar_init(smem_u32(&empty_bar[g][s]), kU);
+        mbar_init(smem_u32(&empty_bar[g][s]), U);
       }
       issued_n[g] = 0;
       consumed_n[g] = 0;
@@ -385,7 +401,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
     const int g = st / p.n_stages, s = st % p.n_stages;
     if (r >= G * (kQPitch / 16))
       reinterpret_cast<int4 *>(smem + g * ring_bytes + s * kStage +
-                               ChunkStage::q)[r] = make_int4(0, 0, 0, 0);
+                               Stage::q)[r] = make_int4(0, 0, 0, 0);
   }
   fence_proxy_async();
   __syncthreads();
@@ -394,11 +410,11 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   if (warp >= consumers) {
     const int g = warp - consumers;
     if (g < p.n_groups)
-      produce<kFork, kRkv>(p, &tmK, &tmV, &tmTK, &tmTV, smem + g * ring_bytes,
+      produce<kFork, kRkv, U>(p, &tmK, &tmV, &tmTK, &tmTV, smem + g * ring_bytes,
                      full_bar[g], empty_bar[g], g, mine, lane, &s_abort,
                      &issued_n[g]);
   } else {
-    const int g = warp / kU, w = warp % kU, bar_id = 1 + g;
+    const int g = warp / U, w = warp % U, bar_id = 1 + g;
     unsigned char *ring = smem + g * ring_bytes;
     unsigned char *ga =
         smem + p.n_groups * ring_bytes + g * GL.bytes;
@@ -427,25 +443,26 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
       for (;;) {
         const int s = seq % p.n_stages;
         const uint32_t ph = (uint32_t)(seq / p.n_stages) & 1u;
-        // One warp waits (bounded) and tells the group, so that both warps
-        // take the same branch before the group's next barrier.
+        // One warp waits (bounded) and tells the group, so that all its warps
+        // take the same branch before the group's next barrier (by parity: the
+        // word is not written again before every warp has read it).
         if (w == 0 && lane == 0) {
           const bool ok =
               mbar_wait(smem_u32(&full_bar[g][s]), ph, &s_abort, c.wait_ns);
-          s_ok[g] = ok ? 1 : 0;
+          s_ok[g][seq & 1] = ok ? 1 : 0;
           if (!ok) {
             atomicOr(c.err, ERR_TIMEOUT);
             s_abort = 1;
           }
         }
-        group_bar(bar_id, 32 * kU);
-        if (!s_ok[g]) {
+        group_bar(bar_id, 32 * U);
+        if (!s_ok[g][seq & 1]) {
           stop = true;
           break;
         }
         mbar_try_wait(smem_u32(&full_bar[g][s]), ph);  // acquire for this thread
         unsigned char *st = ring + s * kStage;
-        const int *h = reinterpret_cast<const int *>(st + ChunkStage::hdr);
+        const int *h = reinterpret_cast<const int *>(st + Stage::hdr);
         const int flags = h[H_FLAGS], base = h[H_BASE], valid = h[H_VALID];
         const int loaded = h[H_LOADED];
         if (flags & F_FIRST) {
@@ -453,7 +470,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           t = h[H_T];
           ntot = h[H_NTOT];
           nA = h[H_NA];
-          const uint32_t qa = smem_u32(st + ChunkStage::q) +
+          const uint32_t qa = smem_u32(st + Stage::q) +
                               (lane & 7) * kQPitch + (lane >> 3) * 16;
 #pragma unroll
           for (int i = 0; i < 4; ++i)
@@ -463,9 +480,9 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
         skip = (flags & F_SKIP) != 0;
         if constexpr (kRkv) {
           if ((flags & F_FIRST) && !skip) {
-            const float4 rs = reinterpret_cast<const float4 *>(st + ChunkStage::rs)[lane];
+            const float4 rs = reinterpret_cast<const float4 *>(st + Stage::rs)[lane];
             float kn[4];
-            key4(st + ChunkStage::kn, lane, kn);
+            key4(st + Stage::kn, lane, kn);
             const float inv = inv_norm(kn);
             S4[0] = fmaf(kn[0], inv, rs.x);
             S4[1] = fmaf(kn[1], inv, rs.y);
@@ -486,20 +503,20 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
             __syncwarp();
           }
         }
-        unsigned char *K0 = st + ChunkStage::k0, *K1 = st + ChunkStage::k1;
-        unsigned char *V0 = st + ChunkStage::v0, *V1 = st + ChunkStage::v1;
+        unsigned char *K0 = st + Stage::k0, *K1 = st + Stage::k1;
+        unsigned char *V0 = st + Stage::v0, *V1 = st + Stage::v1;
         const int tr0 = kBox * w;
         bool wrote = false;  // generic-proxy writes to the stage
         if (!skip && (flags & F_NEW) && w == 0)
           nrow = *reinterpret_cast<const int4 *>(
-              st + (lane < 16 ? ChunkStage::kn : ChunkStage::vn) + (lane & 15) * 16);
+              st + (lane < 16 ? Stage::kn : Stage::vn) + (lane & 15) * 16);
         if (!skip && tr0 < valid) {
           // New row (from the inputs) and zero V past the live rows.
           if ((flags & F_NEW) && h[H_NEWROW] >= tr0 && h[H_NEWROW] < tr0 + kBox) {
             const int rn = h[H_NEWROW];
             const int ch = lane & 15, half = ch >> 3, cc = ch & 7;
             unsigned char *dst = lane < 16 ? (half ? K1 : K0) : (half ? V1 : V0);
-            const unsigned char *src = st + (lane < 16 ? ChunkStage::kn : ChunkStage::vn);
+            const unsigned char *src = st + (lane < 16 ? Stage::kn : Stage::vn);
             *reinterpret_cast<int4 *>(dst + rn * 128 + ((cc ^ (rn & 7)) << 4)) =
                 *reinterpret_cast<const int4 *>(src + ch * 16);
             wrote = true;
@@ -514,8 +531,8 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           if (lane < kBox) {
             const int r = tr0 + lane;
             if (r < loaded) {
-              GSC[base + r] = reinterpret_cast<const float *>(st + ChunkStage::sc)[r];
-              GPS[base + r] = reinterpret_cast<const int32_t *>(st + ChunkStage::ps)[r];
+              GSC[base + r] = reinterpret_cast<const float *>(st + Stage::sc)[r];
+              GPS[base + r] = reinterpret_cast<const int32_t *>(st + Stage::ps)[r];
             } else if (r < valid) {  // the new row
               GSC[base + r] = 0.f;
               GPS[base + r] = t;
@@ -638,31 +655,33 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
         l1 += __shfl_xor_sync(0xffffffffu, l1, off);
       }
       if (lane < 4) XS4[w * 5 + lane] = make_float4(m0, m1, l0, l1);
-      // The partials of the head-dim tiles the other warp owns (mt of the
-      // other parity); each warp keeps its own tiles' partials in registers.
+      // U == 2: the partials of the head-dim tiles the other warp owns (mt of
+      // the other parity); each warp keeps its own tiles' partials in registers.
+      if constexpr (U == 2) {
 #pragma unroll
-      for (int mt = 0; mt < 8; ++mt)
-        if ((mt & 1) != w)
-          OX[(w * 4 + (mt >> 1)) * 32 + lane] =
-              make_float4(o[mt][0], o[mt][1], o[mt][2], o[mt][3]);
-      group_bar(bar_id, 32 * kU);
+        for (int mt = 0; mt < 8; ++mt)
+          if ((mt & 1) != w)
+            OX[(w * 4 + (mt >> 1)) * 32 + lane] =
+                make_float4(o[mt][0], o[mt][1], o[mt][2], o[mt][3]);
+      }
+      group_bar(bar_id, 32 * U);
       // Per head: the merged maximum and 1 / sum, for all 8 heads (the
       // scores need every head) and the warps' rescale factors for this
       // lane's heads c2, c2 + 1.
-      float Mh[8], iZ[8], fv0[kU], fv1[kU];
+      float Mh[8], iZ[8], fv0[U], fv1[U];
 #pragma unroll
       for (int cp = 0; cp < 4; ++cp) {
-        float4 r[kU];
+        float4 r[U];
         float Ma = -INFINITY, Mb = -INFINITY;
 #pragma unroll
-        for (int v = 0; v < kU; ++v) {
+        for (int v = 0; v < U; ++v) {
           r[v] = XS4[v * 5 + cp];
           if (r[v].z > 0.f) Ma = fmaxf(Ma, r[v].x);
           if (r[v].w > 0.f) Mb = fmaxf(Mb, r[v].y);
         }
-        float Za = 0.f, Zb = 0.f, ea[kU], eb[kU];
+        float Za = 0.f, Zb = 0.f, ea[U], eb[U];
 #pragma unroll
-        for (int v = 0; v < kU; ++v) {
+        for (int v = 0; v < U; ++v) {
           ea[v] = r[v].z > 0.f ? ex2(r[v].x - Ma) : 0.f;
           eb[v] = r[v].w > 0.f ? ex2(r[v].y - Mb) : 0.f;
           Za += r[v].z * ea[v];
@@ -675,7 +694,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
         iZ[2 * cp + 1] = ib;
         if (cp == (lane & 3)) {
 #pragma unroll
-          for (int v = 0; v < kU; ++v) {
+          for (int v = 0; v < U; ++v) {
             fv0[v] = ea[v] * ia;
             fv1[v] = eb[v] * ib;
           }
@@ -685,26 +704,12 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           atomicOr(c.err, ERR_NONFINITE);
       }
       const Job jb = job_of(p, idx);
-      // Output: warp w owns head-dim tiles of parity w; the two warps'
-      // terms are added in warp order.
+      // Output.
       {
         constexpr int osz = kOutBf16 ? 2 : 4;
         unsigned char *gout = reinterpret_cast<unsigned char *>(p.out) +
                               jb.orow * G * 128 * osz;
-#pragma unroll
-        for (int mt = 0; mt < 8; ++mt) {
-          if ((mt & 1) != w) continue;
-          const float4 mine = make_float4(o[mt][0], o[mt][1], o[mt][2], o[mt][3]);
-          const float4 other = OX[((1 - w) * 4 + (mt >> 1)) * 32 + lane];
-          float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
-#pragma unroll
-          for (int v = 0; v < kU; ++v) {
-            const float4 x = v == w ? mine : other;
-            e0 += x.x * fv0[v];
-            e1 += x.y * fv1[v];
-            e2 += x.z * fv0[v];
-            e3 += x.w * fv1[v];
-          }
+        auto put = [&](int mt, float e0, float e1, float e2, float e3) {
           if (kOutBf16) {
             const uint32_t lo = movm_t(pack_bf16(e0, e1));
             const uint32_t hi = movm_t(pack_bf16(e2, e3));
@@ -725,6 +730,67 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
               of[(c2 + 1) * 128 + d0 + 8] = e3;
             }
           }
+        };
+        if constexpr (U == 2) {
+          // Warp w owns head-dim tiles of parity w; the two warps' terms are
+          // added in warp order.
+#pragma unroll
+          for (int mt = 0; mt < 8; ++mt) {
+            if ((mt & 1) != w) continue;
+            const float4 mine = make_float4(o[mt][0], o[mt][1], o[mt][2], o[mt][3]);
+            const float4 other = OX[((1 - w) * 4 + (mt >> 1)) * 32 + lane];
+            float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+              const float4 x = v == w ? mine : other;
+              e0 += x.x * fv0[v];
+              e1 += x.y * fv1[v];
+              e2 += x.z * fv0[v];
+              e3 += x.w * fv1[v];
+            }
+            put(mt, e0, e1, e2, e3);
+          }
+        } else {
+          // Each warp's partials at the common scale, then added over the
+          // pairs (w, w ^ 1), which halves the tiles a warp holds, and over
+          // the pairs (w, w ^ 2), which halves them again: warp w ends with
+          // tiles mt of parity w & 1 and bit 1 of mt equal to w >> 1.
+          float s0 = fv0[0], s1 = fv1[0];
+#pragma unroll
+          for (int v = 1; v < U; ++v) {
+            s0 = v == w ? fv0[v] : s0;
+            s1 = v == w ? fv1[v] : s1;
+          }
+          const bool odd = (w & 1) != 0, up = (w & 2) != 0;
+          float4 keep[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float4 a = make_float4(o[2 * x][0] * s0, o[2 * x][1] * s1, o[2 * x][2] * s0,
+                                         o[2 * x][3] * s1);
+            const float4 b = make_float4(o[2 * x + 1][0] * s0, o[2 * x + 1][1] * s1,
+                                         o[2 * x + 1][2] * s0, o[2 * x + 1][3] * s1);
+            keep[x] = odd ? b : a;
+            OX[(w * 4 + x) * 32 + lane] = odd ? a : b;
+          }
+          group_bar(bar_id, 32 * U);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float4 y = OX[((w ^ 1) * 4 + x) * 32 + lane];
+            keep[x] = make_float4(keep[x].x + y.x, keep[x].y + y.y, keep[x].z + y.z,
+                                  keep[x].w + y.w);
+          }
+          group_bar(bar_id, 32 * U);
+          // keep[x] is tile 2 x + odd: bit 1 of the tile is x & 1.
+#pragma unroll
+          for (int x = 0; x < 2; ++x)
+            OX[(w * 4 + x) * 32 + lane] = up ? keep[2 * x] : keep[2 * x + 1];
+          group_bar(bar_id, 32 * U);
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const float4 y = OX[((w ^ 2) * 4 + x) * 32 + lane];
+            const float4 m = up ? keep[2 * x + 1] : keep[2 * x];
+            put(4 * x + (up ? 2 : 0) + (odd ? 1 : 0), m.x + y.x, m.y + y.y, m.z + y.z, m.w + y.w);
+          }
         }
       }
       // Accumulated attention of every row from the kept logits; the
@@ -735,7 +801,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
       unsigned long long best = ~0ull;
       int bi = -1;
       float ssum = 0.f, esum = 0.f;
-      for (int r = tid; r < ntot; r += 32 * kU) {
+      for (int r = tid; r < ntot; r += 32 * U) {
         const float4 la = *reinterpret_cast<const float4 *>(LG + r * 8);
         const float4 lb = *reinterpret_cast<const float4 *>(LG + r * 8 + 4);
         const float lg8[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
@@ -775,13 +841,18 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
             ssum += __shfl_xor_sync(0xffffffffu, ssum, o2);
             esum += __shfl_xor_sync(0xffffffffu, esum, o2);
           }
-          if (lane == 0) XS4[kU * 5 + w] = make_float4(ssum, esum, 0.f, 0.f);
-          group_bar(bar_id, 32 * kU);
-          const float4 x0 = XS4[kU * 5], x1 = XS4[kU * 5 + 1];
-          const float ss = x0.x + x1.x;
+          if (lane == 0) XS4[U * 5 + w] = make_float4(ssum, esum, 0.f, 0.f);
+          group_bar(bar_id, 32 * U);
+          float ss = 0.f, es = 0.f;
+#pragma unroll
+          for (int v = 0; v < U; ++v) {
+            const float4 x = XS4[U * 5 + v];
+            ss += x.x;
+            es += x.y;
+          }
           const float ci = ss > 0.f ? p.lam / ss : 0.f;
-          const float cr = (1.f - p.lam) / (x0.y + x1.y);
-          for (int r = tid; r < ntot; r += 32 * kU) {
+          const float cr = (1.f - p.lam) / es;
+          for (int r = tid; r < ntot; r += 32 * U) {
             const int pr = GPS[r];
             if (pr <= wlo) {
               const unsigned long long key =
@@ -810,11 +881,11 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           XW[w * 5 + 4] = make_uint4((uint32_t)best, (uint32_t)(best >> 32),
                                      (uint32_t)bi, 0u);
       }
-      group_bar(bar_id, 32 * kU);  // new scores (and candidates) visible
+      group_bar(bar_id, 32 * U);  // new scores (and candidates) visible
       if (evict) {
         const uint4 *XW = reinterpret_cast<const uint4 *>(XS4);
 #pragma unroll
-        for (int v = 0; v < kU; ++v) {
+        for (int v = 0; v < U; ++v) {
           const uint4 a = XW[v * 5 + 4];
           const unsigned long long kb = ((unsigned long long)a.y << 32) | a.x;
           if (kb < best) {
@@ -829,7 +900,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
         const int nt = ntot - 1 - nA;  // tail rows before the append
         float *ps = p.f.pscore + jb.cu * c.sstride;
         float *ts = p.f.tscore + jb.cu * p.f.tstride;
-        for (int r = tid; r < ntot; r += 32 * kU) {
+        for (int r = tid; r < ntot; r += 32 * U) {
           if (r < nA) ps[r] = GNS[r];
           else ts[r - nA] = GNS[r];
         }
@@ -852,7 +923,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           vk = reinterpret_cast<const uint2 *>(
               reinterpret_cast<const __nv_bfloat16 *>(c.K) +
               (jb.ug * (size_t)c.cap + victim) * 128)[lane];
-        for (int r = tid; r < m; r += 32 * kU)
+        for (int r = tid; r < m; r += 32 * U)
           gsc[r] = r == victim ? NS[m] : NS[r];
         const int slot = victim < 0 ? m : (victim < m ? victim : -1);
         if (kRkv && w == 0) {
@@ -892,7 +963,7 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
           }
         }
       }
-      group_bar(bar_id, 32 * kU);  // the group area is free for the next job
+      group_bar(bar_id, 32 * U);  // the group area is free for the next job
     }
   }
   __syncthreads();
@@ -906,17 +977,17 @@ __global__ void __launch_bounds__(kMaxGroups * (kU + 1) * 32, 1)
   }
 }
 
-template <bool kFork, bool kRkv>
+template <bool kFork, bool kRkv, int U>
 cudaError_t launch_k(const CUtensorMap &tmK, const CUtensorMap &tmV,
                      const CUtensorMap &tmTK, const CUtensorMap &tmTV,
                      const ChunkParams &p, int grid, size_t smem,
                      cudaStream_t st) {
-  auto kern = p.c.out_bf16 ? chunk_step_kernel<kFork, true, kRkv>
-                           : chunk_step_kernel<kFork, false, kRkv>;
+  auto kern = p.c.out_bf16 ? chunk_step_kernel<kFork, true, kRkv, U>
+                           : chunk_step_kernel<kFork, false, kRkv, U>;
   cudaError_t e = cudaFuncSetAttribute(
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(grid), dim3(32 * p.n_groups * (kU + 1)), smem,
+  return launch_pdl(kern, dim3(grid), dim3(32 * p.n_groups * (U + 1)), smem,
                     st, tmK, tmV, tmTK, tmTV, p);
 }
 
@@ -926,32 +997,36 @@ int chunk_box_rows() { return kBox; }
 int chunk_max_rows() { return kMaxRowsChunk; }
 int chunk_max_groups() { return kMaxGroups; }
 int chunk_max_stages() { return kMaxStages; }
-size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, bool rkv) {
-  return (size_t)n_groups *
-             ((size_t)n_stages * stage_bytes(rkv) + ChunkGroup(n_max).bytes) +
-         1024;
+size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, int warps, bool rkv) {
+  const size_t one =
+      warps == 4 ? (size_t)n_stages * stage_bytes<4>(rkv) + ChunkGroup<4>(n_max).bytes
+                 : (size_t)n_stages * stage_bytes<2>(rkv) + ChunkGroup<2>(n_max).bytes;
+  return (size_t)n_groups * one + 1024;
 }
 
 cudaError_t launch_chunk_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                               const CUtensorMap *tmTK, const CUtensorMap *tmTV,
                               const ChunkParams &p, int grid,
                               cudaStream_t st) {
-  if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.n_stages < 2 ||
+  if ((p.warps != 2 && (p.warps != 4 || p.fork || p.n_groups > kWideGroups)) ||
+      p.n_groups < 1 || p.n_groups > kMaxGroups || p.n_stages < 2 ||
       p.n_stages > kMaxStages || p.n_max < 1 || p.n_max > kMaxRowsChunk ||
       p.c.G > 8 || (p.fork && (!tmTK || !tmTV || p.rkv)))
     return cudaErrorInvalidValue;
-  const size_t smem = chunk_smem_bytes(p.n_max, p.n_groups, p.n_stages, p.rkv != 0);
+  const size_t smem = chunk_smem_bytes(p.n_max, p.n_groups, p.n_stages, p.warps, p.rkv != 0);
   if (p.fork)
-    return launch_k<true, false>(tmK, tmV, *tmTK, *tmTV, p, grid, smem, st);
+    return launch_k<true, false, 2>(tmK, tmV, *tmTK, *tmTV, p, grid, smem, st);
   if (p.rkv) {
     // Units whose kept key sum another call has left stale, first.
     const int units = p.c.S * p.nl * p.c.H;
     const cudaError_t e =
         launch_pdl(rkv_sum_kernel, dim3(units), dim3(128), 0, st, p.c, p.lb, p.nl);
     if (e != cudaSuccess) return e;
-    return launch_k<false, true>(tmK, tmV, tmK, tmV, p, grid, smem, st);
+    return p.warps == 4 ? launch_k<false, true, 4>(tmK, tmV, tmK, tmV, p, grid, smem, st)
+                        : launch_k<false, true, 2>(tmK, tmV, tmK, tmV, p, grid, smem, st);
   }
-  return launch_k<false, false>(tmK, tmV, tmK, tmV, p, grid, smem, st);
+  return p.warps == 4 ? launch_k<false, false, 4>(tmK, tmV, tmK, tmV, p, grid, smem, st)
+                      : launch_k<false, false, 2>(tmK, tmV, tmK, tmV, p, grid, smem, st);
 }
 
 }  // namespace kvr

@@ -340,6 +340,7 @@ struct ChunkParams {
   int n_jobs;                  // S * nl * H, times N for candidates
   int n_max;                   // largest job (rows with the new row)
   int n_groups, n_stages;      // consumer groups; ring stages per group
+  int warps;                   // consumer warps a group: 2, or 4 (plain units)
   int budget, window, evict;
   float scale_log2e, inv_g;
   // R-KV eviction (App. C) instead of the accumulated-attention TopB, plain
@@ -352,7 +353,8 @@ int chunk_box_rows();
 int chunk_max_rows();
 int chunk_max_groups();
 int chunk_max_stages();
-size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, bool rkv = false);
+size_t chunk_smem_bytes(int n_max, int n_groups, int n_stages, int warps,
+                        bool rkv = false);
 cudaError_t launch_chunk_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                               const CUtensorMap *tmTK, const CUtensorMap *tmTV,
                               const ChunkParams &p, int grid, cudaStream_t st);
