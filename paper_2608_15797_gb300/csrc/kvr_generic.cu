@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T, int D, int NT, bool kByRank>
 __global__ void __launch_bounds__(NT)
     evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow, int max_list,
-                 int cached) {
+                 int cached, int max_rows) {
   pdl_begin();
   extern __shared__ int lists[];  // holes | movers [max_list each] | scores
   __shared__ unsigned s_wsum[NT / 32];
@@ -397,6 +397,12 @@ __global__ void __launch_bounds__(NT)
   const int n = c.state[4 * x.u] + grow;
   const int newest = c.state[4 * x.u + 1] + grow - 1;
   __syncthreads();
+  // Longer than the host thinks: the blocked absorb left such a unit alone, and
+  // an eviction has no room for its lists.
+  if (n < grow || n > (grow ? min(max_rows, c.cap) : max(max_rows, B + W))) {
+    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+    return;
+  }
   if (tid == 0 && grow) {
     c.state[4 * x.u] = n;
     c.state[4 * x.u + 1] = newest + 1;
@@ -562,7 +568,7 @@ cudaError_t evict_launch(const CacheView &c, int lb, int nl, int max_rows, int B
       kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(NT), bytes, st, c, lb, nl, B, W, grow,
-                    max_list, cached);
+                    max_list, cached, max_rows);
 }
 
 template <typename T, int D>
