@@ -174,6 +174,18 @@ def test_entropy_padded_and_unaligned_rows(dtype, stride):
     run_lockstep(8, 1000, 30, dtype, stride=stride)
 
 
+# Rows at every offset from a 16-byte boundary: shorter than the way to it, one
+# logit past it, a piece's vectors (16,384 bf16, 8,192 fp32 logits) exactly,
+# with a head and a tail, and one vector into the next piece; several pieces.
+@pytest.mark.parametrize("dtype,vocab,stride", [
+    ("bf16", 3, 3), ("bf16", 9, 9), ("bf16", 16384, 16385),
+    ("bf16", 16391, 16391), ("bf16", 16399, 16399), ("bf16", 50001, 50001),
+    ("f32", 2, 2), ("f32", 8192, 8195), ("f32", 8197, 8197),
+    ("f32", 25001, 25001)])
+def test_entropy_unaligned_row_vectors(dtype, vocab, stride):
+    run_lockstep(9, vocab, 26, dtype, stride=stride)
+
+
 def test_entropy_temperature_window_guard_variants():
     run_lockstep(8, 5000, 30, "bf16", window=1, guard=0, tau=6.5)
     run_lockstep(8, 5000, 30, "f32", window=64, guard=3, tau=7.5,
