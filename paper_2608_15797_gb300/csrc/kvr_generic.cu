@@ -16,7 +16,8 @@
 //   their rows: scores are kept in shared memory, the lists take two passes
 //   and one exchange of counts (448 units of 700 to 16,384 rows: 152 us with
 //   64-bit keys read from global memory eight times and block-wide list
-//   building, 55 now; 1,792 units of 697 rows: 96 and 62).
+//   building, 49 now; 1,792 units of 697 rows: 96 and 25, of which the moves,
+//   a warp a row with half its lanes idle, had taken 28 more).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -181,21 +182,30 @@ __device__ void compact_unit(const CacheView &c, size_t u, int n, int nk, Keep k
     om += __popc(bm);
   }
   __syncthreads();
-  // Move every survivor beyond nk into a freed slot below it (disjoint).
-  constexpr int kChunks = D * (int)sizeof(T) / 16;
-  for (int j = warp; j < nh; j += kNW) {
+  // Move every survivor beyond nk into a freed slot below it (disjoint), four
+  // 16-byte pieces a thread in flight.
+  for (int j = tid; j < nh; j += NT) {
     const int dst = holes[j], src = movers[j];
-    const int4 *ks = reinterpret_cast<const int4 *>(Ku + (size_t)src * D);
-    const int4 *vs = reinterpret_cast<const int4 *>(Vu + (size_t)src * D);
-    int4 *kd = reinterpret_cast<int4 *>(Ku + (size_t)dst * D);
-    int4 *vd = reinterpret_cast<int4 *>(Vu + (size_t)dst * D);
-    for (int q = lane; q < kChunks; q += 32) {
-      kd[q] = ks[q];
-      vd[q] = vs[q];
+    su[dst] = su[src];
+    pu[dst] = pu[src];
+  }
+  constexpr int kChunks = D * (int)sizeof(T) / 16, kAhead = 4;
+  const int pieces = nh * 2 * kChunks;  // of a row's K, then of its V
+  for (int i0 = tid; i0 < pieces; i0 += kAhead * NT) {
+    int4 v[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      const int i = i0 + k * NT;
+      if (i < pieces)
+        v[k] = reinterpret_cast<const int4 *>(
+            ((i / kChunks) & 1 ? Vu : Ku) + (size_t)movers[i / (2 * kChunks)] * D)[i % kChunks];
     }
-    if (lane == 0) {
-      su[dst] = su[src];
-      pu[dst] = pu[src];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      const int i = i0 + k * NT;
+      if (i < pieces)
+        reinterpret_cast<int4 *>(((i / kChunks) & 1 ? Vu : Ku) +
+                                 (size_t)holes[i / (2 * kChunks)] * D)[i % kChunks] = v[k];
     }
   }
   if (tid == 0) {
