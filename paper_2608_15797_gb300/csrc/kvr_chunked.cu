@@ -224,7 +224,7 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
       const uint32_t ph = (uint32_t)(seq / p.n_stages) & 1u;
       int got = 1;
       if (lane == 0)
-        got = mbar_wait(smem_u32(&empty[s]), ph ^ 1u, abort, c.wait_ns);
+        got = mbar_wait_idle(smem_u32(&empty[s]), ph ^ 1u, abort, c.wait_ns);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (!got) {
         if (lane == 0) {
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
         // word is not written again before every warp has read it).
         if (w == 0 && lane == 0) {
           const bool ok =
-              mbar_wait(smem_u32(&full_bar[g][s]), ph, &s_abort, c.wait_ns);
+              mbar_wait_idle(smem_u32(&full_bar[g][s]), ph, &s_abort, c.wait_ns);
           s_ok[g][seq & 1] = ok ? 1 : 0;
           if (!ok) {
             atomicOr(c.err, ERR_TIMEOUT);
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
     volatile int never = 0;
     for (int g = 0; g < p.n_groups; ++g)
       for (int q = consumed_n[g]; q < issued_n[g]; ++q)
-        mbar_wait(smem_u32(&full_bar[g][q % p.n_stages]),
+        mbar_wait_idle(smem_u32(&full_bar[g][q % p.n_stages]),
                   (uint32_t)(q / p.n_stages) & 1u, &never);
   }
 }

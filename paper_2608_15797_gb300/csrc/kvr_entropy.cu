@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(kSThreads, 3)
           const int n = min(left, kStageVecs);
           const int st = q % kSStages;
           const uint32_t ph = static_cast<uint32_t>(q / kSStages) & 1u;
-          if (!mbar_wait(smem_u32(&empty[st]), ph ^ 1u, abort)) {
+          if (!mbar_wait_idle(smem_u32(&empty[st]), ph ^ 1u, abort)) {
             atomicOr(v.err, kvr::ERR_TIMEOUT);
             *abort = 1;
             ok = false;
@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kSThreads, 3)
       if (ok) {  // terminator: a stage with no data
         const int st = q % kSStages;
         const uint32_t ph = static_cast<uint32_t>(q / kSStages) & 1u;
-        if (mbar_wait(smem_u32(&empty[st]), ph ^ 1u, abort)) {
+        if (mbar_wait_idle(smem_u32(&empty[st]), ph ^ 1u, abort)) {
           hdr[st] = make_int4(0, 0, 0, F_DONE);
           mbar_arrive(smem_u32(&full[st]));
         } else {
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(kSThreads, 3)
       const int st = q % kSStages;
       const uint32_t ph = static_cast<uint32_t>(q / kSStages) & 1u;
       int got = 1;
-      if (lane == 0) got = mbar_wait(smem_u32(&full[st]), ph, abort);
+      if (lane == 0) got = mbar_wait_idle(smem_u32(&full[st]), ph, abort);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (!got) {
         if (lane == 0) {
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kSThreads, 3)
   if (s_abort && tid == 0) {
     volatile int never = 0;
     for (int q = s_waited; q < s_issued; ++q)
-      mbar_wait(smem_u32(&full[q % kSStages]),
+      mbar_wait_idle(smem_u32(&full[q % kSStages]),
                 static_cast<uint32_t>(q / kSStages) & 1u, &never);
   }
 }

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kThr, 2)
   volatile int *abort = &s_abort;
   // A whole warp's bounded wait for completion n of a barrier.
   auto wait_warp = [&](uint64_t &bar, int n) {
-    return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar), (uint32_t)(n & 1), abort)) != 0;
+    return __all_sync(0xffffffffu, mbar_wait_idle(smem_u32(&bar), (uint32_t)(n & 1), abort)) != 0;
   };
   if (warp == 8) tmem_alloc(smem_u32(&s_tmem), kCols);
   if (tid == 0) {
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kThr, 2)
       auto load_block = [&](bool kbuf, bool k, const TileUnit &u, int j) {
         int &n = kbuf ? nk : nv;
         if (n > 0)
-          ok = mbar_wait(smem_u32(kbuf ? &b_kfree : &b_vfree), (uint32_t)((n - 1) & 1), abort);
+          ok = mbar_wait_idle(smem_u32(kbuf ? &b_kfree : &b_vfree), (uint32_t)((n - 1) & 1), abort);
         if (!ok) return;
         ++n;
         const uint32_t bar = smem_u32(kbuf ? &b_kfull : &b_vfull), dst = kbuf ? aK : aV;
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThr, 2)
       auto load_q = [&](int i) {
         if (q_unit >= i) return;
         const int b = nq & 1;
-        if (nq > 1) ok = mbar_wait(smem_u32(&b_qfree[b]), (uint32_t)((nq / 2 - 1) & 1), abort);
+        if (nq > 1) ok = mbar_wait_idle(smem_u32(&b_qfree[b]), (uint32_t)((nq / 2 - 1) & 1), abort);
         if (!ok) return;
         const uint32_t bar = smem_u32(&b_qfull[b]), st = smem_u32(stage) + b * kNew;
         mbar_expect_tx(bar, q_bytes);
@@ -218,9 +218,9 @@ __global__ void __launch_bounds__(kThr, 2)
       // (bounded) before the CTA's shared memory is given back.
       volatile int never = 0;
       for (int k = max(0, nq - 2); k < nq; ++k)
-        mbar_wait(smem_u32(&b_qfull[k & 1]), (uint32_t)((k / 2) & 1), &never);
-      if (nk) mbar_wait(smem_u32(&b_kfull), (uint32_t)((nk - 1) & 1), &never);
-      if (nv) mbar_wait(smem_u32(&b_vfull), (uint32_t)((nv - 1) & 1), &never);
+        mbar_wait_idle(smem_u32(&b_qfull[k & 1]), (uint32_t)((k / 2) & 1), &never);
+      if (nk) mbar_wait_idle(smem_u32(&b_kfull), (uint32_t)((nk - 1) & 1), &never);
+      if (nv) mbar_wait_idle(smem_u32(&b_vfull), (uint32_t)((nv - 1) & 1), &never);
     }
   } else if (warp == 9) {
     // Issuer (one thread's MMAs run in the order of issue; see
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kThr, 2)
       // Every MMA issued has completed before TMEM is freed.
       volatile int never = 0;
       tc_commit(smem_u32(&b_drain));
-      mbar_wait(smem_u32(&b_drain), 0, &never);
+      mbar_wait_idle(smem_u32(&b_drain), 0, &never);
     }
   } else {
     // Softmax: warps wq and wq + 4 share lanes 32 wq .. 32 wq + 31, candidates

@@ -41,6 +41,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same, with the thread suspended for up to `ns` until the phase ends.
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity, uint32_t ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(ns)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -54,6 +66,24 @@ __device__ inline bool mbar_wait(uint32_t bar, uint32_t parity,
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   while (!mbar_try_wait(bar, parity)) {
+    if (*abort || global_ns() - t0 > limit_ns) return false;
+  }
+  return true;
+}
+// The same with suspended tries instead of polls a clock reading apart.  What
+// polls takes issue slots from the warps that work: with tries one right after
+// the other the 64-token absorb went from 878 us to 1,122.  Suspended tries
+// are the better ones where groups or units wait on rings of their own (7B,
+// 64 sequences of 521 rows 354.4 -> 352.6 us, R-KV 146.7 -> 145.5, the
+// candidate tiles 1,698 -> 1,686 a pass, the entropy test 34.2 -> 34.1), the
+// readings in the split step (1,053 against 1,061) and the 64-token absorb
+// (877 against 882).
+__device__ inline bool mbar_wait_idle(uint32_t bar, uint32_t parity, volatile int *abort,
+                                      uint64_t limit_ns = kWaitNs) {
+  constexpr uint32_t kTryNs = 10000;
+  if (mbar_try_wait(bar, parity, kTryNs)) return true;
+  const uint64_t t0 = global_ns();
+  while (!mbar_try_wait(bar, parity, kTryNs)) {
     if (*abort || global_ns() - t0 > limit_ns) return false;
   }
   return true;
