@@ -16,8 +16,8 @@
 //   their rows: scores are kept in shared memory, the lists take two passes
 //   and one exchange of counts (448 units of 700 to 16,384 rows: 152 us with
 //   64-bit keys read from global memory eight times and block-wide list
-//   building, 49 now; 1,792 units of 697 rows: 96 and 25, of which the moves,
-//   a warp a row with half its lanes idle, had taken 28 more).
+//   building, 47 now; 1,792 units of 697 rows: 96 and 33, and 54 when a warp
+//   moved one row at a time with half its lanes idle).
 #include <cuda_bf16.h>
 #include <math.h>
 
