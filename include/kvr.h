@@ -475,9 +475,12 @@ kvr_status kvr_cache_set_absorb_kernel(kvr_cache *cache, int kernel);
 
 /* How the cache's last kvr_absorb_chunk ran: 0 = the tensor-memory kernel,
  * 1 = the mma.sync kernel, 2 = token by token, 3 = in blocks on the tensor
- * cores (four launches; any chunk and unit length, bf16 in and out, head_dim
- * 128, G <= 8, 16-byte aligned tensors); -1 before the first call (or for
- * NULL).  Host state only: no synchronisation. */
+ * cores (four launches, six where rows are evicted; any chunk and unit
+ * length, bf16 in and out, head_dim 128, G <= 8, 16-byte aligned tensors); -1
+ * before the first call (or for NULL).  From one state, 2 and 3 retain the
+ * same rows in the same slots: 3 settles near ties of the scores as 2 would
+ * (up to 96 rows of a unit, units of up to 50 K / G rows).  Host state only:
+ * no synchronisation. */
 int kvr_cache_last_absorb_kernel(const kvr_cache *cache);
 
 /* ---- the same step for callers that cannot allocate -------------------- */

@@ -8,7 +8,7 @@
 // The work is a contraction: C tokens x G heads against m + C rows, causal.
 // Run token by token it was one launch a token, each reading every row again
 // (7B, two 1,000-token prompts: 140 ms; 16 sequences absorbing 57 tokens into
-// 640 rows: 39.8 ms).  Here it is four launches (0.91 ms and 0.75 ms):
+// 640 rows: 39.8 ms).  Here it is four steps (0.90 ms and 0.73 ms):
 //   1. append: the chunk's rows go to slots m.. of each unit, score 0.
 //   2. attend (tcgen05): tiles of 128 query rows (128 / G whole tokens) over
 //      128-row key blocks with an online softmax; writes the outputs and each
@@ -17,6 +17,12 @@
 //      over all queries is a sum inside one thread; the probabilities come
 //      exactly from the normalisers, and each key's sum is added once.
 //   4. finish: lengths, and the eviction where one is due (kvr_generic.cu).
+// Sums in another order can trade two rows whose scores agree to their
+// rounding, and the freed slots are filled in order, so that one traded row
+// moves others: where the rows around the cut lie that close, their scores are
+// formed again token by token, by the generic kernel's arithmetic to the bit,
+// and the rows that stay are those that a token-by-token absorb of the same
+// state keeps (kvr_generic.cu).
 // Recomputing Q K^T in 3 costs one contraction of four, against column sums
 // over the lanes in 2 (124 shuffles a warp and block) and probabilities that
 // are only final after a row's last block.
@@ -71,9 +77,8 @@ __device__ __forceinline__ LUnit unit_at(const AbsorbParams &p, int x) {
   const CacheView &c = p.c;
   LUnit u;
   u.h = x % c.H;
-  const int lr = (x / c.H) % p.nl, sq = x / (c.H * p.nl);
-  u.ug = ((size_t)sq * c.L + p.lb + lr) * c.H + u.h;
-  u.row0 = ((size_t)sq * p.nl + lr) * p.chunk;
+  u.ug = unit_index(c, p.lb, p.nl, x);
+  u.row0 = (size_t)(x / c.H) * p.chunk;
   u.m = c.state[4 * u.ug];
   return u;
 }
@@ -92,6 +97,18 @@ __global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) 
   pdl_begin();
   const CacheView &c = p.c;
   const LUnit u = unit_at(p, blockIdx.x);
+  if (p.settle && blockIdx.y == 0) {
+    if (threadIdx.x == 0) {
+      c.state[4 * u.ug + 2] = 0;  // the key sum's place is the ties' now
+      if (blockIdx.x == 0) tie_words(c, u.ug)[kTieUnits] = 0;
+    }
+    // The scores before the call, behind the normalisers.
+    if (unit_ok(p, u)) {
+      float *old = c.logits + (u.ug + 1) * (size_t)c.G * c.cap - u.m;
+      for (int i = threadIdx.x; i < u.m; i += 256)
+        old[i] = c.score[u.ug * (size_t)c.sstride + i];
+    }
+  }
   if (!unit_ok(p, u)) {
     if (threadIdx.x == 0)
       atomicOr(c.err, u.m >= 0 && u.m + p.chunk > c.cap ? ERR_CAPACITY : ERR_LENGTH);

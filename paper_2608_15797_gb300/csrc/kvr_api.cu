@@ -579,7 +579,7 @@ bool try_long_step(kvr_cache *c, const StepArgs &a, cudaStream_t stream,
 bool try_absorb_long(kvr_cache *c, int lb, int le, int chunk, const void *q,
                      const void *k_new, const void *v_new, void *out,
                      int max_rows, int budget, int window, bool evict,
-                     cudaStream_t stream, cudaError_t *err) {
+                     cudaStream_t stream, cudaError_t *err, int *launches) {
   const CacheView &v = c->view;
   if (!c->fused || !v.kv_bf16 || !v.out_bf16 || v.d != 128 || v.G > 8)
     return false;
@@ -605,12 +605,15 @@ bool try_absorb_long(kvr_cache *c, int lb, int le, int chunk, const void *q,
   p.max_rows = max_rows;
   p.scale_log2e = v.scale * 1.4426950408889634f;
   p.inv_g = 1.f / (float)v.G;
+  p.settle = evict && max_rows > budget + window && kvr::can_settle(v, max_rows);
   *err = kvr::launch_absorb_long(maps->first, maps->second, tmq, p, c->sm_count,
                                  stream);
   if (*err == cudaSuccess)
-    *err = kvr::launch_evict_generic(v, lb, p.nl, max_rows,
-                                     evict ? budget : max_rows,
-                                     evict ? window : 0, stream, chunk);
+    *err = p.settle ? kvr::launch_evict_absorbed(p, budget, window, c->sm_count, stream)
+                    : kvr::launch_evict_generic(v, lb, p.nl, max_rows,
+                                                evict ? budget : max_rows,
+                                                evict ? window : 0, stream, chunk);
+  *launches = p.settle ? 6 : 4;
   return true;
 }
 
@@ -1036,11 +1039,12 @@ kvr_status kvr_absorb_chunk(kvr_cache *c, int lb, int le, int chunk,
     return KVR_OK;
   }
   cudaError_t e = cudaSuccess;
+  int launched = 0;
   if (try_absorb_long(c, lb, le, chunk, q, k_new, v_new, out, m + chunk, budget,
-                      window, evict != 0, as_stream(stream), &e)) {
+                      window, evict != 0, as_stream(stream), &e, &launched)) {
     if (e != cudaSuccess) return cuda_fail("kvr_absorb_chunk", e);
     c->last_absorb = 3;
-    c->launches += 4;
+    c->launches += launched;
     mirror_append(c, lb, le, chunk);
     if (evict) mirror_evict(c, lb, le, budget, window);
     return KVR_OK;

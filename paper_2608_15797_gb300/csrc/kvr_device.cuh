@@ -41,6 +41,36 @@ __device__ __forceinline__ float warp_max(float x) {
   return x;
 }
 
+// The arithmetic by which attend_score_kernel scores a row, every rounding
+// written out: the blocked absorb settles near ties by the same (kvr_absorb_long.cu),
+// and the two have to agree to the bit.  A logit is the lanes' chains of
+// D / 32 products (lane_dot) summed over offsets 16, 8, 4, 2, 1, times the
+// scale; probabilities are head_prob; a row's probabilities are added over the
+// heads in order, and their mean goes onto the score by add_mean.
+template <int E>
+__device__ __forceinline__ float lane_dot(const float *q, const float (&k)[E]) {
+  float acc = 0.f;
+#pragma unroll
+  for (int e = 0; e < E; ++e) acc = fmaf(q[e], k[e], acc);
+  return acc;
+}
+// One warp: the greatest of n logits, and the sum of their exponentials.
+__device__ __forceinline__ void warp_softmax(const float *lg, int n, int lane, float &m,
+                                             float &z) {
+  m = -INFINITY;
+  for (int i = lane; i < n; i += 32) m = fmaxf(m, lg[i]);
+  m = warp_max(m);
+  z = 0.f;
+  for (int i = lane; i < n; i += 32) z += expf(lg[i] - m);
+  z = warp_sum(z);
+}
+__device__ __forceinline__ float head_prob(float lg, float m, float inv_z) {
+  return __fmul_rn(expf(lg - m), inv_z);
+}
+__device__ __forceinline__ float add_mean(float score, float sum, float inv_g) {
+  return fmaf(sum, inv_g, score);
+}
+
 // Collect, in index order, the indices i in [lo, hi) with pred(i) into list.
 // Every thread of the block must call it; returns the count.
 template <typename Pred>

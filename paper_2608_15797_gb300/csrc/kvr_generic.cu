@@ -21,6 +21,10 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
 #include "kvr_device.cuh"
 #include "kvr_internal.h"
 
@@ -293,10 +297,7 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
     for (int g = 0; g < kMaxG; ++g) {
       if (g < G) {
-        float acc = 0.f;
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc += qs[g * D + lane * E + e] * kv[e];
-        acc = warp_sum(acc);
+        const float acc = warp_sum(lane_dot<E>(qs + g * D + lane * E, kv));
         if (lane == 0) lg[(size_t)g * ls + i] = acc * c.scale;
       }
     }
@@ -305,13 +306,8 @@ __global__ void __launch_bounds__(kThreads)
 
   // Softmax statistics: warp g owns query head g.
   if (warp < G) {
-    const float *lr = lg + (size_t)warp * ls;
-    float m = -INFINITY;
-    for (int i = lane; i < n; i += 32) m = fmaxf(m, lr[i]);
-    m = warp_max(m);
-    float z = 0.f;
-    for (int i = lane; i < n; i += 32) z += expf(lr[i] - m);
-    z = warp_sum(z);
+    float m, z;
+    warp_softmax(lg + (size_t)warp * ls, n, lane, m, z);
     if (lane == 0) {
       stat_m[warp] = m;
       stat_iz[warp] = 1.f / z;
@@ -325,11 +321,11 @@ __global__ void __launch_bounds__(kThreads)
   for (int i = tid; i < n; i += kThreads) {
     float acc = 0.f;
     for (int g = 0; g < G; ++g) {
-      const float p = expf(lg[(size_t)g * ls + i] - stat_m[g]) * stat_iz[g];
+      const float p = head_prob(lg[(size_t)g * ls + i], stat_m[g], stat_iz[g]);
       lg[(size_t)g * ls + i] = p;
-      acc += p;
+      acc = __fadd_rn(acc, p);
     }
-    su[i] += acc * inv_g;
+    su[i] = add_mean(su[i], acc, inv_g);
   }
   __syncthreads();
 
@@ -388,44 +384,85 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// Cut every unit longer than B + W back to B + W rows.  kByRank: units of at
-// most NT rows, one row a thread, kept by rank; otherwise the B-th best score
-// is selected over the unit's scores, which shared memory holds once
-// (`cached`; else they are read from global memory on every pass).
-template <typename T, int D, int NT, bool kByRank>
-__global__ void __launch_bounds__(NT)
-    evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow, int max_list,
-                 int cached, int max_rows) {
-  pdl_begin();
-  extern __shared__ int lists[];  // holes | movers [max_list each] | scores
+// A near tie: the least score kept and the greatest dropped lie closer than the
+// blocked absorb's sums are certain to, so which of the rows around the cut a
+// token-by-token absorb would keep is not known.  Lists those rows and enters
+// the unit in the call's list; false where there is no tie, or one of more than
+// kMaxTied rows (whose scores are as a rule equal to the bit on either path).
+// val(i): a candidate's score bits, kNone for the window's rows; keep(i): as the
+// scores stand.  Every thread must call it.
+template <int NT, typename Val, typename Keep>
+__device__ bool near_tie(const CacheView &c, int lb, int nl, size_t u, int n, int chunk,
+                         float band, Val val, Keep keep) {
+  __shared__ unsigned s_lo[NT / 32], s_hi[NT / 32];
+  __shared__ int s_n;
+  const int tid = threadIdx.x;
+  unsigned lo = kNone, hi = 0;
+  for (int i = tid; i < n; i += NT) {
+    const unsigned b = val(i);
+    if (b == kNone) continue;
+    if (keep(i)) lo = min(lo, b);
+    else hi = max(hi, b);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((tid & 31) == 0) {
+    s_lo[tid >> 5] = lo;
+    s_hi[tid >> 5] = hi;
+  }
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) {
+    lo = min(lo, s_lo[w]);
+    hi = max(hi, s_hi[w]);
+  }
+  const float least = __uint_as_float(lo), most = __uint_as_float(hi), w = band * least;
+  if (lo == kNone || !(least - most <= w)) return false;
+  int *words = tie_words(c, u);
+  for (int i = tid; i < n; i += NT) {
+    const unsigned b = val(i);
+    const float x = __uint_as_float(b);
+    if (b != kNone && x >= most - w && x <= least + w) {
+      const int k = atomicAdd(&s_n, 1);
+      if (k < kMaxTied) words[kTieRows + k] = i;
+    }
+  }
+  __syncthreads();
+  const int nt = s_n;
+  if (nt > kMaxTied) return false;
+  if (tid == 0) {
+    words[kTieCount] = nt;
+    const int e = atomicAdd(&tie_words(c, unit_index(c, lb, nl, 0))[kTieUnits], 1);
+    tie_words(c, unit_index(c, lb, nl, e))[kTieEntry] = blockIdx.x;
+  }
+  return true;
+}
+
+// Cut a unit of n > B + W rows back to B + W.  kByRank: units of at most NT
+// rows, one row a thread, kept by rank; otherwise the B-th best score is
+// selected over the unit's scores, which shared memory holds once (`cached`;
+// else they are read from global memory on every pass).  tied(val, keep) is
+// asked first, and true leaves the unit as it is.  Every thread must call it.
+template <typename T, int D, int NT, bool kByRank, typename Tied>
+__device__ void evict_unit(const CacheView &c, size_t u, int n, int newest, int B, int W,
+                           int *lists, int max_list, int cached, Tied tied) {
   __shared__ unsigned s_wsum[NT / 32];
   __shared__ int2 s_cnt[NT / 32];
-
-  const Unit x = unit_of(c, lb, nl);
   const int tid = threadIdx.x;
-  // `grow` rows were appended whose length is not recorded yet.
-  const int n = c.state[4 * x.u] + grow;
-  const int newest = c.state[4 * x.u + 1] + grow - 1;
-  __syncthreads();
-  // Longer than the host thinks: the blocked absorb left such a unit alone, and
-  // an eviction has no room for its lists.
-  if (n < grow || n > (grow ? min(max_rows, c.cap) : max(max_rows, B + W))) {
-    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
-    return;
-  }
-  if (tid == 0 && grow) {
-    c.state[4 * x.u] = n;
-    c.state[4 * x.u + 1] = newest + 1;
-    c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
-  }
-  if (n <= B + W) return;
-  float *su = c.score + x.u * (size_t)c.sstride;
-  int32_t *pu = c.pos + x.u * (size_t)c.sstride;
+  float *su = c.score + u * (size_t)c.sstride;
+  int32_t *pu = c.pos + u * (size_t)c.sstride;
   // The W most recent positions are protected; a row is a candidate iff its
   // position is at most newest - W.
   const int wlo = newest - W;
-  auto finish = [&](auto keep) {
-    compact_unit<T, D, NT>(c, x.u, n, B + W, keep, lists, max_list, s_cnt);
+  // A candidate's score bits (scores are >= 0: they order like the values),
+  // kNone for the window's rows.
+  auto bits = [&](int i) {
+    return pu[i] <= wlo ? min(__float_as_uint(su[i]), kNone - 1) : kNone;
+  };
+  auto finish = [&](auto val, auto keep) {
+    if (tied(val, keep)) return;
+    compact_unit<T, D, NT>(c, u, n, B + W, keep, lists, max_list, s_cnt);
   };
   if constexpr (kByRank) {
     __shared__ unsigned long long s_key[NT];
@@ -433,15 +470,10 @@ __global__ void __launch_bounds__(NT)
     block_rank_keep(
         n, B, [&](int i) { return pu[i] <= wlo; },
         [&](int i) { return rank_key(su[i], pu[i]); }, s_key, s_keep);
-    finish([&](int i) { return s_keep[i] != 0; });
+    finish(bits, [&](int i) { return s_keep[i] != 0; });
   } else {
     __shared__ SelectSmem m;
     unsigned *sv = reinterpret_cast<unsigned *>(lists + 2 * max_list);
-    // A candidate's score bits (scores are >= 0: they order like the values),
-    // kNone for the window's rows.
-    auto bits = [&](int i) {
-      return pu[i] <= wlo ? min(__float_as_uint(su[i]), kNone - 1) : kNone;
-    };
     int have = 0;
     unsigned lo = kNone, hi = 0;
     for (int i0 = tid; i0 < n; i0 += 4 * NT) {  // four rows' loads in flight
@@ -489,12 +521,180 @@ __global__ void __launch_bounds__(NT)
         last = select_desc<NT>(n, rest, low_pos, lo, hi, m, &r2, &t2);
       }
     }
-    finish([&](int i) {
+    finish(val, [&](int i) {
       const unsigned b = val(i);
       if (b == kNone) return true;
       if (B == 0) return false;
       return b > thr || (b == thr && ~(unsigned)pu[i] - 1u >= last);
     });
+  }
+}
+
+// Cut every unit longer than B + W back to B + W rows.  kTies (the blocked
+// absorb of `grow` tokens): units with a near tie are listed and left long.
+template <typename T, int D, int NT, bool kByRank, bool kTies>
+__global__ void __launch_bounds__(NT)
+    evict_kernel(CacheView c, int lb, int nl, int B, int W, int grow, int max_list,
+                 int cached, int max_rows, float band) {
+  pdl_begin();
+  extern __shared__ int lists[];  // holes | movers [max_list each] | scores
+
+  const Unit x = unit_of(c, lb, nl);
+  const int tid = threadIdx.x;
+  // `grow` rows were appended whose length is not recorded yet.
+  const int n = c.state[4 * x.u] + grow;
+  const int newest = c.state[4 * x.u + 1] + grow - 1;
+  __syncthreads();
+  // Longer than the host thinks: the blocked absorb left such a unit alone, and
+  // an eviction has no room for its lists.
+  if (n < grow || n > (grow ? min(max_rows, c.cap) : max(max_rows, B + W))) {
+    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+    return;
+  }
+  if (tid == 0 && grow) {
+    c.state[4 * x.u] = n;
+    c.state[4 * x.u + 1] = newest + 1;
+    c.state[4 * x.u + 2] = 0;  // the R-KV key sum no longer matches
+  }
+  if (n <= B + W) return;
+  evict_unit<T, D, NT, kByRank>(c, x.u, n, newest, B, W, lists, max_list, cached,
+                                [&](auto val, auto keep) {
+                                  if constexpr (kTies)
+                                    return near_tie<NT>(c, lb, nl, x.u, n, grow, band, val, keep);
+                                  return false;
+                                });
+}
+
+// Of token `tok` of a blocked absorb: put(i, x) with x the sum over the heads of
+// the probabilities of the unit's i-th tied row, by the arithmetic of
+// attend_score_kernel to the bit: a warp a row, its lanes' products summed over
+// the same offsets (the heads' sums are folded into each other, so that the five
+// steps take 9 exchanges for eight heads).  smem: tie_smem() bytes.  Every
+// thread must call it.
+template <typename Put>
+__device__ void tie_sums(const AbsorbParams &p, int x, int tok, float *smem, Put put) {
+  __shared__ float s_m[kMaxG], s_iz[kMaxG];
+  const CacheView &c = p.c;
+  const int G = c.G, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x;
+  float *lg = smem;  // [G][max_rows]
+  const size_t u = unit_index(c, p.lb, p.nl, x);
+  const int n = c.state[4 * u] - p.chunk + tok + 1;  // rows that the token sees
+  auto row4 = [](uint2 w, float(&v)[4]) {
+    v[0] = __uint_as_float(w.x << 16);
+    v[1] = __uint_as_float(w.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(w.y << 16);
+    v[3] = __uint_as_float(w.y & 0xFFFF0000u);
+  };
+  const uint2 *Q = reinterpret_cast<const uint2 *>(p.q) +
+                   (((size_t)(x / c.H) * p.chunk + tok) * c.H + x % c.H) * (size_t)G * 32;
+  const uint2 *K = reinterpret_cast<const uint2 *>(c.K) + u * (size_t)c.cap * 32;
+  float q[kMaxG][4];
+#pragma unroll
+  for (int h = 0; h < kMaxG; ++h) row4(h < G ? Q[h * 32 + lane] : make_uint2(0u, 0u), q[h]);
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  const int g = lane >> 2;  // the head whose sum this lane ends with
+#pragma unroll 2
+  for (int i = warp; i < n; i += NT / 32) {
+    float k[4], a[kMaxG];
+    row4(K[(size_t)i * 32 + lane], k);
+#pragma unroll
+    for (int h = 0; h < kMaxG; ++h) a[h] = lane_dot<4>(q[h], k);
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      a[h] = (b4 ? a[h + 4] : a[h]) + __shfl_xor_sync(0xffffffffu, b4 ? a[h] : a[h + 4], 16);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      a[h] = (b3 ? a[h + 2] : a[h]) + __shfl_xor_sync(0xffffffffu, b3 ? a[h] : a[h + 2], 8);
+    float s = (b2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a[0] : a[1], 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if ((lane & 3) == 0 && g < G) lg[(size_t)g * p.max_rows + i] = s * c.scale;
+  }
+  __syncthreads();
+  if (warp < G) {
+    float m, z;
+    warp_softmax(lg + (size_t)warp * p.max_rows, n, lane, m, z);
+    if (lane == 0) {
+      s_m[warp] = m;
+      s_iz[warp] = 1.f / z;
+    }
+  }
+  __syncthreads();
+  const int *words = tie_words(c, u);
+  for (int i = tid; i < words[kTieCount]; i += NT) {
+    const int slot = words[kTieRows + i];
+    float sum = 0.f;
+    if (slot < n)
+      for (int h = 0; h < G; ++h)
+        sum = __fadd_rn(sum, head_prob(lg[(size_t)h * p.max_rows + slot], s_m[h], s_iz[h]));
+    put(i, sum);
+  }
+  __syncthreads();
+}
+size_t tie_smem(const CacheView &c, int max_rows) {
+  return (size_t)c.G * max_rows * sizeof(float);
+}
+
+// Those sums for every listed unit, one CTA a token and unit.  Few units have
+// ties, and a launch that finds none ends at once.
+__global__ void __launch_bounds__(kThreads) tie_sums_kernel(const AbsorbParams p) {
+  pdl_begin();
+  extern __shared__ __align__(16) float tie_mem[];
+  const CacheView &c = p.c;
+  const int count = tie_words(c, unit_index(c, p.lb, p.nl, 0))[kTieUnits];
+  for (long long job = blockIdx.x; job < (long long)count * p.chunk; job += gridDim.x) {
+    const int e = (int)(job / p.chunk), tok = (int)(job % p.chunk);
+    const int x = tie_words(c, unit_index(c, p.lb, p.nl, e))[kTieEntry];
+    const size_t u = unit_index(c, p.lb, p.nl, x);
+    if (!tie_room(c, tie_words(c, u)[kTieCount], p.chunk, c.state[4 * u] - p.chunk)) continue;
+    float *sums = c.logits + u * (size_t)c.G * c.cap;
+    const int tied = tie_words(c, u)[kTieCount];
+    tie_sums(p, x, tok, tie_mem, [&](int i, float sum) { sums[(size_t)tok * tied + i] = sum; });
+  }
+}
+
+// The listed units, one a CTA at a time: the tied rows' scores, token by token
+// as attend_score_kernel adds them (the sums formed here where the unit's
+// scratch, at G = 1 or 2, had no room for them), then the eviction.
+template <typename T, int D, int NT, bool kByRank>
+__global__ void __launch_bounds__(NT)
+    evict_tied_kernel(const AbsorbParams p, int B, int W, int max_list, int cached) {
+  pdl_begin();
+  extern __shared__ __align__(16) float tie_mem[];  // tie_sums' or evict_unit's
+  int *lists = reinterpret_cast<int *>(tie_mem);
+  __shared__ float s_score[kMaxTied];
+  const CacheView &c = p.c;
+  const int count = tie_words(c, unit_index(c, p.lb, p.nl, 0))[kTieUnits];
+  for (int e = blockIdx.x; e < count; e += gridDim.x) {
+    const int x = tie_words(c, unit_index(c, p.lb, p.nl, e))[kTieEntry];
+    const size_t u = unit_index(c, p.lb, p.nl, x);
+    const int *words = tie_words(c, u);
+    const int n = c.state[4 * u], newest = c.state[4 * u + 1] - 1, m = n - p.chunk;
+    const int tied = words[kTieCount];
+    const float *sums = c.logits + u * (size_t)c.G * c.cap;
+    const float *old = sums + (size_t)c.G * c.cap - m;
+    const bool room = tie_room(c, tied, p.chunk, m);
+    for (int i = threadIdx.x; i < tied; i += NT) {
+      const int slot = words[kTieRows + i];
+      float s = slot < m ? old[slot] : 0.f;
+      if (room) {
+#pragma unroll 32
+        for (int j = 0; j < p.chunk; ++j)  // (0 from a token that does not see the row)
+          s = add_mean(s, sums[(size_t)j * tied + i], p.inv_g);
+      }
+      s_score[i] = s;
+    }
+    if (!room)
+      for (int j = 0; j < p.chunk; ++j)
+        tie_sums(p, x, j, tie_mem, [&](int i, float sum) {
+          s_score[i] = add_mean(s_score[i], sum, p.inv_g);
+        });
+    for (int i = threadIdx.x; i < tied; i += NT)  // (each thread its own)
+      c.score[u * (size_t)c.sstride + words[kTieRows + i]] = s_score[i];
+    __syncthreads();
+    evict_unit<T, D, NT, kByRank>(c, u, n, newest, B, W, lists, max_list, cached,
+                                  [](auto, auto) { return false; });
+    __syncthreads();
   }
 }
 
@@ -565,30 +765,36 @@ cudaError_t attend_ext_dispatch(const CacheView &c, const StepArgs &a,
 // which a unit takes 1,024 threads instead of 256 (few units, long scans).
 constexpr int kCachedRows = 49152, kWideRows = 2048;
 
-template <typename T, int D, int NT, bool kByRank>
-cudaError_t evict_launch(const CacheView &c, int lb, int nl, int max_rows, int B, int W,
-                         int grow, cudaStream_t st) {
-  const int nk = B + W;
-  const int max_list = max(1, min(nk, max_rows - nk));
-  const int cached = !kByRank && max_rows <= kCachedRows &&
+// An eviction's launch: the kernel's threads a unit and whether it ranks, by the
+// longest unit, and its shared memory.
+template <typename Run>
+cudaError_t evict_shape(int max_rows, int nk, Run run) {
+  const int max_list = std::max(1, std::min(nk, max_rows - nk));
+  const bool by_rank = max_rows <= kThreads;
+  const int cached = !by_rank && max_rows <= kCachedRows &&
                      (2 * (size_t)max_list + max_rows) * sizeof(int) <= 200 * 1024;
   const size_t bytes = (2 * (size_t)max_list + (cached ? max_rows : 0)) * sizeof(int);
-  auto kern = evict_kernel<T, D, NT, kByRank>;
-  cudaError_t e = cudaFuncSetAttribute(
-      kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(NT), bytes, st, c, lb, nl, B, W, grow,
-                    max_list, cached, max_rows);
+  using std::integral_constant;
+  if (by_rank)
+    return run(integral_constant<int, kThreads>{}, std::true_type{}, max_list, cached, bytes);
+  if (max_rows <= kWideRows)
+    return run(integral_constant<int, kThreads>{}, std::false_type{}, max_list, cached, bytes);
+  return run(integral_constant<int, 1024>{}, std::false_type{}, max_list, cached, bytes);
 }
 
-template <typename T, int D>
-cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows,
-                           int B, int W, int grow, cudaStream_t st) {
-  if (max_rows <= kThreads)
-    return evict_launch<T, D, kThreads, true>(c, lb, nl, max_rows, B, W, grow, st);
-  if (max_rows <= kWideRows)
-    return evict_launch<T, D, kThreads, false>(c, lb, nl, max_rows, B, W, grow, st);
-  return evict_launch<T, D, 1024, false>(c, lb, nl, max_rows, B, W, grow, st);
+template <typename T, int D, bool kTies = false>
+cudaError_t evict_dispatch(const CacheView &c, int lb, int nl, int max_rows, int B, int W,
+                           int grow, cudaStream_t st, float band = 0.f) {
+  return evict_shape(max_rows, B + W, [&](auto nt, auto rank, int max_list, int cached,
+                                          size_t bytes) {
+    constexpr int NT = decltype(nt)::value;
+    auto kern = evict_kernel<T, D, NT, decltype(rank)::value, kTies>;
+    const cudaError_t e = cudaFuncSetAttribute(
+        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kern, dim3(c.S * nl * c.H), dim3(NT), bytes, st, c, lb, nl, B, W, grow,
+                      max_list, cached, max_rows, band);
+  });
 }
 
 }  // namespace
@@ -648,6 +854,44 @@ cudaError_t launch_evict_generic(const CacheView &c, int lb, int nl,
                                                  window, grow, st)
                     : evict_dispatch<float, 64>(c, lb, nl, max_rows, budget,
                                                 window, grow, st);
+}
+
+// Scores of the blocked absorb and of the token-by-token one differ by the order
+// of their sums, one rounding a token on the latter's side: near the cut by
+// 1.3e-7 rms and 7.3e-7 at most after 57 tokens (7B, 16 sequences of 640 rows,
+// three inputs; 4.6e-7 after 10), 5.7e-7 and 2.5e-6 after 1,000.  Two rows'
+// order is taken as certain beyond more than twice the most.  Settling them
+// is 3 us of 727 and, where a prompt of 1,000 tokens has a tie, 0.1 ms of 0.9.
+float tie_band(int chunk) { return 0x1p-19f * std::max(1.f, std::sqrt(chunk / 64.f)); }
+
+bool can_settle(const CacheView &c, int max_rows) {
+  return tie_smem(c, max_rows) <= 200 * 1024;
+}
+
+cudaError_t launch_evict_absorbed(const AbsorbParams &p, int budget, int window, int sms,
+                                  cudaStream_t st) {
+  using T = __nv_bfloat16;
+  const CacheView &c = p.c;
+  cudaError_t e = evict_dispatch<T, 128, true>(c, p.lb, p.nl, p.max_rows, budget, window,
+                                               p.chunk, st, tie_band(p.chunk));
+  if (e != cudaSuccess) return e;
+  const size_t sums = tie_smem(c, p.max_rows);
+  e = cudaFuncSetAttribute(tie_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sums);
+  if (e == cudaSuccess)
+    e = launch_pdl(tie_sums_kernel, dim3(4 * sms), dim3(kThreads), sums, st, p);
+  if (e != cudaSuccess) return e;
+  return evict_shape(p.max_rows, budget + window, [&](auto nt, auto rank, int max_list,
+                                                      int cached, size_t lists) {
+    constexpr int NT = decltype(nt)::value;
+    auto kern = evict_tied_kernel<T, 128, NT, decltype(rank)::value>;
+    const size_t bytes = std::max(lists, sums);
+    const cudaError_t e1 = cudaFuncSetAttribute(
+        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e1 != cudaSuccess) return e1;
+    return launch_pdl(kern, dim3(std::min(c.S * p.nl * c.H, sms)), dim3(NT), bytes, st, p,
+                      budget, window, max_list, cached);
+  });
 }
 
 cudaError_t launch_load(const CacheView &c, int seq, const void *k,

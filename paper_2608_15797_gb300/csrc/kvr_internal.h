@@ -303,6 +303,7 @@ struct AbsorbParams {
   int max_rows;  // largest unit after the chunk over the call
   int budget, window, evict;
   float scale_log2e, inv_g;
+  int settle;    // kvr_absorb_long.cu only
 };
 int absorb_max_chunk();
 int absorb_max_rows();
@@ -320,10 +321,35 @@ cudaError_t launch_absorb(const AbsorbParams &p, int kernel, const CUtensorMap *
 // outputs and add the scores; the lengths are left to the launch_evict_generic
 // (grow = chunk) that follows.  tmK, tmV: the slab with boxes of
 // absorb_long_box_rows() rows; tmQ as for launch_absorb.
+// p.settle: the old scores are kept and the list of ties emptied for
+// launch_evict_absorbed.
 int absorb_long_box_rows();
 cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
                                const CUtensorMap &tmQ, const AbsorbParams &p,
                                int sms, cudaStream_t st);
+// Its end where rows are evicted (kvr_generic.cu), after which the rows that
+// stay are those of a token-by-token absorb from the same state.  can_settle:
+// whether a unit's logits fit in shared memory, as it asks.
+bool can_settle(const CacheView &c, int max_rows);
+cudaError_t launch_evict_absorbed(const AbsorbParams &p, int budget, int window,
+                                  int sms, cudaStream_t st);
+// Index of unit x in [0, S * nl * H) of a call over layers [lb, lb + nl).
+__device__ __forceinline__ size_t unit_index(const CacheView &c, int lb, int nl, int x) {
+  const int h = x % c.H, lr = (x / c.H) % nl, s = x / (c.H * nl);
+  return ((size_t)s * c.L + lb + lr) * c.H + h;
+}
+// Where a call keeps its ties: in the units' R-KV key sums, which an absorb
+// makes stale.  Of the call's first unit: how many units are listed; of its
+// e-th: entry e, a unit's index in the call; of a listed unit: its tied rows.
+// Their head sums go to its logit scratch, [token][row], where there is room
+// before the old scores at the scratch's end.
+enum : int { kTieUnits = 0, kTieEntry = 1, kTieCount = 2, kTieRows = 4, kMaxTied = 96 };
+__device__ __forceinline__ int *tie_words(const CacheView &c, size_t u) {
+  return reinterpret_cast<int *>(c.rsum + u * 128);
+}
+__device__ __forceinline__ bool tie_room(const CacheView &c, int tied, int chunk, int m) {
+  return (size_t)tied * chunk <= (size_t)c.G * c.cap - m;
+}
 
 // Persistent chunked step (kvr_chunked.cu): bf16, d = 128, G <= 8, at most
 // chunk_max_rows() rows per job with the new row.  A job is one unit of the
