@@ -273,7 +273,6 @@ __global__ void __launch_bounds__(kAttThr, 2)
     for (int i = blockIdx.x; i < n_items && ok; i += gridDim.x) {
       AttItem it;
       if (!att_item(p, i, units, n_qt, Jt, it)) continue;
-      const int n = it.u.m + p.chunk;
       for (int j = 0; j < it.nb; ++j) {
         const int ncol = min(kBlk, (it.lim - j * kBlk + 15) & ~15);
         ok = wait_warp(b_kfull, nk++) && (j > 0 || wait_warp(b_qfull, nq++));
@@ -293,12 +292,13 @@ __global__ void __launch_bounds__(kAttThr, 2)
         }
         ok = wait_warp(b_vfull, nv);
         if (!ok) break;
-        // V rows past the unit's last one, up to the 16-row step of PV,
-        // meet P = 0 and must be finite: zeros.
-        const int v0 = n - j * kBlk, v1 = min(kBlk, (v0 + 15) & ~15);
-        if (it.lim == n && v0 > 0 && v0 < v1) {
+        // V rows past the last one that the tile sees, up to the 16-row step of
+        // PV, meet P = 0 and must be finite: zeros.  (They are a later tile's,
+        // or the cache's slots past the unit's end, which may hold anything.)
+        const int v0 = it.lim - j * kBlk;
+        if (v0 < ncol) {
           unsigned char *V = smem + 2 * kTile;
-          for (int x = lane; x < (v1 - v0) * 16; x += 32)
+          for (int x = lane; x < (ncol - v0) * 16; x += 32)
             reinterpret_cast<int4 *>(V + ((x >> 3) & 1) * kHalf + (v0 + (x >> 4)) * 128)[x & 7] =
                 make_int4(0, 0, 0, 0);
           fence_proxy_async();

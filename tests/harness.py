@@ -18,8 +18,10 @@ from paper_2608_15797_gb300 import inputs, kvr
 # Canary guard regions: every device buffer the parity runs hand to the
 # library sits between two GUARD-byte regions filled with CANARY, and the
 # regions are checked after each run, so a write past either end of a
-# caller buffer fails the test that made it.
-GUARD, CANARY = 4096, 0xA5
+# caller buffer fails the test that made it.  The buffers themselves start as
+# UNWRITTEN bytes, a NaN in bf16 and fp32, so that a kernel that lets a slot
+# nobody has written into a sum fails too.
+GUARD, CANARY, UNWRITTEN = 4096, 0xA5, 0xFF
 
 
 class Guarded:
@@ -30,6 +32,7 @@ class Guarded:
         self.raw = torch.full((nbytes + 2 * GUARD,), CANARY, dtype=torch.uint8,
                               device=device)
         self.buf = self.raw[GUARD:GUARD + nbytes]
+        self.buf.fill_(UNWRITTEN)
 
     def intact(self) -> bool:
         return bool((self.raw[:GUARD] == CANARY).all().item() and

@@ -43,6 +43,19 @@ def test_absorb_long_shapes(G, old, chunk):
     harness.lockstep(c, o, w, 90 + G, 2, w.budget, w.window, step0=100)
 
 
+@pytest.mark.parametrize("G,old,chunk", [(7, [640, 633], 57), (7, [0, 0], 200),
+                                         (3, [500, 11], 43), (1, [3, 250], 130)])
+def test_absorb_long_beside_slots_that_nothing_has_written(G, old, chunk):
+    """Query tiles that end within 16 rows of the unit's end, in a cache with
+    room behind it: PV's last step reads slots that hold NaN, with P = 0."""
+    w = inputs.Workload("al", 1, 2, G, 128, "bf16", 48, 8, 0, 0, sigma=1.0)
+    c, o = harness.make_pair(w, 95 + G, 2, cap=max(old) + chunk + 16,
+                             prompt_lens=old, out_dtype="bf16")
+    absorb_lockstep(c, o, w, 95 + G, chunk, w.budget, w.window)
+    assert c.last_absorb_kernel() == 3
+    harness.check_guards(c)
+
+
 def test_absorb_long_without_eviction_and_budget_edges():
     """No eviction (every unit grows), then a chunk cut to a budget of one
     row and no window; peaked logits (scores of 3-sigma keys) move the online
