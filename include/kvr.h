@@ -254,7 +254,8 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *fork, int layer_begin,
  * parent's state: kept prefix rows stay, freed parent slots receive the kept
  * tail rows, and the parent's scores become the candidate's.  Every layer's
  * tails must have the same length.  The fork is spent afterwards (further
- * calls return KVR_ESTATE). */
+ * calls return KVR_ESTATE).  KVR_ECAPACITY, with nothing changed, where a unit
+ * would hold more rows than the parent's capacity. */
 kvr_status kvr_fork_commit(kvr_fork *fork, const int32_t *chosen, int budget,
                            int window, void *stream);
 

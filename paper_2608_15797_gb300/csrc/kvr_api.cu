@@ -1650,8 +1650,14 @@ kvr_status kvr_fork_commit(kvr_fork *f, const int32_t *chosen, int budget,
       return fail(KVR_EINVAL, "chosen[%d] = %d outside [0, %d)", s, chosen[s],
                   f->view.N);
   int max_rows = 1;
-  for (size_t i = 0; i < p->len.size(); ++i)
-    max_rows = std::max(max_rows, p->len[i] + f->tlen[i]);
+  for (size_t i = 0; i < p->len.size(); ++i) {
+    const int rows = p->len[i] + f->tlen[i];
+    if (std::min<long long>(rows, (long long)budget + window) > p->desc.capacity)
+      return fail(KVR_ECAPACITY, "a unit would hold %d rows of at most %lld; "
+                  "capacity %d", rows, (long long)budget + window,
+                  p->desc.capacity);
+    max_rows = std::max(max_rows, rows);
+  }
   cudaStream_t strm = as_stream(stream);
   cudaError_t e = cudaMemcpyAsync(f->chosen_dev, chosen,
                                   p->desc.n_seq * sizeof(int32_t),

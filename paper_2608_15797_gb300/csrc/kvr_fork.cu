@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(kThreads)
   atomicAdd(&s_count, mine);
   __syncthreads();
   const int nk = s_count;
-  if (nk != (evict ? B + W : n)) {
-    if (tid == 0) atomicOr(c.err, ERR_LENGTH);
+  if (nk != (evict ? B + W : n) || nk > c.cap) {  // nothing has been written
+    if (tid == 0) atomicOr(c.err, nk > c.cap ? ERR_CAPACITY : ERR_LENGTH);
     return;
   }
   // Staying rows: kept prefix rows below nk.  Holes: parent slots below nk
@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(NT)
   int nk = 0;
 #pragma unroll
   for (int w = 0; w < kNW; ++w) nk += s_keep[w];
-  if (nk != (evict ? B + W : n)) {
-    if (r == 0) atomicOr(c.err, ERR_LENGTH);
+  if (nk != (evict ? B + W : n) || nk > c.cap) {  // nothing has been written
+    if (r == 0) atomicOr(c.err, nk > c.cap ? ERR_CAPACITY : ERR_LENGTH);
     return;
   }
   // Staying rows: kept prefix rows below nk, whose scores become the

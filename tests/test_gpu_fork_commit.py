@@ -1,9 +1,10 @@
 """kvr_fork_commit where every row of prefix + tail has a thread (up to 128 and
 up to 256 rows) and one row past that, against the oracle."""
+import numpy as np
 import pytest
 import torch
 
-from paper_2608_15797_gb300 import inputs
+from paper_2608_15797_gb300 import inputs, kvr
 from tests import harness
 
 pytestmark = pytest.mark.gpu
@@ -35,3 +36,29 @@ def test_commit_shapes(np_, nt, B, W, d, dtype):
     harness.check_guards(c)
     if B and np_ + nt < 200:
         harness.lockstep(c, o2, w, 500 + np_, 2, B, W, step0=100)
+
+
+@pytest.mark.parametrize("np_", [72, 300])  # by rank, and by select
+def test_commit_past_the_capacity_is_refused(np_):
+    """A 16-token tail on a parent with one free row: a budget that keeps all of
+    it is refused on the host with the fork as it was; one that fits commits."""
+    w = inputs.Workload("fc", 1, 2, 2, 128, "bf16", np_ + 56, 8, 0, 0, sigma=1.0)
+    c, o = harness.make_pair(w, 510, 2, cap=np_ + 1, prompt_lens=[np_, 5])
+    f = harness.guarded_fork(c, 2, 16)
+    for t in range(16):
+        f.attend_score(*(harness.dev(a, w.dtype)[None].expand(
+            2, *a.shape).contiguous() for a in inputs.step_inputs(w, 510, t, 2)))
+    before = c.export(0)
+    launches = c.launch_count()
+    with pytest.raises(kvr.KvrError) as e:
+        f.commit(np.array([1, 0], np.int32), np_ + 56, 8)
+    assert e.value.status == kvr.KVR_ECAPACITY
+    assert c.launch_count() == launches
+    assert c.lengths().tolist() == [[np_], [5]]
+    after = c.export(0)
+    for name in ("K", "V", "score", "pos", "len"):
+        assert np.array_equal(before[name], after[name], equal_nan=True)
+    f.commit(np.array([1, 0], np.int32), np_ - 7, 8)      # np_ + 1 rows: the capacity
+    assert c.lengths().tolist() == [[np_ + 1], [21]]
+    c.sync_status()
+    harness.check_guards(c, f)
