@@ -488,11 +488,13 @@ __global__ void __launch_bounds__(kAttThr, 2)
       const float inv = 1.f / l;
       const size_t qrow = ((it.u.row0 + it.tok0 + tk) * c.H + it.u.h) * G + (r - tk * G);
       unsigned char *orow = reinterpret_cast<unsigned char *>(p.out) + qrow * 256 + 128 * hf;
+      float note = 0.f;
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         float o[32];
         tmem_ld32(tO + 32 * k, o);
         tmem_wait_ld();
+        note += nonfinite(o);
         if (valid) {
           uint32_t w[16];
 #pragma unroll
@@ -508,6 +510,21 @@ __global__ void __launch_bounds__(kAttThr, 2)
           }
         }
       }
+      if (valid && note != 0.f && l < INFINITY) {
+        // Perhaps not this row's doing: its outputs from the rows it sees.
+        const size_t row = it.u.ug * (size_t)c.cap * 128;
+        for (int k = 0; k < 2; ++k) {
+          float o[32];
+          for (int x = 0; x < 32; ++x) o[x] = 0.f;
+          attend_row(p.q + qrow * 128, reinterpret_cast<const __nv_bfloat16 *>(c.K) + row,
+                     reinterpret_cast<const __nv_bfloat16 *>(c.V) + row,
+                     it.u.m + it.tok0 + tk + 1, c0 + 32 * k, scale, ref, o);
+          for (int x = 0; x < 16; ++x)
+            reinterpret_cast<uint32_t *>(orow + 64 * k)[x] =
+                pack_bf16(o[2 * x] * inv, o[2 * x + 1] * inv);
+        }
+      }
+      __syncwarp();
       if (valid && hf == 0)
         lse[it.u.ug * (size_t)G * c.cap + (size_t)it.tok0 * G + r] = ref + log2f(l);
       tc_fence_before();

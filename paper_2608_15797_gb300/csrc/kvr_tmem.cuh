@@ -82,5 +82,57 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a, uint64_t b, ui
       : "memory");
 }
 
+// One query row on its own, over the n rows it sees of K and V (128 bf16 a row):
+// o[x] += 2^(q.k scale - ref) v[c0 + x].  For the rows of a tile whose outputs are
+// not finite: the rows that a tile's mask hides have P = 0 in its product with
+// V, and 0 x NaN or 0 x Inf there is NaN, so a row that another query (a
+// later token's, another candidate's) put a non-finite value in would reach
+// queries that do not see it.  As a rule never called.
+static __device__ __noinline__ void attend_row(const __nv_bfloat16 *q, const __nv_bfloat16 *K,
+                                        const __nv_bfloat16 *V, int n, int c0, float scale,
+                                        float ref, float *o) {
+  auto lo = [](uint32_t w) { return __uint_as_float(w << 16); };
+  auto hi = [](uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); };
+  const uint4 *q4 = reinterpret_cast<const uint4 *>(q);
+  for (int i = 0; i < n; ++i) {
+    const uint4 *k4 = reinterpret_cast<const uint4 *>(K + (size_t)i * 128);
+    float s = 0.f;
+#pragma unroll 4
+    for (int x = 0; x < 16; ++x) {
+      const uint4 a = q4[x], b = k4[x];
+      s = fmaf(lo(a.x), lo(b.x), fmaf(hi(a.x), hi(b.x), s));
+      s = fmaf(lo(a.y), lo(b.y), fmaf(hi(a.y), hi(b.y), s));
+      s = fmaf(lo(a.z), lo(b.z), fmaf(hi(a.z), hi(b.z), s));
+      s = fmaf(lo(a.w), lo(b.w), fmaf(hi(a.w), hi(b.w), s));
+    }
+    const float w = ex2(fmaf(s, scale, -ref));
+    const uint4 *v4 = reinterpret_cast<const uint4 *>(V + (size_t)i * 128 + c0);
+#pragma unroll 1
+    for (int x = 0; x < 4; ++x) {
+      const uint4 v = v4[x];
+      float *p = o + 8 * x;
+      p[0] = fmaf(w, lo(v.x), p[0]);
+      p[1] = fmaf(w, hi(v.x), p[1]);
+      p[2] = fmaf(w, lo(v.y), p[2]);
+      p[3] = fmaf(w, hi(v.y), p[3]);
+      p[4] = fmaf(w, lo(v.z), p[4]);
+      p[5] = fmaf(w, hi(v.z), p[5]);
+      p[6] = fmaf(w, lo(v.w), p[6]);
+      p[7] = fmaf(w, hi(v.w), p[7]);
+    }
+  }
+}
+// NaN where one of v is not finite, else 0.
+__device__ __forceinline__ float nonfinite(const float (&v)[32]) {
+  const uint64_t zero = pk2(0.f, 0.f);
+  uint64_t n[4] = {zero, zero, zero, zero};
+#pragma unroll
+  for (int x = 0; x < 32; x += 2)
+    n[(x >> 1) & 3] = fma2(pk2(v[x], v[x + 1]), zero, n[(x >> 1) & 3]);
+  float a, b;
+  upk2(add2(add2(n[0], n[1]), add2(n[2], n[3])), a, b);
+  return a + b;
+}
+
 }  // namespace ptx
 }  // namespace kvr
