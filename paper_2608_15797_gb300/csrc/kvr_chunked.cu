@@ -41,10 +41,10 @@
 //    of normalised keys S (a B operand of three bf16 terms) and its squared
 //    norm (the diagonal of the tile's Gram block), so that no key is read
 //    twice.  One more exchange of sums at the end of a job gives z.  Units
-//    with no current S get one from rkv_sum_kernel, launched before.  7B, 16
-//    sequences, 641-row units: 145 us against 113 for the plain step; the
-//    separate eviction pass it replaces (two readings of the keys, a radix
-//    select) took 337 us after the 113.
+//    with no current S, or an old one, get one from rkv_sum_kernel, launched
+//    before.  7B, 16 sequences, 641-row units: 150 us against 113 for the plain
+//    step; the separate eviction pass it replaces (two readings of the keys, a
+//    radix select) took 337 us after the 113.
 //  - Launched with programmatic stream serialization; every mbarrier wait is
 //    bounded (about 2 s) and on timeout sets ERR_TIMEOUT and drains its own
 //    copies.
@@ -311,39 +311,62 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
 }
 
 // R-KV: the sum of a unit's normalised keys, where the unit has none that is
-// current (state word 2); one CTA a unit, a warp a row.  In the steady state
-// every unit has one and this is the launch of an empty kernel.
-__global__ void __launch_bounds__(128) rkv_sum_kernel(CacheView c, int lb, int nl) {
+// current (state word 2), or one that kSumSteps steps have added a key to and
+// taken one from (word 3 counts them), whose roundings would go on adding up.
+// One CTA a unit, a warp four rows at a time.  Rms error of the sum's elements
+// against fp64, 640 rows: 2.6e-7 formed here, 3.7e-7 after 12 steps (and 1.3e-6
+// after 400); 3.8e-7 as the eviction pass forms it at every step.  In the steady
+// state this is an empty launch but for one step in kSumSteps: 7B, 16 sequences,
+// 145 us a step without new sums, 150 with.
+constexpr int kSumSteps = 12;
+__global__ void __launch_bounds__(256) rkv_sum_kernel(CacheView c, int lb, int nl) {
   pdl_begin();
-  __shared__ float4 s_S[4][32];
-  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int h = b % c.H, lr = (b / c.H) % nl, sq = b / (c.H * nl);
-  const size_t u = ((size_t)sq * c.L + lb + lr) * c.H + h;
-  const int n = c.state[4 * u];
-  if (c.state[4 * u + 2] == 1 || n < 0 || n > c.cap) return;
+  constexpr int kW = 8, kAhead = 4;
+  __shared__ float4 s_S[kW][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t u = unit_index(c, lb, nl, blockIdx.x);
+  const int4 st = *reinterpret_cast<const int4 *>(c.state + 4 * u);
+  const int n = st.x;
+  __syncthreads();  // every thread has read the words
+  if (st.z == 1 && st.w >= 0 && st.w < kSumSteps) {
+    if (threadIdx.x == 0) c.state[4 * u + 3] = st.w + 1;
+    return;
+  }
+  if (n < 0 || n > c.cap) return;
   const unsigned char *K = reinterpret_cast<const unsigned char *>(c.K) + u * (size_t)c.cap * 256;
   float S[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-  for (int i = warp; i < n; i += 4) {
-    float k[4];
-    key4(K + (size_t)i * 256, lane, k);
-    const float inv = inv_norm(k);
+  for (int i = warp * kAhead; i < n; i += kW * kAhead) {
+    float k[kAhead][4];
 #pragma unroll
-    for (int x = 0; x < 4; ++x) S[x] = fmaf(k[x], inv, S[x]);
+    for (int r = 0; r < kAhead; ++r) {
+      k[r][0] = k[r][1] = k[r][2] = k[r][3] = 0.f;
+      if (i + r < n) key4(K + (size_t)(i + r) * 256, lane, k[r]);
+    }
+    float inv[kAhead];
+#pragma unroll
+    for (int r = 0; r < kAhead; ++r) inv[r] = inv_norm(k[r]);
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      S[x] += fmaf(k[0][x], inv[0], k[1][x] * inv[1]) + fmaf(k[2][x], inv[2], k[3][x] * inv[3]);
   }
   s_S[warp][lane] = make_float4(S[0], S[1], S[2], S[3]);
   __syncthreads();
   if (warp == 0) {
-    float4 t = s_S[0][lane];
+    auto add = [](float4 a, float4 b) {
+      return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+    };
+    float4 t[kW];
 #pragma unroll
-    for (int w = 1; w < 4; ++w) {
-      t.x += s_S[w][lane].x;
-      t.y += s_S[w][lane].y;
-      t.z += s_S[w][lane].z;
-      t.w += s_S[w][lane].w;
+    for (int w = 0; w < kW; ++w) t[w] = s_S[w][lane];
+#pragma unroll
+    for (int o = 1; o < kW; o *= 2)
+#pragma unroll
+      for (int w = 0; w < kW; w += 2 * o) t[w] = add(t[w], t[w + o]);
+    reinterpret_cast<float4 *>(c.rsum + u * 128)[lane] = t[0];
+    if (lane == 0) {
+      c.state[4 * u + 2] = 1;
+      c.state[4 * u + 3] = 0;
     }
-    reinterpret_cast<float4 *>(c.rsum + u * 128)[lane] = t;
-    if (lane == 0) c.state[4 * u + 2] = 1;
   }
 }
 
@@ -926,6 +949,7 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
         for (int r = tid; r < m; r += 32 * U)
           gsc[r] = r == victim ? NS[m] : NS[r];
         const int slot = victim < 0 ? m : (victim < m ? victim : -1);
+        bool finite = true;
         if (kRkv && w == 0) {
           // The sum of the rows that stay, for the next step.
           if (victim == m) {  // the new row itself: lanes 0-15 hold its key
@@ -940,10 +964,14 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
           float kv[4];
           key4(reinterpret_cast<const unsigned char *>(&vk), 0, kv);
           const float inv = inv_norm(kv);
-          reinterpret_cast<float4 *>(c.rsum + jb.ug * 128)[lane] =
-              make_float4(fmaf(kv[0], -inv, S4[0]), fmaf(kv[1], -inv, S4[1]),
-                          fmaf(kv[2], -inv, S4[2]), fmaf(kv[3], -inv, S4[3]));
-          __syncwarp();  // the victim's key has been read
+          const float4 S = make_float4(fmaf(kv[0], -inv, S4[0]), fmaf(kv[1], -inv, S4[1]),
+                                       fmaf(kv[2], -inv, S4[2]), fmaf(kv[3], -inv, S4[3]));
+          reinterpret_cast<float4 *>(c.rsum + jb.ug * 128)[lane] = S;
+          // A key that is not finite must not outlive its row in the sum.  (The
+          // vote also orders the reads of the victim's key before its slot's
+          // new row.)
+          finite = __all_sync(0xffffffffu, isfinite(S.x) && isfinite(S.y) && isfinite(S.z) &&
+                                               isfinite(S.w));
         }
         if (w == 0) {
           if (slot >= 0) {
@@ -959,7 +987,7 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
           if (lane == 0) {
             c.state[4 * jb.ug] = victim < 0 ? m + 1 : m;
             c.state[4 * jb.ug + 1] = t + 1;
-            c.state[4 * jb.ug + 2] = kRkv ? 1 : 0;  // the kept R-KV key sum
+            c.state[4 * jb.ug + 2] = kRkv && finite ? 1 : 0;  // the kept R-KV key sum
           }
         }
       }
@@ -1020,7 +1048,7 @@ cudaError_t launch_chunk_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
     // Units whose kept key sum another call has left stale, first.
     const int units = p.c.S * p.nl * p.c.H;
     const cudaError_t e =
-        launch_pdl(rkv_sum_kernel, dim3(units), dim3(128), 0, st, p.c, p.lb, p.nl);
+        launch_pdl(rkv_sum_kernel, dim3(units), dim3(256), 0, st, p.c, p.lb, p.nl);
     if (e != cudaSuccess) return e;
     return p.warps == 4 ? launch_k<false, true, 4>(tmK, tmV, tmK, tmV, p, grid, smem, st)
                         : launch_k<false, true, 2>(tmK, tmV, tmK, tmV, p, grid, smem, st);

@@ -55,11 +55,12 @@ struct CacheView {
   void *V;          // [u][cap][d]
   float *score;     // [u][sstride]
   int32_t *pos;     // [u][sstride]
-  int32_t *state;   // [u][4]: live length, next position, rsum valid, 0
+  int32_t *state;   // [u][4]: live length, next position, rsum valid, steps
+                    // that the chunked kernel has kept rsum for
   unsigned *err;    // device error word
   float *logits;    // [u][G][cap] scratch for units beyond on-chip size
   float *rsum;      // [u][d] R-KV: sum of the live rows' normalised keys,
-                    // kept by kvr_decode_step_rkv's one-launch step; valid
+                    // kept by kvr_decode_step_rkv's fused and chunked steps; valid
                     // while the unit's state word 2 is 1 (every other call
                     // that changes the unit's rows writes 0 there)
   int S, L, H, G, d, cap;
@@ -75,6 +76,12 @@ struct CacheView {
   // wait runs out and the launch ends with ERR_TIMEOUT.
   int hold_first;
 };
+
+// Index of unit x in [0, S * nl * H) of a call over layers [lb, lb + nl).
+__device__ __forceinline__ size_t unit_index(const CacheView &c, int lb, int nl, int x) {
+  const int h = x % c.H, lr = (x / c.H) % nl, s = x / (c.H * nl);
+  return ((size_t)s * c.L + lb + lr) * c.H + h;
+}
 
 // Work description of one decode call over layers [lb, lb + nl).
 struct StepArgs {
@@ -333,11 +340,6 @@ cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
 bool can_settle(const CacheView &c, int max_rows);
 cudaError_t launch_evict_absorbed(const AbsorbParams &p, int budget, int window,
                                   int sms, cudaStream_t st);
-// Index of unit x in [0, S * nl * H) of a call over layers [lb, lb + nl).
-__device__ __forceinline__ size_t unit_index(const CacheView &c, int lb, int nl, int x) {
-  const int h = x % c.H, lr = (x / c.H) % nl, s = x / (c.H * nl);
-  return ((size_t)s * c.L + lb + lr) * c.H + h;
-}
 // Where a call keeps its ties: in the units' R-KV key sums, which an absorb
 // makes stale.  Of the call's first unit: how many units are listed; of its
 // e-th: entry e, a unit's index in the call; of a listed unit: its tied rows.

@@ -69,3 +69,75 @@ def test_rkv_chunked_duplicate_and_zero_keys():
     rkv_lockstep(c, o, w, 141, 1, n - 2, 2, 0.0, fused=True)
     kept = c.export(0, kv=False)["pos"][0, 0, :n].tolist()
     assert 145 not in kept and {20, 50, 140, 152} <= set(kept)
+
+
+def _kept_sum(c):
+    """The units' kept key sums: the cache buffer's last array."""
+    n = c.S * c.L * c.H * c.d * 4
+    need = c.buf.numel() // 256 * 256
+    return c.buf[need - n:need].view(torch.float32).view(c.S, c.L, c.H, c.d)
+
+
+def _rkv_steps(caches, steps, seed, B, W, mark=None):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    for _ in range(steps):
+        c = caches[0]
+        q, k, v = (torch.randn(c.S, c.L, h, c.d, generator=gen, device="cuda")
+                   .bfloat16() for h in (c.H * c.G, c.H, c.H))
+        if mark is not None:
+            q[..., 0] = mark
+        for x in caches:
+            x.step_rkv(q, k, v, B, W, 0.1)
+
+
+def test_rkv_chunked_kept_sum_is_formed_anew():
+    """What the kept sum is off by does not outlive 64 steps: 66 steps after it
+    was spoilt, and after 2,000 steps, it is the sum of the live rows' keys.
+    Bound: the roundings of 64 steps and of a sum of 208 keys, 340 of 2^-24 of
+    partial sums below 40, taken as if all fell one way."""
+    B, W, S, H = 200, 8, 2, 2
+    c = harness.guarded_cache(S, 1, H, 7, 128, B + W + 1, kv_dtype="bf16",
+                              out_dtype="bf16")
+    for s in range(S):
+        c.load(s, *(torch.randn(1, H, B + W, 128, device="cuda").bfloat16()
+                    for _ in range(2)))
+
+    def worst():
+        k = torch.stack([torch.from_numpy(c.export(s)["K"][:, :, :B + W])
+                         for s in range(S)]).double()
+        want = torch.nn.functional.normalize(k, dim=-1).sum(-2)
+        return (_kept_sum(c).cpu().double() - want).abs().max().item()
+    _rkv_steps([c], 2, 1, B, W)
+    assert worst() < 340 * 2.0 ** -24 * 40
+    _kept_sum(c)[0, 0, 1] += 0.25
+    _rkv_steps([c], 66, 2, B, W)
+    assert worst() < 340 * 2.0 ** -24 * 40
+    _rkv_steps([c], 2000, 3, B, W)
+    assert worst() < 340 * 2.0 ** -24 * 40
+
+
+def test_rkv_chunked_infinite_key_leaves_with_its_row():
+    """A key with an infinite element (its logits are -inf, its probability 0)
+    makes its unit's sum, and every z, NaN while its row lives.  The row is the
+    first to go (of equal z the highest position), and the steps after it rank
+    as a cache that forms the sum anew does."""
+    B, W = 200, 8
+    c, d = (harness.guarded_cache(1, 1, 2, 8, 128, B + W + 1, kv_dtype="bf16",
+                                  out_dtype="bf16") for _ in range(2))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(8)
+    k, v = (torch.randn(1, 2, B + W, 128, generator=gen, device="cuda").bfloat16()
+            for _ in range(2))
+    k[0, 0, B, 0] = float("inf")  # (the newest candidate once a row is appended)
+    c.load(0, k, v)
+    _rkv_steps([c], 1, 9, B, W, mark=-1.0)
+    e = c.export(0)
+    assert np.isfinite(e["K"][..., :B + W, :]).all()
+    assert B not in e["pos"][0, 0, :B + W]
+    for t in range(3):
+        d.import_state(0, c.export(0))
+        _rkv_steps([c, d], 1, 10 + t, B, W, mark=-1.0)
+        a, b = c.export(0, kv=False), d.export(0, kv=False)
+        assert np.array_equal(a["pos"][..., :B + W], b["pos"][..., :B + W])
+    c.sync_status()
