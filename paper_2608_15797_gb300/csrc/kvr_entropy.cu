@@ -184,10 +184,25 @@ __device__ __forceinline__ void to_float(const uint4 &w,
 // Add the vectors v[k] (k < K, those with ok[k]) to acc: the fast path,
 // with the careful path redoing the batch on a non-finite result.  A thread
 // with no reference yet takes the largest logit of its first vector.
-template <bool kBf16, int K>
+// kTrack: the careful path alone, whose reference follows the largest logit.
+// The fast one keeps its first reference, and where a far larger logit follows,
+// log(s) and t / s are both large and their difference, the entropy, is left
+// with fewer bits (relative error up to 5e-6, against some 1e-7).
+template <bool kBf16, bool kTrack = false, int K>
 __device__ __forceinline__ void add_vectors(Online &acc, const uint4 (&v)[K],
                                             const bool (&ok)[K], float c) {
   constexpr int kPer = kBf16 ? 8 : 4;
+  if constexpr (kTrack) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      if (ok[k]) {
+        float x[kPer];
+        to_float<kBf16>(v[k], x);
+        acc.add(x, c);
+      }
+    }
+    return;
+  }
   if (!(fabsf(acc.mx) < INFINITY) && ok[0]) {
     float x[kPer];
     to_float<kBf16>(v[0], x);
@@ -305,8 +320,8 @@ __device__ void finish_row(const EntropyView &v, const StepIO &io, int r,
 // (at most 7 and 7) go with the last piece.  It is bound by the loads in
 // flight: with one logit a thread and load, as unaligned rows used to be read,
 // 512 rows of 50,001 logits took 36.5 us (bf16) and 41.4 (fp32) a call, with
-// vectors 18.6 and 26.8.
-template <bool kBf16>
+// vectors 19.5 and 26.7.
+template <bool kBf16, bool kTrack>
 __global__ void __launch_bounds__(kThreads, 4)
     entropy_kernel(const EntropyView v, const StepIO io) {
   kvr::pdl_begin();
@@ -343,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       ok[u] = i < nvec;
       w[u] = ok[u] ? __ldcs(vec + i) : make_uint4(0, 0, 0, 0);
     }
-    add_vectors<kBf16, kUnroll>(acc, w, ok, c);
+    add_vectors<kBf16, kTrack>(acc, w, ok, c);
   }
   if (p == v.pieces - 1) {
     const int body = nvec * kPer;
@@ -568,7 +583,7 @@ __global__ void __launch_bounds__(kSThreads, 3)
         ok[k] = i < h.z;
         w[k] = ok[k] ? src[i] : make_uint4(0, 0, 0, 0);
       }
-      add_vectors<kBf16, kV>(acc, w, ok, c);
+      add_vectors<kBf16>(acc, w, ok, c);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
       if (h.w & F_ROW_END) {
@@ -799,8 +814,9 @@ kvr_status kvr_entropy_step(kvr_entropy *det, const void *logits,
     ++det->launches;
     return KVR_OK;
   }
-  e = kvr::launch_pdl(bf16 ? entropy_kernel<true> : entropy_kernel<false>, grid,
-                      dim3(kThreads), 0, st, det->v, io);
+  auto kern = bf16 ? (vec ? entropy_kernel<true, false> : entropy_kernel<true, true>)
+                   : (vec ? entropy_kernel<false, false> : entropy_kernel<false, true>);
+  e = kvr::launch_pdl(kern, grid, dim3(kThreads), 0, st, det->v, io);
   if (e != cudaSuccess) return cuda_fail("kvr_entropy_step", e);
   ++det->launches;
   return KVR_OK;

@@ -186,6 +186,22 @@ def test_entropy_unaligned_row_vectors(dtype, vocab, stride):
     run_lockstep(9, vocab, 26, dtype, stride=stride)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_entropy_unaligned_rows_follow_the_largest_logit(dtype):
+    """Three peaks far above a row's first logits.  Terms kept relative to one of
+    those would leave log(s) and t / s at 60 to 120 and their difference, the
+    entropy (about 1), with errors of 2^-24 of that, some 5e-6; relative to the
+    largest logit they are a few 2^-24 of the entropy."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    x = torch.randn(128, 5001, generator=g, device="cuda")
+    x[:, 2500:2503] += 40 + 40 * torch.rand(128, 1, generator=g, device="cuda")
+    x = x.to(kvr.TORCH_DTYPES[dtype])
+    h = kvr.EntropyDetector(128, 5001, logits_dtype=dtype).step(x)[0].double()
+    want = torch.special.entr(torch.softmax(x.double(), -1)).sum(-1)
+    assert ((h - want) / (want + 0.1)).square().mean().sqrt().item() < 5e-7
+
+
 def test_entropy_temperature_window_guard_variants():
     run_lockstep(8, 5000, 30, "bf16", window=1, guard=0, tau=6.5)
     run_lockstep(8, 5000, 30, "f32", window=64, guard=3, tau=7.5,
