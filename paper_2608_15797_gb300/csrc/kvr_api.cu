@@ -546,6 +546,7 @@ bool try_long_step(kvr_cache *c, const StepArgs &a, cudaStream_t stream,
   if (!aligned16(a.q) || !aligned16(a.k_new) || !aligned16(a.v_new) ||
       !aligned16(a.out))
     return false;
+  if (!device_facts(c)) return false;
   const std::pair<CUtensorMap, CUtensorMap> *maps =
       slab_maps(c, kvr::split_rows_per_stage());
   if (!maps) return false;
@@ -568,7 +569,7 @@ bool try_long_step(kvr_cache *c, const StepArgs &a, cudaStream_t stream,
     });
   }
   *err = kvr::launch_long_step(maps->first, maps->second, p, order, a.max_rows,
-                               a.out, stream);
+                               c->sm_count, a.out, stream);
   return true;
 }
 

@@ -214,7 +214,7 @@ struct SeqOrder {
 };
 cudaError_t launch_long_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                              const SplitParams &p, const SeqOrder &order,
-                             int max_rows, void *out, cudaStream_t st);
+                             int max_rows, int sms, void *out, cudaStream_t st);
 
 // Candidates of one cache (kvr_fork.cu).  A candidate unit cu = c * units + u.
 struct ForkView {

@@ -391,7 +391,6 @@ __global__ void __launch_bounds__(128) split_combine_kernel(const SplitParams p,
 
 constexpr int kCluster = 8;         // CTAs a cluster, at most
 constexpr int kClusterRows = 1024;  // rows a CTA should have
-constexpr int kFillCtas = 400;      // about one for each of an SM's three places
 
 __device__ __forceinline__ void cluster_sync() {
   asm volatile(
@@ -565,7 +564,7 @@ cudaError_t launch_split_attend(const CUtensorMap &tmK, const CUtensorMap &tmV,
 
 cudaError_t launch_long_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
                              const SplitParams &p, const SeqOrder &order, int max_rows,
-                             void *out, cudaStream_t st) {
+                             int sms, void *out, cudaStream_t st) {
   const int smem = SmemLayout::bytes + 1024;
   cudaLaunchConfig_t cfg = {};
   // Eight CTAs a unit only where its rows or the launch's width ask for them:
@@ -574,7 +573,8 @@ cudaError_t launch_long_step(const CUtensorMap &tmK, const CUtensorMap &tmV,
   // 224).
   const int units = p.c.S * p.nl * p.c.H;
   int nc = 1;
-  while (nc < kCluster && (max_rows > nc * kClusterRows * 2 || units * nc < kFillCtas)) nc *= 2;
+  const int fill = 8 * sms / 3;  // about one for each of an SM's three places
+  while (nc < kCluster && (max_rows > nc * kClusterRows * 2 || units * nc < fill)) nc *= 2;
   cfg.gridDim = dim3(nc, units);
   cfg.blockDim = dim3(32 * kWarps);
   cfg.dynamicSmemBytes = smem;
