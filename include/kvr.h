@@ -275,16 +275,17 @@ void kvr_fork_destroy(kvr_fork *fork);
 
 /* Which kernel runs the fork's candidate steps (for testing and
  * measurement; every choice computes the same step, Sec. 2.2 Eq. 2).
- * kernel: 0 = the library's choice (5, at any lengths, for four candidates and
- * more over many units; else the first of 1, 2, 3 that applies, else 4); 1 = candidate-batched (bf16, head_dim 128, G <= 8, N <= 8: a
- * warp per candidate, each prefix row read once per unit for all
- * candidates); 2 = chunked (one job per candidate and unit); 3 = one CTA per
- * unit; 4 = generic; 5 = candidate-batched on 5th-generation tensor cores
- * (bf16, head_dim 128, G <= 8, N <= 8, at most 128 parent rows and 64 tail
- * rows before the append: the N x G query rows of a unit are one
- * contraction against each block of the prefix and of all tails).  A choice that does not
- * apply to a call runs the generic kernel for that call.  Returns
- * KVR_EINVAL outside [0, 5]. */
+ * kernel: 0 = the library's choice (5, whatever the prefix, for four candidates
+ * and more over many units unless their tails are long for the prefix; else
+ * the first of 1, 2, 3 that applies, else 4); 1 = candidate-batched (bf16,
+ * head_dim 128, G <= 8, N <= 8: a warp per candidate, each prefix row read once
+ * per unit for all candidates); 2 = chunked (one job per candidate and unit);
+ * 3 = one CTA per unit; 4 = generic; 5 = candidate-batched on 5th-generation
+ * tensor cores (bf16, head_dim 128, G <= 8, N <= 8; asked for, at most 128 parent
+ * rows and 64 tail rows before the append: the N x G query rows of a unit are
+ * one contraction against each block of the prefix and of all tails).  A
+ * choice that does not apply to a call runs the generic kernel for that call.
+ * Returns KVR_EINVAL outside [0, 5]. */
 kvr_status kvr_fork_set_kernel(kvr_fork *fork, int kernel);
 
 /* The kernel (1..5, numbered as for kvr_fork_set_kernel) that ran the

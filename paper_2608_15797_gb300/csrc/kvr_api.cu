@@ -1515,22 +1515,47 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
   for (int s = 0; s < p->desc.n_seq && nt_same; ++s)
     for (int l = lb; l < le; ++l)
       nt_same = nt_same && f->tlen[(size_t)s * p->desc.n_layers + l] == nt_max;
+  // What the warp-a-candidate and the chunked kernel (0 = the library's first
+  // and second choice) could take.
+  const bool mma16 = p->fused && pv.kv_bf16 && pv.d == 128 && pv.G <= 8 &&
+                     (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
+                     aligned16(q) && aligned16(k_new) && aligned16(v_new) &&
+                     aligned16(out) && device_facts(p);
+  const bool batch_fits = mma16 && f->batch_maps &&
+      f->view.N <= kvr::fork_batch_max_cand() &&
+      kvr::fork_batch_smem_bytes(n_max, f->view.N) + 512 <= (size_t)p->smem_optin;
+  kvr::ChunkParams cp{};
+  cp.fork = 1;
+  const bool chunk_fits = mma16 && p->chunk_groups >= 0 && f->tail_maps &&
+      n_max <= kvr::chunk_max_rows() && chunk_config(p, n_max, 0, &cp);
   // By itself the library takes tiles on the tensor cores for four candidates
   // and more where every SM gets several units: a tile costs the same for any
   // number of candidates, and its long chain of steps wants other units to
   // hide behind.  72B geometry, 64 + 8 rows, a fork of 16 tokens and commit,
   // against one warp a candidate: 640 units, N = 8: 637 and 774 us, N = 4: 576
   // and 598, N = 2: 566 and 542; 2,560 units, N = 8: 1,786 and 2,482, N = 4: 1,640
-  // and 1,915; 448 units (7B), N = 8: 490 and 511, N = 4: 455 and 405.  Asked for
-  // (kernel 5), within the limits that choice has.
-  const int call_units = pv.S * (le - lb) * pv.H;
+  // and 1,915; 448 units (7B), N = 8: 490 and 511, N = 4: 455 and 405.
+  // A tail block holds 16 (8 / N) rows of each candidate against 128 of the
+  // prefix, so that tails that are long for the prefix go elsewhere.  us a
+  // token, tiles against the kernel that would run (2,560 units of 72B | 672 of
+  // 7B, N = 8 unless said):
+  //   one warp a candidate, prefix 16: tail 24 143, 143 | 46, 42;
+  //     72: 40 192, 209 | 65, 67; 64 284, 273 | 93, 85; 192 640, 530;
+  //     136: 48 288, 298 | 94, 93; 96 422, 388; N = 4, 72: 64 179, 180 | 61, 57;
+  //     N = 6, 200: 64 301, 317 | 97, 97; N = 5, 300: 96 405, 420;
+  //   chunked, prefix 300: 128 581, 848 | 182, 226; 256 | 291, 289;
+  //     N = 6: 192 659, 727 | 207, 196; N = 4: 96 340, 411 | 106, 110;
+  //     200: 96 439, 532 | 137, 141, N = 6 382, 412 | 122, 110.
+  // Asked for (kernel 5): within the limits that choice has.
+  const int call_units = pv.S * (le - lb) * pv.H, N = f->view.N;
+  const bool tile_best = N >= 4 && call_units >= 4 * p->sm_count &&
+      (batch_fits   ? max_prefix >= 48 &&
+                          nt_max <= 32 + max_prefix / (N == 5 || N == 6 ? 5 : 8)
+       : chunk_fits ? nt_max <= max_prefix / (N >= 7 ? 2 : 3)
+                    : true);
   CUtensorMap tile_q, tile_k, tile_v;
-  const bool tile_ok =
-      (want == 0 || (want == 5 && max_prefix <= 128 && nt_max <= 64)) && p->fused && pv.kv_bf16 && pv.d == 128 && nt_same && pv.G <= 8 &&
-      f->view.N <= kvr::fork_tile_max_cand() && device_facts(p) &&
-      (want == 5 || (f->view.N >= 4 && call_units >= 4 * p->sm_count)) &&
-      (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
-      aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
+  const bool tile_ok = mma16 && nt_same && f->view.N <= kvr::fork_tile_max_cand() &&
+      (want == 0 ? tile_best : want == 5 && max_prefix <= 128 && nt_max <= 64) &&
       (maps = slab_maps(p, kvr::fork_tile_box_rows())) != nullptr &&
       encode_cand_q(&tile_q, q, pv.G, (size_t)call_units, f->view.N) &&
       encode_tail_tile(&tile_k, f->view.TK, std::max(nt_max, 1), f->view.tcap,
@@ -1539,31 +1564,15 @@ kvr_status kvr_fork_decode_attend_score(kvr_fork *f, int lb, int le,
       encode_tail_tile(&tile_v, f->view.TV, std::max(nt_max, 1), f->view.tcap,
                        (size_t)pv.S * pv.L * pv.H, f->view.N,
                        kvr::fork_tile_tail_rows(f->view.N));
-  const bool batch_ok = !tile_ok &&
-      (want == 0 || want == 1) && p->fused && f->batch_maps && pv.G <= 8 &&
-      f->view.N <= kvr::fork_batch_max_cand() && device_facts(p) &&
-      kvr::fork_batch_smem_bytes(n_max, f->view.N) + 512 <=
-          (size_t)p->smem_optin &&
-      (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
-      aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
+  const bool batch_ok = !tile_ok && (want == 0 || want == 1) && batch_fits &&
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr &&
       (maps128 = slab_maps(p, kvr::fork_batch_prefix_box_rows())) != nullptr;
-  kvr::ChunkParams cp{};
-  cp.fork = 1;
-  const bool chunk_ok = !batch_ok && !tile_ok && (want == 0 || want == 2) &&
-      p->fused && p->chunk_groups >= 0 && f->tail_maps && pv.G <= 8 &&
-      n_max <= kvr::chunk_max_rows() && device_facts(p) &&
-      chunk_config(p, n_max, 0, &cp) &&
-      (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
-      aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
+  const bool chunk_ok = !batch_ok && !tile_ok && (want == 0 || want == 2) && chunk_fits &&
       (maps = slab_maps(p, kvr::chunk_box_rows())) != nullptr;
   const bool mma_ok = !batch_ok && !tile_ok && !chunk_ok && (want == 0 || want == 3) &&
-      p->fused && f->tail_maps && pv.G <= 8 &&
-      f->view.N <= kvr::fork_mma_max_cand() && device_facts(p) &&
+      mma16 && f->tail_maps && f->view.N <= kvr::fork_mma_max_cand() &&
       kvr::fork_mma_smem_bytes(max_prefix, nt_max, f->view.N) + 512 <=
           (size_t)p->smem_optin &&
-      (size_t)pv.S * pv.L * pv.H * pv.cap < (size_t)INT32_MAX &&
-      aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out) &&
       (maps = slab_maps(p, kvr::fork_mma_box_rows())) != nullptr;
   if (tile_ok) {
     kvr::ForkTileParams tp{};

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2608_15797_gb300 import inputs
+from paper_2608_15797_gb300 import inputs, kvr
 from tests import harness
 
 pytestmark = pytest.mark.gpu
@@ -37,15 +37,15 @@ def test_fork_tile_shapes(N, G, lens, tokens, out_dtype):
 
 
 def test_fork_tile_is_the_choice_for_many_units():
-    """608 units (four for each SM) of ragged prefixes up to three blocks, N = 8,
+    """Four units for each SM, of ragged prefixes up to three blocks, N = 8,
     tails crossing a block: every CTA works through several units, reusing
     its buffers.  Three candidates, or half the layers, go elsewhere."""
-    w = inputs.Workload("fm", 38, 4, 1, 128, "bf16", 24, 8, 0, 0, sigma=1.0)
+    layers = -(-torch.cuda.get_device_properties(0).multi_processor_count // 4)
+    w = inputs.Workload("fm", layers, 4, 1, 128, "bf16", 24, 8, 0, 0, sigma=1.0)
     c, o = harness.make_pair(w, 170, 4, cap=280, prompt_lens=[257, 7, 129, 0],
                              out_dtype="bf16")
     _, _, st = harness.fork_lockstep(c, o, w, 170, 8, 18, w.budget, w.window)
-    if torch.cuda.get_device_properties(0).multi_processor_count <= 152:
-        assert st.kernels == [5] * 18
+    assert st.kernels == [5] * 18
     q, k, v = (np.stack([x, x, x]) for x in inputs.step_inputs(w, 170, 900, 4))
     dq, dk, dv = (harness.dev(a, w.dtype) for a in (q, k, v))
     f = harness.guarded_fork(c, 3, 2)
@@ -71,3 +71,25 @@ def test_fork_tile_layer_ranges():
     assert g.last_kernel() == 5
     assert torch.equal(whole, torch.cat(part, 2))
     harness.check_guards(c, g)
+
+
+# (N, prefix, the first tail that goes elsewhere, the kernel it goes to): against
+# one warp a candidate, against the chunked kernel, and a prefix too short.
+@pytest.mark.parametrize("N,prefix,last,other", [
+    (8, 72, 42, 1), (4, 136, 50, 1), (8, 20, 0, 1), (8, 300, 151, 2),
+    (5, 330, 99, 1)])
+def test_long_tails_go_elsewhere(N, prefix, last, other):
+    layers = torch.cuda.get_device_properties(0).multi_processor_count
+    c = kvr.Cache(1, layers, 4, 1, 128, prefix + 1, kv_dtype="bf16",
+                  out_dtype="bf16")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+
+    def rnd(*shape):
+        return torch.randn(shape, generator=g, device="cuda").bfloat16()
+    c.load(0, rnd(layers, 4, prefix, 128), rnd(layers, 4, prefix, 128))
+    f = kvr.Fork(c, N, last + 1)
+    q, k, v = (rnd(N, 1, layers, 4, 128) for _ in range(3))
+    for t in range(last + 1):
+        f.attend_score(q, k, v)
+        assert f.last_kernel() == (5 if t < last else other), f"tail {t}"
