@@ -91,7 +91,8 @@ __device__ __forceinline__ bool unit_ok(const AbsorbParams &p, const LUnit &u) {
 
 // ---- 1. append ----------------------------------------------------------------
 
-constexpr int kAppendRows = 32;  // rows a CTA copies
+constexpr int kAppendRows = 32;    // rows a CTA copies at a time
+constexpr int kAppendCtas = 1024;  // CTAs a unit, at most
 
 __global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) {
   pdl_begin();
@@ -114,22 +115,25 @@ __global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) 
       atomicOr(c.err, u.m >= 0 && u.m + p.chunk > c.cap ? ERR_CAPACITY : ERR_LENGTH);
     return;
   }
-  const int j0 = blockIdx.y * kAppendRows, nr = min(kAppendRows, p.chunk - j0);
-  const size_t dst = u.ug * (size_t)c.cap + u.m + j0;
   const int4 *kn = reinterpret_cast<const int4 *>(p.k_new);
   const int4 *vn = reinterpret_cast<const int4 *>(p.v_new);
-  int4 *K = reinterpret_cast<int4 *>(c.K) + dst * 16;
-  int4 *V = reinterpret_cast<int4 *>(c.V) + dst * 16;
-  for (int i = threadIdx.x; i < nr * 16; i += 256) {
-    const size_t src = ((u.row0 + j0 + (i >> 4)) * c.H + u.h) * 16 + (i & 15);
-    const int4 a = kn[src], b = vn[src];
-    K[i] = a;
-    V[i] = b;
-  }
-  if ((int)threadIdx.x < nr) {
-    const size_t s = u.ug * (size_t)c.sstride + u.m + j0 + threadIdx.x;
-    c.score[s] = 0.f;
-    c.pos[s] = c.state[4 * u.ug + 1] + j0 + (int)threadIdx.x;
+  const int next = c.state[4 * u.ug + 1];
+  for (int j0 = blockIdx.y * kAppendRows; j0 < p.chunk; j0 += gridDim.y * kAppendRows) {
+    const int nr = min(kAppendRows, p.chunk - j0);
+    const size_t dst = u.ug * (size_t)c.cap + u.m + j0;
+    int4 *K = reinterpret_cast<int4 *>(c.K) + dst * 16;
+    int4 *V = reinterpret_cast<int4 *>(c.V) + dst * 16;
+    for (int i = threadIdx.x; i < nr * 16; i += 256) {
+      const size_t src = ((u.row0 + j0 + (i >> 4)) * c.H + u.h) * 16 + (i & 15);
+      const int4 a = kn[src], b = vn[src];
+      K[i] = a;
+      V[i] = b;
+    }
+    if ((int)threadIdx.x < nr) {
+      const size_t s = u.ug * (size_t)c.sstride + u.m + j0 + threadIdx.x;
+      c.score[s] = 0.f;
+      c.pos[s] = next + j0 + (int)threadIdx.x;
+    }
   }
 }
 
@@ -879,7 +883,8 @@ cudaError_t launch_absorb_long(const CUtensorMap &tmK, const CUtensorMap &tmV,
   // chunk * G of its G * cap.
   float *lse = p.c.logits;
   e = launch_pdl(long_append_kernel,
-                 dim3(units, (p.chunk + kAppendRows - 1) / kAppendRows), dim3(256), 0, st, p);
+                 dim3(units, min((p.chunk - 1) / kAppendRows + 1, kAppendCtas)), dim3(256), 0,
+                 st, p);
   if (e != cudaSuccess) return e;
   const int n_att = units * n_qt, n_sc = units * n_kp;
   e = launch_pdl(long_attend_kernel, dim3(n_att < 2 * sms ? n_att : 2 * sms), dim3(kAttThr),

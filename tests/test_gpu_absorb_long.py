@@ -88,3 +88,31 @@ def test_absorb_long_layer_range():
     e = c.export(0, kv=False)
     assert (e["score"][0, :, :200] == 0).all()
     c.sync_status()
+
+
+def test_absorb_long_prompt_beyond_one_append_grid():
+    """33,000 tokens in one call: more rows than the append's CTAs take in one
+    round.  Sampled tokens' outputs against fp64; every row in its slot."""
+    n = 33_000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    q, k, v = (torch.randn(1, 1, n, 1, 128, generator=g, device="cuda").bfloat16()
+               for _ in range(3))
+    c = harness.guarded_cache(1, 1, 1, 1, 128, n, kv_dtype="bf16",
+                              out_dtype="bf16")
+    out = c.absorb(q, k, v, evict=False)[0, 0, :, 0]
+    assert c.last_absorb_kernel() == 3
+    c.sync_status()
+    score, pos, _ = c.scores_view()
+    assert (pos[0, 0, 0, :n].cpu() == torch.arange(n)).all()
+    # every token's probabilities sum to one
+    assert abs(score[0, 0, 0, :n].double().sum().item() - n) < 1e-5 * n
+    e = c.export(0)
+    assert (torch.from_numpy(e["K"][0, 0]) == k[0, 0, :, 0].float().cpu()).all()
+    kk, vv = k[0, 0, :, 0].double(), v[0, 0, :, 0].double()
+    for t in (0, 1, 127, 128, 20_000, 32_767, 32_768, n - 1):
+        p = torch.softmax(kk[:t + 1] @ q[0, 0, t, 0].double() / 128 ** 0.5, 0)
+        ref = p @ vv[:t + 1]
+        # one rounding to bf16 of outputs, fp32 sums before it
+        assert ((out[t].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 2e-5).all()
+    harness.check_guards(c)
