@@ -339,6 +339,12 @@ kvr_status kvr_cache_set_fused_tuning(kvr_cache *cache, int groups,
 kvr_status kvr_cache_set_chunk_tuning(kvr_cache *cache, int groups,
                                       int stages);
 
+/* How the cache's last step on the chunked kernel ran (for testing and
+ * measurement): its consumer groups per SM, and in *warps (if given) the warps
+ * of a group, 2 or 4; 0 and 0 before the first one or for NULL.  Host state
+ * only: no synchronisation. */
+int kvr_cache_last_chunk_groups(const kvr_cache *cache, int *warps);
+
 /* Absorb a chunk of `chunk` tokens per sequence in one call, and optionally
  * cut every unit back to B + W once afterwards (Algorithm 1: when a helper
  * step is accepted, the base model encodes its tokens in a single forward

@@ -104,7 +104,9 @@ struct kvr_cache {
   int chunk_groups = 0;           // chunked kernel: groups (0 auto, -1 off)
   int chunk_stages = 0;           // chunked kernel: stages per group (0 auto)
   int absorb_kernel = 0;          // 0 tcgen05, 1 mma.sync (kvr_absorb_chunk)
-  int last_absorb = -1;           // kernel of the last kvr_absorb_chunk (0, 1, 2)
+  int last_absorb = -1;           // how the last kvr_absorb_chunk ran (0..3)
+  int last_chunk_groups = 0;      // of the last chunked step: groups,
+  int last_chunk_warps = 0;       // warps a group
   int forks = 0;                  // live forks: the cache is read-only meanwhile
   int sm_count = 0;               // of the device, queried on first use
   int smem_optin = 0;
@@ -531,6 +533,8 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
   const int grid = std::min(c->sm_count, p.n_jobs);
   *err = kvr::launch_chunk_step(maps->first, maps->second, nullptr, nullptr, p,
                                 grid, stream);
+  c->last_chunk_groups = p.n_groups;
+  c->last_chunk_warps = p.warps;
   return true;
 }
 
@@ -1742,6 +1746,11 @@ kvr_status kvr_fork_export(const kvr_fork *f, int cand, int seq,
 }
 
 int kvr_fork_last_kernel(const kvr_fork *f) { return f ? f->last_kernel : 0; }
+
+int kvr_cache_last_chunk_groups(const kvr_cache *c, int *warps) {
+  if (warps) *warps = c ? c->last_chunk_warps : 0;
+  return c ? c->last_chunk_groups : 0;
+}
 
 int kvr_cache_last_absorb_kernel(const kvr_cache *c) { return c ? c->last_absorb : -1; }
 

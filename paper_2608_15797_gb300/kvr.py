@@ -82,6 +82,7 @@ _SIGS = {
     "kvr_fork_last_kernel": (_I, [_P]),
     "kvr_cache_set_absorb_kernel": (_S, [_P, _I]),
     "kvr_cache_last_absorb_kernel": (_I, [_P]),
+    "kvr_cache_last_chunk_groups": (_I, [_P, _P]),
     "kvr_cache_scores": (_S, [_P, _P, _P, _P, _P]),
     "kvr_sync_status": (_S, [_P, _P]),
     "kvr_last_error": (ctypes.c_char_p, []),
@@ -450,6 +451,14 @@ class Cache:
         """kvr_absorb_chunk's one-launch kernel: 0 tcgen05, 1 mma.sync."""
         _check(lib.kvr_cache_set_absorb_kernel(self.handle, kernel),
                "kvr_cache_set_absorb_kernel")
+
+    def last_chunk_groups(self):
+        """(groups per SM, warps a group) of the last step on the chunked
+        kernel (kvr_cache_last_chunk_groups), (0, 0) before the first."""
+        warps = ctypes.c_int()
+        groups = lib.kvr_cache_last_chunk_groups(self.handle,
+                                                 ctypes.byref(warps))
+        return int(groups), warps.value
 
     def last_absorb_kernel(self) -> int:
         """How the last absorb ran (kvr_cache_last_absorb_kernel): 0 tcgen05,

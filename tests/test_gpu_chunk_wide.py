@@ -36,19 +36,23 @@ def test_plain_step_lengths(rows, G, out, chunk):
     n0 = c.launch_count()
     harness.lockstep(c, o, w, 200 + rows, 4, B, W)
     assert c.launch_count() - n0 == 4
+    assert c.last_chunk_groups() == ((1, 4) if chunk == (0, 0) else (2, 2))
     harness.check_guards(c)
 
 
-# (units, rows, R-KV): the lines of the rule that picks the groups, in units
-# an SM on 152 SMs.  Two; three (pairs); four and more at lengths below and
-# above the line; lengths at which two groups of four do not fit.
-@pytest.mark.parametrize("S,L,rows,rkv", [
-    (28, 10, 200, False), (45, 10, 400, False), (58, 10, 400, False),
-    (58, 10, 425, False), (88, 10, 425, False), (28, 10, 800, False),
-    (28, 10, 200, True), (58, 10, 489, True), (28, 10, 800, True)])
-def test_units_an_sm(S, L, rows, rkv):
+# (units an SM, rows, R-KV, warps a group): the lines of the rule that picks the
+# groups.  Two; three (pairs); four and six at lengths below and above the
+# line; lengths at which two groups of four do not fit.
+@pytest.mark.parametrize("per,rows,rkv,warps", [
+    (2, 200, False, 4), (3, 400, False, 2), (4, 400, False, 4),
+    (4, 425, False, 4), (6, 400, False, 2), (6, 425, False, 4),
+    (2, 800, False, 2), (2, 200, True, 4), (4, 489, True, 4),
+    (6, 470, True, 2), (2, 800, True, 2)])
+def test_units_an_sm(per, rows, rkv, warps):
     """Several units an SM; the oracle holds two of the sequences, one of
     them in the last round of units."""
+    L = 10
+    S = per * torch.cuda.get_device_properties(0).multi_processor_count // L
     B, W = rows - 9, 8
     w = inputs.Workload("cu", L, 1, 7, 128, "bf16", B, W, rows - 1, 0,
                         sigma=1.0)
@@ -59,6 +63,7 @@ def test_units_an_sm(S, L, rows, rkv):
                      sample=sample)
     else:
         harness.lockstep(c, o, w, 300 + rows, 2, B, W, sample=sample)
+    assert c.last_chunk_groups()[1] == warps
     harness.check_guards(c)
 
 
@@ -70,4 +75,5 @@ def test_rkv_groups_of_two(rows, G):
     c, o = harness.make_pair(w, 400 + rows, 2, cap=rows + 1,
                              prompt_lens=[rows - 1, rows - 40], chunk=(2, 2))
     rkv_lockstep(c, o, w, 400 + rows, 4, B, W, 0.1, fused=True)
+    assert c.last_chunk_groups() == (2, 2)
     harness.check_guards(c)
