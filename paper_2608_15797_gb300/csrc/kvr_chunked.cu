@@ -63,21 +63,6 @@ namespace {
 using namespace ptx;
 using dev::rkv_key;
 
-// Packed fp32 pairs (round to nearest, no flush).
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 constexpr int kBox = 16;      // rows per TMA box (and per MMA tile)
 constexpr int kMaxGroups = 4;
 // U consumer warps a group (2, or 4 in at most kWideGroups groups), one tile of
@@ -644,8 +629,10 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
           const __nv_bfloat162 hb0 = *reinterpret_cast<const __nv_bfloat162 *>(&h0);
           const __nv_bfloat162 hb1 = *reinterpret_cast<const __nv_bfloat162 *>(&h1);
           const uint32_t bp0 = movm_t(h0), bp1 = movm_t(h1);
-          const uint32_t bl0 = movm_t(pack_bf16(s4[0] - __low2float(hb0), s4[1] - __high2float(hb0)));
-          const uint32_t bl1 = movm_t(pack_bf16(s4[2] - __low2float(hb1), s4[3] - __high2float(hb1)));
+          const uint32_t bl0 =
+              movm_t(pack_bf16(s4[0] - __low2float(hb0), s4[1] - __high2float(hb0)));
+          const uint32_t bl1 =
+              movm_t(pack_bf16(s4[2] - __low2float(hb1), s4[3] - __high2float(hb1)));
           const int row = tr0 + (lane & 7) + ((lane >> 4) << 3);
           const uint32_t b0 = smem_u32(V0) + row * 128, b1 = smem_u32(V1) + row * 128;
 #pragma unroll

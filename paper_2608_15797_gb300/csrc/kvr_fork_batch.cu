@@ -47,21 +47,6 @@ namespace {
 
 using namespace ptx;
 
-// Packed fp32 pairs (round to nearest, no flush).
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 constexpr int kBox = 16;         // rows per partial-prefix TMA box, per MMA tile
 constexpr int kBlockRows = 128;  // rows of a block
 constexpr int kMaxCand = 8;

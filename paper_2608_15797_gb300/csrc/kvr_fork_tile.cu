@@ -16,11 +16,11 @@
 // (kvr_fork_batch.cu) pays both per candidate and is bound by its instruction
 // latencies.  72B geometry, 4 sequences, N = 8, 72 + up to 16 rows: 108 us a
 // token against 150; what bounds it is the chain of a unit's steps, about 2
-// to 4 thousand cycles each for two units an SM.  Per unit: S = Q K^T, online softmax, O += P V block by block
-// (P as two bf16 terms in tensor memory), then a second contraction with the
-// keys on the lanes for the scores, as in kvr_absorb_long.cu: a row's sum
-// over a candidate's heads is a sum inside one thread, and its probabilities
-// are exact because the normalisers are known.
+// to 4 thousand cycles each for two units an SM.  Per unit: S = Q K^T, online
+// softmax, O += P V block by block (P as two bf16 terms in tensor memory), then
+// a second contraction with the keys on the lanes for the scores, as in
+// kvr_absorb_long.cu: a row's sum over a candidate's heads is a sum inside one
+// thread, and its probabilities are exact because the normalisers are known.
 //  - Persistent, two CTAs an SM (256 TMEM columns, 101 KB each), a unit at a
 //    time; one CTA's waits are the other's tensor time.  Eight softmax warps
 //    (two for each 32 lanes, half of a block's columns each), a loading and an

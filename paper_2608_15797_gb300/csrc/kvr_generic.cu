@@ -18,6 +18,9 @@
 //   64-bit keys read from global memory eight times and block-wide list
 //   building, 47 now; 1,792 units of 697 rows: 96 and 33, and 54 when a warp
 //   moved one row at a time with half its lanes idle).
+// tie_sums_kernel, evict_tied_kernel: the end of a blocked absorb
+//   (kvr_absorb_long.cu) in units whose scores leave open which rows a
+//   token-by-token absorb would keep.
 #include <cuda_bf16.h>
 #include <math.h>
 

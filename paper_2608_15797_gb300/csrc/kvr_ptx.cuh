@@ -193,6 +193,30 @@ __device__ __forceinline__ float rcp(float x) {
   return y;
 }
 
+// Packed fp32 pairs (round to nearest, no flush: the scalar code's results).
+__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
 
 // ---- 5th-generation tensor cores (tcgen05) and tensor memory -------------
 // Shared-memory matrix descriptor of a 128B-swizzled operand (1024-byte
@@ -209,13 +233,11 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr, uint32_t lbo,
   d |= (uint64_t)2 << 61;  // 128-byte swizzle
   return d;
 }
-// Instruction descriptor of kind::f16 with bf16 A and B, fp32 D; A and B
-// each K-major or MN-major.
-__device__ __forceinline__ uint32_t idesc_bf16(int M, int N, bool b_mn_major,
-                                               bool a_mn_major = false) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major ? 1u << 15 : 0u) |
-         (b_mn_major ? 1u << 16 : 0u) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor of kind::f16 with bf16 A and B, fp32 D; A K-major, B
+// K-major or MN-major.
+__device__ __forceinline__ uint32_t idesc_bf16(int M, int N, bool b_mn_major) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? 1u << 16 : 0u) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // One warp: allocate `cols` TMEM columns (a power of two >= 32); the base
 // address lands in shared memory at dst.
@@ -253,18 +275,9 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
       : "memory");
 }
-// 16 consecutive 32-bit TMEM columns of this thread's lane, without waiting
-// (tmem_wait_ld() before the registers are read).
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,"
-      "%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-        "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
-        "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-}
-// The same into float registers (the bits of fp32 accumulators).
+// 16 consecutive 32-bit TMEM columns of this thread's lane into float registers
+// (the bits of fp32 accumulators), without waiting (tmem_wait_ld() before the
+// registers are read).
 __device__ __forceinline__ void tmem_ld16f_nowait(uint32_t taddr, float (&v)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,"

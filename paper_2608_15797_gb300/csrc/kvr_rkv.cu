@@ -26,38 +26,18 @@
 
 #include "kvr_device.cuh"
 #include "kvr_internal.h"
+#include "kvr_ptx.cuh"
 
 namespace kvr {
 namespace {
 
 using namespace dev;
-
-// Packed fp32 pairs (round to nearest, no flush).
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
+using ptx::fma2;
+using ptx::pk2;
+using ptx::upk2;
 
 using dev::ord_bits;
 using dev::rkv_key;
-
-// The unit of this CTA: blocks run over (sequence, layer in [lb, lb + nl),
-// KV head), head fastest.
-__device__ __forceinline__ size_t unit_index(const CacheView &c, int lb,
-                                             int nl) {
-  const int b = blockIdx.x;
-  const int h = b % c.H, lr = (b / c.H) % nl, s = b / (c.H * nl);
-  return ((size_t)s * c.L + lb + lr) * c.H + h;
-}
 
 template <typename Op>
 __device__ float block_reduce(float v, Op op, float *s_red) {
@@ -108,7 +88,7 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ float s_S[kWarps][D];
   extern __shared__ __align__(16) unsigned char dyn[];
 
-  const struct { size_t u; } x = {unit_index(c, lb, nl)};
+  const struct { size_t u; } x = {unit_index(c, lb, nl, blockIdx.x)};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = c.state[4 * x.u];
   if (n <= B + W) return;

@@ -1,32 +1,12 @@
 // kvr_tmem.cuh -- helpers of the kernels that keep logits, probabilities and
-// outputs in tensor memory: packed fp32 pairs, wide TMEM loads and stores,
-// MMAs with their A operand in TMEM.
+// outputs in tensor memory: wide TMEM loads and stores, MMAs with their A
+// operand in TMEM, and a query row's attention on its own.
 #pragma once
 
 #include "kvr_ptx.cuh"
 
 namespace kvr {
 namespace ptx {
-
-// Packed fp32 pairs (round to nearest, no flush).
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 
 // 32 consecutive TMEM columns of this thread's lane (no wait).
 __device__ __forceinline__ void tmem_ld32(uint32_t ta, float (&v)[32]) {
