@@ -98,17 +98,9 @@ __global__ void __launch_bounds__(256) long_append_kernel(const AbsorbParams p) 
   pdl_begin();
   const CacheView &c = p.c;
   const LUnit u = unit_at(p, blockIdx.x);
-  if (p.settle && blockIdx.y == 0) {
-    if (threadIdx.x == 0) {
-      c.state[4 * u.ug + 2] = 0;  // the key sum's place is the ties' now
-      if (blockIdx.x == 0) tie_words(c, u.ug)[kTieUnits] = 0;
-    }
-    // The scores before the call, behind the normalisers.
-    if (unit_ok(p, u)) {
-      float *old = c.logits + (u.ug + 1) * (size_t)c.G * c.cap - u.m;
-      for (int i = threadIdx.x; i < u.m; i += 256)
-        old[i] = c.score[u.ug * (size_t)c.sstride + i];
-    }
+  if (p.settle && blockIdx.y == 0 && threadIdx.x == 0) {
+    c.state[4 * u.ug + 2] = 0;  // the key sum's place is the ties' now
+    if (blockIdx.x == 0) tie_words(c, u.ug)[kTieUnits] = 0;
   }
   if (!unit_ok(p, u)) {
     if (threadIdx.x == 0)
@@ -837,7 +829,13 @@ __global__ void __launch_bounds__(kScThr, 1)
       // The two warpgroups' sums, added one after the other.
       sum *= p.inv_g;
       float *su = c.score + it.u.ug * (size_t)c.sstride + slot;
-      if (b == 0 && ok && slot < it.n) *su += sum;
+      if (b == 0 && ok && slot < it.n) {
+        const float before = *su;
+        // For settling ties: behind the normalisers, which end before it.
+        if (p.settle && slot < it.u.m)
+          c.logits[(it.u.ug + 1) * (size_t)G * c.cap - it.u.m + slot] = before;
+        *su = before + sum;
+      }
       int bad;
       asm volatile(
           "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"

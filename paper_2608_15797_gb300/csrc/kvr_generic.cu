@@ -596,22 +596,32 @@ __device__ void tie_sums(const AbsorbParams &p, int x, int tok, float *smem, Put
   for (int h = 0; h < kMaxG; ++h) row4(h < G ? Q[h * 32 + lane] : make_uint2(0u, 0u), q[h]);
   const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
   const int g = lane >> 2;  // the head whose sum this lane ends with
-#pragma unroll 2
-  for (int i = warp; i < n; i += NT / 32) {
-    float k[4], a[kMaxG];
-    row4(K[(size_t)i * 32 + lane], k);
+  constexpr int kAhead = 8;  // rows a warp has in flight
+  for (int i0 = warp; i0 < n; i0 += kAhead * (NT / 32)) {
+    uint2 kw[kAhead];
 #pragma unroll
-    for (int h = 0; h < kMaxG; ++h) a[h] = lane_dot<4>(q[h], k);
+    for (int r = 0; r < kAhead; ++r) {
+      const int i = i0 + r * (NT / 32);
+      kw[r] = i < n ? K[(size_t)i * 32 + lane] : make_uint2(0u, 0u);
+    }
 #pragma unroll
-    for (int h = 0; h < 4; ++h)
-      a[h] = (b4 ? a[h + 4] : a[h]) + __shfl_xor_sync(0xffffffffu, b4 ? a[h] : a[h + 4], 16);
+    for (int r = 0; r < kAhead; ++r) {
+      const int i = i0 + r * (NT / 32);
+      float k[4], a[kMaxG];
+      row4(kw[r], k);
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      a[h] = (b3 ? a[h + 2] : a[h]) + __shfl_xor_sync(0xffffffffu, b3 ? a[h] : a[h + 2], 8);
-    float s = (b2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a[0] : a[1], 4);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    if ((lane & 3) == 0 && g < G) lg[(size_t)g * p.max_rows + i] = s * c.scale;
+      for (int h = 0; h < kMaxG; ++h) a[h] = lane_dot<4>(q[h], k);
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        a[h] = (b4 ? a[h + 4] : a[h]) + __shfl_xor_sync(0xffffffffu, b4 ? a[h] : a[h + 4], 16);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        a[h] = (b3 ? a[h + 2] : a[h]) + __shfl_xor_sync(0xffffffffu, b3 ? a[h] : a[h + 2], 8);
+      float s = (b2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a[0] : a[1], 4);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if (i < n && (lane & 3) == 0 && g < G) lg[(size_t)g * p.max_rows + i] = s * c.scale;
+    }
   }
   __syncthreads();
   if (warp < G) {
@@ -863,9 +873,12 @@ cudaError_t launch_evict_generic(const CacheView &c, int lb, int nl,
 // of their sums, one rounding a token on the latter's side: near the cut by
 // 1.3e-7 rms and 7.3e-7 at most after 57 tokens (7B, 16 sequences of 640 rows,
 // three inputs; 4.6e-7 after 10), 5.7e-7 and 2.5e-6 after 1,000.  Two rows'
-// order is taken as certain beyond more than twice the most.  Settling them
-// is 3 us of 727 and, where a prompt of 1,000 tokens has a tie, 0.1 ms of 0.9.
-float tie_band(int chunk) { return 0x1p-19f * std::max(1.f, std::sqrt(chunk / 64.f)); }
+// order is taken as certain beyond 1.2e-6, six times the rms of two rows'
+// difference (and five times after 1,000 tokens: 4.7e-6).  Settling one to four
+// tied units is 28 us for the sums and 13 for the rest of 768; without ties the
+// launches are 12 of 741, and a prompt of 1,000 tokens with a tied unit takes
+// 0.1 ms more than 0.92.
+float tie_band(int chunk) { return 0x1.4p-20f * std::max(1.f, std::sqrt(chunk / 64.f)); }
 
 bool can_settle(const CacheView &c, int max_rows) {
   return tie_smem(c, max_rows) <= 200 * 1024;

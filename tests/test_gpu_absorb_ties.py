@@ -56,7 +56,7 @@ SHAPES = [(7, 300, 20, 330, 150, 8), (7, 200, 30, 230, 100, 0),
 @pytest.mark.parametrize("G,m,chunk,cap,budget,window", SHAPES)
 def test_near_ties_keep_the_rows_of_token_by_token(G, m, chunk, cap, budget,
                                                    window):
-    # some 40 tied rows around the cut: the band is 2e-6 either way
+    # some 25 tied rows around the cut: the band is 1.2e-6 either way
     spread = m * 2e-7 * 1.98
     a = _absorbed(G, m, chunk, cap, budget, window, True, spread)
     b = _absorbed(G, m, chunk, cap, budget, window, False, spread)
