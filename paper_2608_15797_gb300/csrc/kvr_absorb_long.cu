@@ -748,8 +748,8 @@ __global__ void __launch_bounds__(kScThr, 1)
       const int tmin_w = max(0, it.k0 + t * kBlk + wq * 32 + 31 - it.u.m);
       const int q1 = it.nk(t) > 0 ? it.q0(t) : n_qt;
       // The row's sum: of each query tile's 128 terms apart, then over the
-      // tiles.  (What is left of the scores' error, 1.3e-7 to 1.7e-7 relative,
-      // is the contraction's accumulation: compensated sums did not move it.)
+      // tiles.  (What is left of the scores' error, about 1.2e-7 relative, is the
+      // contraction's accumulation: compensated sums did not move it.)
       float sum = 0.f;
       for (int q = it.q0(0); q < n_qt; ++q) {
         const int s = nq % kLRing, ph_l = nq / kLRing;

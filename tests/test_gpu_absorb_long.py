@@ -116,3 +116,43 @@ def test_absorb_long_prompt_beyond_one_append_grid():
         # one rounding to bf16 of outputs, fp32 sums before it
         assert ((out[t].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 2e-5).all()
     harness.check_guards(c)
+
+
+def test_absorb_long_scores_are_not_biased():
+    """Scores against fp64, 5% of the keys three times as long.  Roundings go
+    either way; what they leave in the mean is 1 / G's (7: 4.5e-8 high) and half
+    a step of the scale (3e-8).  Logits that the contraction cuts towards zero
+    and nothing makes up for give 1.9e-7: the normalisers lack more of the
+    longest keys' terms than the other rows' scores do of theirs."""
+    S, L, H, G, m, c = 2, 2, 4, 7, 640, 57
+    g = torch.Generator(device="cuda")
+    g.manual_seed(12)
+
+    def rnd(*shape, heavy=False):
+        x = torch.randn(shape, generator=g, device="cuda")
+        if heavy:
+            x[torch.rand(shape[:-1], generator=g, device="cuda") < 0.05] *= 3
+        return x.bfloat16()
+    cache = harness.guarded_cache(S, L, H, G, 128, m + c, kv_dtype="bf16",
+                                  out_dtype="bf16")
+    old = [rnd(L, H, m, 128, heavy=True) for _ in range(S)]
+    for s in range(S):
+        cache.load(s, old[s], rnd(L, H, m, 128))
+    q, k, v = (rnd(S, L, c, H * G, 128), rnd(S, L, c, H, 128, heavy=True),
+               rnd(S, L, c, H, 128))
+    cache.absorb(q, k, v, evict=False)
+    assert cache.last_absorb_kernel() == 3
+    got = cache.scores_view()[0][..., :m].double()
+    errs = []
+    hidden = (torch.arange(m + c, device="cuda")[None] >
+              m + torch.arange(c, device="cuda")[:, None])
+    for s in range(S):
+        kk = torch.cat([old[s], k[s].transpose(1, 2)], 2).double()   # [L][H][m+c]
+        qq = q[s].double().unflatten(2, (H, G)).permute(0, 2, 1, 3, 4)
+        x = torch.einsum("lhcgd,lhnd->lhcgn", qq, kk) / 128 ** 0.5
+        p = torch.softmax(x.masked_fill(hidden[:, None], -float("inf")), -1)
+        want = p.mean(3).sum(2)[..., :m]
+        errs.append((got[s] - want) / want)
+    err = torch.stack(errs)
+    assert abs(err.mean().item()) < 1.1e-7
+    assert err.square().mean().sqrt().item() < 2e-7
