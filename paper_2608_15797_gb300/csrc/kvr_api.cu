@@ -1013,12 +1013,14 @@ kvr_status kvr_absorb_chunk(kvr_cache *c, int lb, int le, int chunk,
   const CacheView &v = c->view;
   // Units beyond the tensor-memory kernel's 144 rows: in blocks rather than on
   // the mma.sync kernel (7B, 64 sequences, 136 rows + 33 tokens: 615 us against
-  // 1,642), unless its one launch is the shorter (one sequence, 136 rows + 16
-  // tokens: 20 us against 25; + 33: 36 against 28) or asked for, or the outputs
-  // are fp32.
+  // 1,642), unless its one launch is the shorter (one sequence, 160 rows + 16
+  // tokens: 22 us against 33; two sequences, 224 units, + 16: 43 against 38, + 4:
+  // 34 against 35; four, + 4: 51 against 44) or asked for, or the outputs are
+  // fp32.
+  const int units = v.S * (le - lb) * v.H;
   const bool blocks = v.out_bf16 && c->absorb_kernel == 0 &&
                       m + chunk > kvr::absorb_tc_max_rows() && device_facts(c) &&
-                      (chunk > 16 || v.S * (le - lb) * v.H > c->sm_count);
+                      (chunk > 16 || units > c->sm_count * (chunk > 8 ? 1 : 2));
   if (c->fused && !blocks && v.kv_bf16 && v.d == 128 && v.G <= 8 &&
       chunk <= kvr::absorb_max_chunk() && m + chunk <= kvr::absorb_max_rows() &&
       aligned16(q) && aligned16(k_new) && aligned16(v_new) && aligned16(out)) {
