@@ -153,8 +153,8 @@ kvr_status kvr_decode_step(kvr_cache *cache, int layer_begin, int layer_end,
  * launch: the redundancy of each row comes from the keys already staged
  * for attention, so no key is read twice.  Up to 1,024 rows it is the same in
  * two launches, the first of which sums the keys of units that hold no
- * current sum, or one kept for 12 steps (kvr_cache_scores, state words 2 and
- * 3), and is empty otherwise.  Any other call runs the two calls.
+ * current sum (kvr_cache_scores, state word 2) and is empty otherwise.  Any
+ * other call runs the two calls.
  * Arguments as kvr_decode_step, plus 0 <= lambda <= 1 (KVR_EINVAL
  * otherwise). */
 kvr_status kvr_decode_step_rkv(kvr_cache *cache, int layer_begin,

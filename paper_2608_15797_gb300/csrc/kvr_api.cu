@@ -507,6 +507,8 @@ bool try_chunked(kvr_cache *c, const StepArgs &a, bool evict, int budget,
   if (!aligned16(a.q) || !aligned16(a.k_new) || !aligned16(a.v_new) ||
       !aligned16(a.out))
     return false;
+  // (R-KV: the low parts of a unit's key sum need 131 floats of its scratch.)
+  if (rkv && (size_t)v.G * v.cap < 131) return false;
   if (!device_facts(c)) return false;
   kvr::ChunkParams p{};
   p.rkv = rkv ? 1 : 0;

@@ -41,10 +41,10 @@
 //    of normalised keys S (a B operand of three bf16 terms) and its squared
 //    norm (the diagonal of the tile's Gram block), so that no key is read
 //    twice.  One more exchange of sums at the end of a job gives z.  Units
-//    with no current S, or an old one, get one from rkv_sum_kernel, launched
-//    before.  7B, 16 sequences, 641-row units: 150 us against 113 for the plain
-//    step; the separate eviction pass it replaces (two readings of the keys, a
-//    radix select) took 337 us after the 113.
+//    with no current S get one from rkv_sum_kernel, launched before.  7B, 16
+//    sequences, 641-row units: 147 us against 113 for the plain step; the
+//    separate eviction pass it replaces (two readings of the keys, a radix
+//    select) took 337 us after the 113.
 //  - Launched with programmatic stream serialization; every mbarrier wait is
 //    bounded (about 2 s) and on timeout sets ERR_TIMEOUT and drains its own
 //    copies.
@@ -149,6 +149,22 @@ __device__ __forceinline__ void key4(const unsigned char *row, int lane, float (
   v[2] = __uint_as_float(x.y << 16);
   v[3] = __uint_as_float(x.y & 0xFFFF0000u);
 }
+// The kept key sum is a pair of floats an element, so that a key that enters and
+// later leaves takes nothing with it but itself: 2.6e-7 rms off fp64 (640 rows) as
+// it is formed and after 400 steps, 1.3e-6 by then with one float; 3.8e-7 as the
+// eviction pass forms it at every step.  The low parts lie in the unit's logit
+// scratch (every call that writes there makes the sum stale), from a 16-byte
+// boundary on; state word 2 says that both are current.
+constexpr int kSumPair = 2;
+__device__ __forceinline__ float *sum_low(const CacheView &c, size_t u) {
+  return c.logits + ((u * (size_t)c.G * c.cap + 3) & ~(size_t)3);
+}
+// (hi, lo) += x, the rounding of hi kept in lo.
+__device__ __forceinline__ void add_pair(float &hi, float &lo, float x) {
+  const float s = __fadd_rn(hi, x), y = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, y)), __fsub_rn(x, y)));
+  hi = s;
+}
 // 1 / |k| of the row that the warp holds four elements a lane (0 for a zero
 // row): the arithmetic by which a key enters the kept sum and leaves it.
 __device__ __forceinline__ float inv_norm(const float (&v)[4]) {
@@ -156,6 +172,20 @@ __device__ __forceinline__ float inv_norm(const float (&v)[4]) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   return ss > 0.f ? rsqrtf(ss) : 0.f;
+}
+// A lane's four elements of a 128-float row.
+__device__ __forceinline__ void load4(const unsigned char *row, int lane, float (&v)[4]) {
+  const float4 x = reinterpret_cast<const float4 *>(row)[lane];
+  v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+}
+// The sum's pairs += sign times a normalised key.
+__device__ __forceinline__ void add_key(const unsigned char *row, int lane, float (&hi)[4],
+                                        float (&lo)[4], float sign) {
+  float k[4];
+  key4(row, lane, k);
+  const float inv = sign * inv_norm(k);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) add_pair(hi[x], lo[x], __fmul_rn(k[x], inv));
 }
 // Term `t` (0-2; 0 beyond) of a pair split into three bf16 terms.
 __device__ __forceinline__ uint32_t s_term(float2 v, int t) {
@@ -262,9 +292,11 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
             cp_async16(s0 + Stage::q + (i >> 4) * kQPitch + (i & 15) * 16,
                        q + i * 16);
         }
-        if (kRkv && ci == 0)  // the kept sum of the live rows' normalised keys
+        if (kRkv && ci == 0) {  // the kept sum of the live rows' normalised keys
           cp_async16(s0 + Stage::rs + lane * 16,
                      c.rsum + jb.ug * 128 + lane * 4);
+          cp_async16(s0 + Stage::rs + 512 + lane * 16, sum_low(c, jb.ug) + lane * 4);
+        }
         if (has_new || (kRkv && ci == 0))
           cp_async16(s0 + (lane < 16 ? Stage::kn : Stage::vn) +
                          (lane & 15) * 16,
@@ -296,28 +328,16 @@ __device__ void produce(const ChunkParams &p, const CUtensorMap *tmK,
 }
 
 // R-KV: the sum of a unit's normalised keys, where the unit has none that is
-// current (state word 2), or one that kSumSteps steps have added a key to and
-// taken one from (word 3 counts them), whose roundings would go on adding up.
-// One CTA a unit, a warp four rows at a time.  Rms error of the sum's elements
-// against fp64, 640 rows: 2.6e-7 formed here, 3.7e-7 after 12 steps (and 1.3e-6
-// after 400); 3.8e-7 as the eviction pass forms it at every step.  In the steady
-// state this is an empty launch but for one step in kSumSteps: 7B, 16 sequences,
-// 145 us a step without new sums, 150 with.
-constexpr int kSumSteps = 12;
+// current (state word 2); one CTA a unit, a warp four rows at a time.  In the
+// steady state every unit has one and this is the launch of an empty kernel.
 __global__ void __launch_bounds__(256) rkv_sum_kernel(CacheView c, int lb, int nl) {
   pdl_begin();
   constexpr int kW = 8, kAhead = 4;
   __shared__ float4 s_S[kW][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t u = unit_index(c, lb, nl, blockIdx.x);
-  const int4 st = *reinterpret_cast<const int4 *>(c.state + 4 * u);
-  const int n = st.x;
-  __syncthreads();  // every thread has read the words
-  if (st.z == 1 && st.w >= 0 && st.w < kSumSteps) {
-    if (threadIdx.x == 0) c.state[4 * u + 3] = st.w + 1;
-    return;
-  }
-  if (n < 0 || n > c.cap) return;
+  const int n = c.state[4 * u];
+  if (c.state[4 * u + 2] == kSumPair || n < 0 || n > c.cap) return;
   const unsigned char *K = reinterpret_cast<const unsigned char *>(c.K) + u * (size_t)c.cap * 256;
   float S[4] = {0.f, 0.f, 0.f, 0.f};
   for (int i = warp * kAhead; i < n; i += kW * kAhead) {
@@ -348,10 +368,8 @@ __global__ void __launch_bounds__(256) rkv_sum_kernel(CacheView c, int lb, int n
 #pragma unroll
       for (int w = 0; w < kW; w += 2 * o) t[w] = add(t[w], t[w + o]);
     reinterpret_cast<float4 *>(c.rsum + u * 128)[lane] = t[0];
-    if (lane == 0) {
-      c.state[4 * u + 2] = 1;
-      c.state[4 * u + 3] = 0;
-    }
+    reinterpret_cast<float4 *>(sum_low(c, u))[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane == 0) c.state[4 * u + 2] = kSumPair;
   }
 }
 
@@ -441,9 +459,10 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
 #pragma unroll
       for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
       uint32_t qb[8][2];
-      // R-KV: the key sum S with the new key, elements 4 lane .. 4 lane + 3, and
+      // R-KV: the key sum S with the new key, elements 4 lane .. 4 lane + 3 (a
+      // pair each; read again at the end instead, 153 us a step against 147), and
       // S as the B operand of K S (columns 0-2: three bf16 terms, exact).
-      float S4[4] = {0.f, 0.f, 0.f, 0.f}, inv_n1 = 0.f;
+      float S4[4] = {0.f, 0.f, 0.f, 0.f}, low4[4] = {0.f, 0.f, 0.f, 0.f}, inv_n1 = 0.f;
       uint32_t sq[8][2];
       int idx = 0, t = 0, ntot = 0, nA = 0;
       int4 nrow = make_int4(0, 0, 0, 0);  // warp 0: the new k (lanes 0-15) / v row
@@ -488,18 +507,14 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
         skip = (flags & F_SKIP) != 0;
         if constexpr (kRkv) {
           if ((flags & F_FIRST) && !skip) {
-            const float4 rs = reinterpret_cast<const float4 *>(st + Stage::rs)[lane];
-            float kn[4];
-            key4(st + Stage::kn, lane, kn);
-            const float inv = inv_norm(kn);
-            S4[0] = fmaf(kn[0], inv, rs.x);
-            S4[1] = fmaf(kn[1], inv, rs.y);
-            S4[2] = fmaf(kn[2], inv, rs.z);
-            S4[3] = fmaf(kn[3], inv, rs.w);
+            load4(st + Stage::rs, lane, S4);
+            load4(st + Stage::rs + 512, lane, low4);
+            add_key(st + Stage::kn, lane, S4, low4, 1.f);
             inv_n1 = ntot > 1 ? 1.f / (float)(ntot - 1) : 0.f;
             // Through this warp's part of the (now idle) output exchange.
             float *sx = reinterpret_cast<float *>(OX + w * 4 * 32);
-            reinterpret_cast<float4 *>(sx)[lane] = make_float4(S4[0], S4[1], S4[2], S4[3]);
+            reinterpret_cast<float4 *>(sx)[lane] =
+                make_float4(S4[0] + low4[0], S4[1] + low4[1], S4[2] + low4[2], S4[3] + low4[3]);
             __syncwarp();
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
@@ -948,17 +963,22 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
             vk = (lane & 1) ? make_uint2((uint32_t)z, (uint32_t)u)
                             : make_uint2((uint32_t)x, (uint32_t)y);
           }
-          float kv[4];
-          key4(reinterpret_cast<const unsigned char *>(&vk), 0, kv);
-          const float inv = inv_norm(kv);
-          const float4 S = make_float4(fmaf(kv[0], -inv, S4[0]), fmaf(kv[1], -inv, S4[1]),
-                                       fmaf(kv[2], -inv, S4[2]), fmaf(kv[3], -inv, S4[3]));
-          reinterpret_cast<float4 *>(c.rsum + jb.ug * 128)[lane] = S;
+          add_key(reinterpret_cast<const unsigned char *>(&vk), 0, S4, low4, -1.f);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float sum = __fadd_rn(S4[x], low4[x]);
+            low4[x] = __fadd_rn(__fsub_rn(S4[x], sum), low4[x]);
+            S4[x] = sum;
+          }
+          reinterpret_cast<float4 *>(c.rsum + jb.ug * 128)[lane] =
+              make_float4(S4[0], S4[1], S4[2], S4[3]);
+          reinterpret_cast<float4 *>(sum_low(c, jb.ug))[lane] =
+              make_float4(low4[0], low4[1], low4[2], low4[3]);
           // A key that is not finite must not outlive its row in the sum.  (The
           // vote also orders the reads of the victim's key before its slot's
           // new row.)
-          finite = __all_sync(0xffffffffu, isfinite(S.x) && isfinite(S.y) && isfinite(S.z) &&
-                                               isfinite(S.w));
+          finite = __all_sync(0xffffffffu, isfinite(S4[0]) && isfinite(S4[1]) &&
+                                               isfinite(S4[2]) && isfinite(S4[3]));
         }
         if (w == 0) {
           if (slot >= 0) {
@@ -974,7 +994,7 @@ __global__ void __launch_bounds__((U == 2 ? kMaxGroups : kWideGroups) * (U + 1) 
           if (lane == 0) {
             c.state[4 * jb.ug] = victim < 0 ? m + 1 : m;
             c.state[4 * jb.ug + 1] = t + 1;
-            c.state[4 * jb.ug + 2] = kRkv && finite ? 1 : 0;  // the kept R-KV key sum
+            c.state[4 * jb.ug + 2] = kRkv && finite ? kSumPair : 0;  // the kept R-KV key sum
           }
         }
       }

@@ -55,13 +55,13 @@ struct CacheView {
   void *V;          // [u][cap][d]
   float *score;     // [u][sstride]
   int32_t *pos;     // [u][sstride]
-  int32_t *state;   // [u][4]: live length, next position, rsum valid, steps
-                    // that the chunked kernel has kept rsum for
+  int32_t *state;   // [u][4]: live length, next position, rsum valid, 0
   unsigned *err;    // device error word
   float *logits;    // [u][G][cap] scratch for units beyond on-chip size
   float *rsum;      // [u][d] R-KV: sum of the live rows' normalised keys,
                     // kept by kvr_decode_step_rkv's fused and chunked steps; valid
-                    // while the unit's state word 2 is 1 (every other call
+                    // while the unit's state word 2 is 1, or 2 where the
+                    // chunked step keeps low parts beside it (every other call
                     // that changes the unit's rows writes 0 there)
   int S, L, H, G, d, cap;
   int sstride;      // cap rounded up to 16 (64-byte aligned score/pos rows)
